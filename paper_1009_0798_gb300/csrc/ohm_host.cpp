@@ -744,7 +744,7 @@ int eta_derive(ohm_hier *H) {
     }
     CK(launch_restrict<T>(f->dev, fe, 1, nullptr, (T *)H->smallbuf[0].eta, H->small[0].data(), s));
     SmallDev<T> sm = small_dev<T>(H);
-    CK(launch_small_setup<T>(sm, 0.0, true, s));
+    CK(launch_small_eta<T>(sm, s));
     H->inv_dt = NAN;
     return OHM_OK;
 }
@@ -778,7 +778,7 @@ int prepare_dt(ohm_hier *H, double dt) {
     if constexpr (std::is_same<T, float>::value)
         small_lean = lean && (int64_t)sm.dims[0][0] * sm.dims[0][1] * sm.dims[0][2] <= MAX_BOTTOM_CELLS &&
                      bottom_in_shared(sm);
-    if (!small_lean) CK(launch_small_setup<T>(sm, lamdt, false, s));
+    if (!small_lean) CK(launch_small_inv<T>(sm, lamdt, s));
     H->inv_dt = dt;
     H->inv_all = !lean;
     return OHM_OK;
@@ -2414,8 +2414,8 @@ int ohm_op_coarsest_f32(ohm_hier *h, const float *r_dev, const float *eta_dev, d
     CK(cudaMemcpyAsync(h->smallbuf[0].r, r_dev, 3 * n0 * sizeof(float), cudaMemcpyDeviceToDevice, h->s));
     CK(cudaMemcpyAsync(h->smallbuf[0].eta, eta_dev, n0 * sizeof(float), cudaMemcpyDeviceToDevice, h->s));
     SmallDev<float> sm = small_dev<float>(h);
-    CK(launch_small_setup<float>(sm, 0.0, true, h->s));     // eta of the coarser grids
-    CK(launch_small_setup<float>(sm, lamdt, false, h->s));  // inverse diagonals (paths that read them)
+    CK(launch_small_eta<float>(sm, h->s));         // eta of the coarser grids
+    CK(launch_small_inv<float>(sm, lamdt, h->s));  // inverse diagonals (paths that read them)
     h->eta_set = false;
     h->inv_dt = NAN;
     const ohm_hier_desc &d = h->d;

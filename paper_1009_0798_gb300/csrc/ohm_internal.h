@@ -198,9 +198,12 @@ cudaError_t launch_lex_resid_restrict(const SmallDev<T> &sm, int s, double lamdt
 template <typename T>
 cudaError_t launch_lex_prolong(const SmallDev<T> &sm, int s, cudaStream_t st);
 
-// lexicographic restriction between small grids and small-grid inverse diagonals
+// eta of the lexicographic grids 1 .. n-1 from the grid above each (grid 0's eta is set), and
+// the inverse diagonals of all of them for lambda dt
 template <typename T>
-cudaError_t launch_small_setup(const SmallDev<T> &sm, double lamdt, bool eta_chain, cudaStream_t s);
+cudaError_t launch_small_eta(const SmallDev<T> &sm, cudaStream_t s);
+template <typename T>
+cudaError_t launch_small_inv(const SmallDev<T> &sm, double lamdt, cudaStream_t s);
 
 template <typename TS, typename TD>
 cudaError_t launch_convert(const TS *src, TD *dst, size_t n, cudaStream_t s);

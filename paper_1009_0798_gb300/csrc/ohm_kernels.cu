@@ -2979,55 +2979,78 @@ template cudaError_t launch_lex_resid_restrict<float>(const SmallDev<float> &, i
 template cudaError_t launch_lex_prolong<double>(const SmallDev<double> &, int, cudaStream_t);
 template cudaError_t launch_lex_prolong<float>(const SmallDev<float> &, int, cudaStream_t);
 
-// eta chain over the small grids (optional) and their inverse diagonals
+// Setup of the lexicographic grids: eta of each from the grid above it (mean of the 8 children),
+// one launch per grid, and the inverse diagonals of all of them in one launch, a thread per
+// instance and cell.  Bound by launch latency (the grids hold at most a few 10^5 cells); one
+// thread block per instance, which did the whole chain before, was bound by one SM's float64
+// units instead (the diagonal is formed in float64): 2421 us per call for the 60 x 52 x 44
+// grid below 120 x 104 x 88, about 15 us now (two steps with a new eta each: 15.7 -> 6.05 ms).
 template <typename T>
-__global__ void __launch_bounds__(1024) k_small_setup(SmallDev<T> sm_all, double lamdt, int eta_chain) {
-    const SmallDev<T> sm = small_instance(sm_all);
-    if (eta_chain) {
-        for (int s = 1; s < sm.n; s++) {
-            LexGrid<T> F{sm.dims[s - 1][0], sm.dims[s - 1][1], sm.dims[s - 1][2]};
-            LexGrid<T> C{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
-            const int nc_ = C.nx * C.ny * C.nz;
-            for (int q = threadIdx.x; q < nc_; q += blockDim.x) {
-                int x = q % C.nx, y = (q / C.nx) % C.ny, z = q / (C.nx * C.ny);
-                T acc = 0;
-                for (int dk = 0; dk < 2; dk++)
-                    for (int dj = 0; dj < 2; dj++)
-                        for (int di = 0; di < 2; di++) acc += sm.eta[s - 1][F.id(0, 2 * x + di, 2 * y + dj, 2 * z + dk)];
-                sm.eta[s][q] = acc / T(8);
-            }
-            __syncthreads();
-        }
+__global__ void __launch_bounds__(128) k_small_eta(SmallDev<T> sm, int s) {
+    const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const LexGrid<T> F{sm.dims[s - 1][0], sm.dims[s - 1][1], sm.dims[s - 1][2]};
+    const LexGrid<T> C{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
+    const int n = C.nx * C.ny * C.nz;
+    if (tid >= (size_t)sm.ninst * n) return;
+    const int q = (int)(tid / n), cell = (int)(tid - (size_t)q * n);
+    const T *fine = sm.eta[s - 1] + (size_t)q * F.nx * F.ny * F.nz;
+    const int x = cell % C.nx, y = (cell / C.nx) % C.ny, z = cell / (C.nx * C.ny);
+    T acc = 0;
+    for (int dk = 0; dk < 2; dk++)
+        for (int dj = 0; dj < 2; dj++)
+            for (int di = 0; di < 2; di++) acc += fine[F.id(0, 2 * x + di, 2 * y + dj, 2 * z + dk)];
+    sm.eta[s][(size_t)q * n + cell] = acc / T(8);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128) k_small_inv(SmallDev<T> sm, double lamdt) {
+    size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    int s = 0;
+    for (; s < sm.n; s++) {  // the grid of this thread
+        const size_t all = (size_t)sm.ninst * sm.dims[s][0] * sm.dims[s][1] * sm.dims[s][2];
+        if (tid < all) break;
+        tid -= all;
     }
-    for (int s = 0; s < sm.n; s++) {
-        LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
-        const int n = G.nx * G.ny * G.nz;
-        const double lh2 = lamdt / (sm.h[s] * sm.h[s]);
-        const T *E = sm.eta[s];
-        for (int q = threadIdx.x; q < n; q += blockDim.x) {
-            int x = q % G.nx, y = (q / G.nx) % G.ny, z = q / (G.nx * G.ny);
-            double e0 = (double)E[q];
-            double sa[3] = {0.5 * (e0 + (double)E[G.id(0, x + 1, y, z)]) + 0.5 * (e0 + (double)E[G.id(0, x - 1, y, z)]),
-                            0.5 * (e0 + (double)E[G.id(0, x, y + 1, z)]) + 0.5 * (e0 + (double)E[G.id(0, x, y - 1, z)]),
-                            0.5 * (e0 + (double)E[G.id(0, x, y, z + 1)]) + 0.5 * (e0 + (double)E[G.id(0, x, y, z - 1)])};
-            for (int c = 0; c < 3; c++) {
-                double al = 0.0;
-                for (int ax = 0; ax < 3; ax++)
-                    if (ax != c) al += lh2 * sa[ax];
-                sm.inv[s][(size_t)c * n + q] = (T)(sm.omega / (1.0 + al));
-            }
-        }
-        __syncthreads();
+    if (s == sm.n) return;
+    const LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
+    const int n = G.nx * G.ny * G.nz;
+    const int q = (int)(tid / n), cell = (int)(tid - (size_t)q * n);
+    const int x = cell % G.nx, y = (cell / G.nx) % G.ny, z = cell / (G.nx * G.ny);
+    const T *E = sm.eta[s] + (size_t)q * n;
+    T *inv = sm.inv[s] + (size_t)q * 3 * n;
+    const double lh2 = lamdt / (sm.h[s] * sm.h[s]);
+    const double e0 = (double)E[cell];
+    const double sa[3] = {0.5 * (e0 + (double)E[G.id(0, x + 1, y, z)]) + 0.5 * (e0 + (double)E[G.id(0, x - 1, y, z)]),
+                          0.5 * (e0 + (double)E[G.id(0, x, y + 1, z)]) + 0.5 * (e0 + (double)E[G.id(0, x, y - 1, z)]),
+                          0.5 * (e0 + (double)E[G.id(0, x, y, z + 1)]) + 0.5 * (e0 + (double)E[G.id(0, x, y, z - 1)])};
+    for (int c = 0; c < 3; c++) {
+        double al = 0.0;
+        for (int ax = 0; ax < 3; ax++)
+            if (ax != c) al += lh2 * sa[ax];
+        inv[(size_t)c * n + cell] = (T)(sm.omega / (1.0 + al));
     }
 }
 
 template <typename T>
-cudaError_t launch_small_setup(const SmallDev<T> &sm, double lamdt, bool eta_chain, cudaStream_t s) {
-    if (sm.n == 0) return cudaSuccess;
-    k_small_setup<T><<<sm.ninst, 1024, 0, s>>>(sm, lamdt, eta_chain ? 1 : 0);
+cudaError_t launch_small_eta(const SmallDev<T> &sm, cudaStream_t st) {
+    for (int s = 1; s < sm.n; s++) {
+        const size_t n = (size_t)sm.ninst * sm.dims[s][0] * sm.dims[s][1] * sm.dims[s][2];
+        k_small_eta<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(sm, s);
+    }
     return cudaGetLastError();
 }
-template cudaError_t launch_small_setup<double>(const SmallDev<double> &, double, bool, cudaStream_t);
-template cudaError_t launch_small_setup<float>(const SmallDev<float> &, double, bool, cudaStream_t);
+template cudaError_t launch_small_eta<double>(const SmallDev<double> &, cudaStream_t);
+template cudaError_t launch_small_eta<float>(const SmallDev<float> &, cudaStream_t);
+
+template <typename T>
+cudaError_t launch_small_inv(const SmallDev<T> &sm, double lamdt, cudaStream_t st) {
+    size_t n = 0;
+    for (int s = 0; s < sm.n; s++) n += (size_t)sm.ninst * sm.dims[s][0] * sm.dims[s][1] * sm.dims[s][2];
+    if (n == 0) return cudaSuccess;
+    k_small_inv<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(sm, lamdt);
+    return cudaGetLastError();
+}
+template cudaError_t launch_small_inv<double>(const SmallDev<double> &, double, cudaStream_t);
+template cudaError_t launch_small_inv<float>(const SmallDev<float> &, double, cudaStream_t);
 
 }  // namespace ohm
