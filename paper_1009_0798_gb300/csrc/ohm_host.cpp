@@ -843,8 +843,16 @@ int sweeps(ohm_hier *H, const GridRef &G, int n, double lamdt, bool zero = false
         if (!zs && (n & 1)) CK(cudaMemcpyAsync(G.e, G.e2, bytes, cudaMemcpyDeviceToDevice, H->s));
         return OHM_OK;
     }
-    if (zero) CK(cudaMemsetAsync(G.e, 0, bytes, H->s));
-    for (int i = 0; i < n; i++) {
+    int i0 = 0;
+    if constexpr (std::is_same<T, double>::value) {
+        if (zero && n > 0) {  // the first float64 sweep from zero: one launch, nothing read for e
+            LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_zero(gdev(H, *G.g), (double *)G.e, (const double *)G.r, (const double *)G.eta,
+                                                                 (const double *)G.inv, (const double *)G.Geta, lamdt, H->s));
+            i0 = 1;
+        }
+    }
+    if (zero && i0 == 0) CK(cudaMemsetAsync(G.e, 0, bytes, H->s));
+    for (int i = i0; i < n; i++) {
         LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth<T>(gdev(H, *G.g), (const T *)G.e, (T *)G.e2, (const T *)G.r, (const T *)G.eta, (const T *)G.inv,
                             (const T *)G.Ge, (const T *)G.Geta, lamdt, 0, H->s));
         LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth<T>(gdev(H, *G.g), (const T *)G.e2, (T *)G.e, (const T *)G.r, (const T *)G.eta, (const T *)G.inv,
@@ -2303,7 +2311,7 @@ int ohm_op_grid_smooth(ohm_hier *h, int m, double *e_dev, const double *r_dev, c
     const size_t bytes = (size_t)G.g->n() * 3 * B3 * sizeof(double);
     CK(cudaMemcpyAsync(G.e, e_dev, bytes, cudaMemcpyDeviceToDevice, h->s));
     CK(cudaMemcpyAsync(G.r, r_dev, bytes, cudaMemcpyDeviceToDevice, h->s));
-    CK(launch_smooth<double>(G.g->dev, (const double *)G.e, (double *)G.e2, (const double *)G.r, (const double *)G.eta,
+    CK(launch_smooth<double>(gdev(h, *G.g), (const double *)G.e, (double *)G.e2, (const double *)G.r, (const double *)G.eta,
                              (const double *)G.inv, nullptr, nullptr, h->d.lambda * dt, colour, h->s));
     CK(cudaMemcpyAsync(e_dev, G.e2, bytes, cudaMemcpyDeviceToDevice, h->s));
     CK(cudaStreamSynchronize(h->s));

@@ -101,6 +101,11 @@ cudaError_t launch_smooth(const GridDev &g, const T *e_in, T *e_out, const T *r,
                           const T *inv, const T *Ge, const T *Geta, double lamdt, int colour,
                           cudaStream_t s);
 
+// The red and the black pass of the first float64 sweep from e = 0 (coarse-fine ghosts of e zero)
+// in one launch
+cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
+                               const double *Geta, double lamdt, cudaStream_t s);
+
 // One full red + black sweep in one launch (grids without coarse-fine ghosts), inverse
 // diagonal formed on the fly; e_in != e_out.
 template <typename T>

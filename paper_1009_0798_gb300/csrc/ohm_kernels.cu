@@ -760,18 +760,257 @@ __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__
     }
 }
 
-template <typename T>
-cudaError_t launch_smooth(const GridDev &g, const T *e_in, T *e_out, const T *r, const T *eta, const T *inv,
-                          const T *Ge, const T *Geta, double lamdt, int colour, cudaStream_t s) {
-    if (g.nblk == 0) return cudaSuccess;
-    T coef = (T)(lamdt / (2.0 * g.h * g.h));
-    k_smooth<T><<<g.nblk, 256, 0, s>>>(g, e_in, e_out, r, eta, inv, Ge, Geta, coef, colour);
+// ---- float64 colour passes.  GB300 issues float64 at 1/60 of the float32 rate, so these passes
+// are bound by the float64 pipe (k_smooth with T = double kept it busy at about 114 operations per
+// updated cell) and everything else is traded for fewer operations:
+// * each tangential pair sum P_a(q) = B_a(q) + B_a(q + e_a) (Eq. 10) is formed once per block in
+//   shared memory and serves the four face fluxes that read it;
+// * the update is written without the cell's own value in the face differences: with
+//   alpha = coef * (sum of the face eta sums), e + omega (r - L e) / (1 + alpha) is
+//   (1 - omega) e + inv (r + coef * sum es (B_nb -+ T/4)), inv = omega / (1 + alpha): two
+//   multiply-adds per face and component instead of four operations;
+// about 61 operations per updated cell.  128^3 FGMRES step (V(3,2), 110 passes): 35.1 -> 26.5 ms; a pass
+// over 96^3 87.8 -> 67.6 us with the float64 pipe 71% busy, 8^3 .. 32^3 grids 12-14 -> 9-11 us
+// (latency).  A thread block takes a slab of NZ planes of an 8^3 block
+// (32 NZ threads, one colour cell each): on grids of few blocks the work of one block is spread
+// over several SMs, at a few more pair sums per cell (9, 10, 12 per updated cell for NZ = 8, 4, 2).
+template <int NZ>
+struct SlabD {
+    static constexpr int NT = 32 * NZ, NP = NZ + 2;
+    static constexpr int CS = 100 * NP;                       // tile component stride (rows of 10)
+    static constexpr int PXY = 90 * NP;                       // pair sums of x (or y) faces
+    static constexpr int SUMS = 2 * PXY + 100 * (NZ + 1);
+    static constexpr size_t BYTES = (4 * CS + SUMS) * sizeof(double);
+};
+
+// rows of tile planes z0 .. z0 + NZ + 1 of block b's 10^3 tile, NC components (as stage_rows)
+template <int NZ, int NC>
+__device__ __forceinline__ void stage_slab(double *__restrict__ tile, const double *__restrict__ F,
+                                           const int *__restrict__ snb, const double *__restrict__ ghost, int z0) {
+    constexpr int R = 10 * SlabD<NZ>::NP;
+    for (int task = threadIdx.x; task < NC * R; task += SlabD<NZ>::NT) {
+        const int c = task / R, rr = task - c * R;
+        const int tj = rr % 10, tk = z0 + rr / 10;
+        const int lj = tj - 1, lk = tk - 1;
+        const int dj = lj < 0 ? -1 : (lj > 7 ? 1 : 0), dk = lk < 0 ? -1 : (lk > 7 ? 1 : 0);
+        const int row = ((lk - 8 * dk) * 8 + (lj - 8 * dj)) * 8;
+        const int *nb = snb + (dk + 1) * 9 + (dj + 1) * 3;
+        const double *gh = ghost ? ghost + c * T3 + tk * 100 + tj * 10 : nullptr;
+        double *dst = tile + c * SlabD<NZ>::CS + rr * 10;
+        if (nb[1] >= 0) {
+            const Row8<double> v = load_row8(F + ((size_t)nb[1] * NC + c) * B3 + row);
+#pragma unroll
+            for (int q = 0; q < 8; q++) dst[1 + q] = v.v[q];
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; q++) dst[1 + q] = gh ? gh[1 + q] : 0.0;
+        }
+        dst[0] = nb[0] >= 0 ? F[((size_t)nb[0] * NC + c) * B3 + row + 7] : (gh ? gh[0] : 0.0);
+        dst[9] = nb[2] >= 0 ? F[((size_t)nb[2] * NC + c) * B3 + row] : (gh ? gh[9] : 0.0);
+    }
+}
+
+// the idx-th position (u, v) of a 10 x NV cross-section without its corners
+template <int NV>
+__device__ __forceinline__ void cross_pos(int idx, int &u, int &v) {
+    if (idx < 8) {
+        u = 1 + idx;
+        v = 0;
+    } else if (idx < 8 + 10 * (NV - 2)) {
+        v = 1 + (idx - 8) / 10;
+        u = (idx - 8) % 10;
+    } else {
+        u = 1 + idx - (8 + 10 * (NV - 2));
+        v = NV - 1;
+    }
+}
+// the same for the positions of one colour ((u + v) & 1 == par); half as many
+template <int NV>
+__device__ __forceinline__ void cross_half(int idx, int par, int &u, int &v) {
+    if (idx < 4) {
+        v = 0;
+        u = 1 + 2 * idx + ((par + 1) & 1);
+    } else if (idx < 4 + 5 * (NV - 2)) {
+        v = 1 + (idx - 4) / 5;
+        u = 2 * ((idx - 4) % 5) + ((par + v) & 1);
+    } else {
+        v = NV - 1;
+        u = 1 + 2 * (idx - (4 + 5 * (NV - 2))) + ((par + v + 1) & 1);
+    }
+}
+
+// Pair sums of one axis: NF face planes of a 10 x NV cross-section.  The first and last plane
+// hold only the sums beside the updated colour's cells (`first` / `last`: the colour parity of the
+// positions needed there).
+template <int NZ, int NF, int NV>
+__device__ __forceinline__ void pair_sums_axis(const double *__restrict__ Ba, double *__restrict__ P, int sa, int su, int sv,
+                                               int first, int last) {
+    constexpr int FULL = 10 * NV - 4, HALF = FULL / 2, N = (NF - 2) * FULL + 2 * HALF;
+    for (int e = threadIdx.x; e < N; e += SlabD<NZ>::NT) {
+        int fn, u, v;
+        if (e < (NF - 2) * FULL) {
+            fn = 1 + e / FULL;
+            cross_pos<NV>(e % FULL, u, v);
+        } else {
+            const int h = e - (NF - 2) * FULL;
+            fn = h < HALF ? 0 : NF - 1;
+            cross_half<NV>(h < HALF ? h : h - HALF, h < HALF ? first : last, u, v);
+        }
+        const double *p = Ba + fn * sa + u * su + v * sv;
+        P[(fn * NV + v) * 10 + u] = p[sa] + p[0];
+    }
+}
+
+__device__ __forceinline__ bool nonfinite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+
+// One colour pass.  ZERO: both passes of the sweep from e = 0 in one launch (colour = 1, the black
+// pass; its red neighbours hold the pointwise red update inv r, its black ones 0), reading r and inv
+// for the red cells of the halo instead of e.
+template <int NZ, bool ZERO>
+__global__ void __launch_bounds__(32 * NZ) k_smooth_d(GridDev g, const double *__restrict__ e_in, double *__restrict__ e_out,
+                                                      const double *__restrict__ r, const double *__restrict__ eta,
+                                                      const double *__restrict__ inv, const double *__restrict__ Ge,
+                                                      const double *__restrict__ Geta, double coef, double om1, int colour) {
+    using S = SlabD<NZ>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
+    __shared__ int snb[27];
+    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
+    if (skip_block(g, b)) return;
+    const int slot = g.gslot ? g.gslot[b] : -1;
+    if (NZ == 2 || threadIdx.x < 32) stage_nbr(snb, g.nbr, b);
+    __syncthreads();
+    stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
+    const int t = threadIdx.x, i2 = t & 3, j = (t >> 2) & 7, kl = t >> 5;
+    const int odd = (j + z0 + kl + colour) & 1;  // the updated cell of the x-pair (2 i2, 2 i2 + 1)
+    const int ic = 2 * i2 + odd;
+    const size_t cpair = (size_t)b * 3 * B3 + ((z0 + kl) * 8 + j) * 8 + 2 * i2;
+    if constexpr (ZERO) {
+        // tile: inv r at red cells ((i + j + k) even, block coordinates), 0 elsewhere
+        for (int h = t; h < S::CS / 2; h += S::NT) {
+            const int row = h / 5, tj = row % 10, tk = z0 + row / 10, pr = 2 * (h % 5), sft = (tj + tk + 1) & 1;
+            const int li = pr + sft - 1, lj = tj - 1, lk = tk - 1;
+            const int di = li < 0 ? -1 : (li > 7 ? 1 : 0), dj = lj < 0 ? -1 : (lj > 7 ? 1 : 0), dk = lk < 0 ? -1 : (lk > 7 ? 1 : 0);
+            const int src = snb[(dk + 1) * 9 + (dj + 1) * 3 + (di + 1)];
+            const size_t id = (size_t)(src >= 0 ? src : 0) * 3 * B3 + ((lk - 8 * dk) * 8 + (lj - 8 * dj)) * 8 + (li - 8 * di);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                tB[c * S::CS + row * 10 + pr + sft] = src >= 0 ? inv[id + c * B3] * r[id + c * B3] : 0.0;
+                tB[c * S::CS + row * 10 + pr + 1 - sft] = 0.0;
+            }
+        }
+    } else {
+        stage_slab<NZ, 3>(tB, e_in, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr, z0);
+    }
+    double2 rp[3], ip[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        rp[c] = __ldg(reinterpret_cast<const double2 *>(r + cpair + c * B3));
+        ip[c] = __ldg(reinterpret_cast<const double2 *>(inv + cpair + c * B3));
+    }
+    __syncthreads();
+    if constexpr (!ZERO) {
+        // a boundary face's pair sum is read where the inside cell beside it is updated, i.e. at
+        // positions whose own inside cell has the other colour: (u + v) parity of the block
+        // coordinates u - 1, v - 1 (v - 1 + z0 on x and y faces) and the inside plane's coordinate
+        const int x = (colour + 1 + z0) & 1;
+        pair_sums_axis<NZ, 9, NZ + 2>(tB, P, 1, 10, 100, x, (x + 7) & 1);
+        pair_sums_axis<NZ, 9, NZ + 2>(tB + S::CS, P + S::PXY, 10, 1, 100, x, (x + 7) & 1);
+        pair_sums_axis<NZ, NZ + 1, 10>(tB + 2 * S::CS, P + 2 * S::PXY, 100, 1, 10, x, (x + NZ - 1) & 1);
+        __syncthreads();
+    }
+    const int u = ic + 1, v = j + 1, w = kl + 1;
+    const int p = w * 100 + v * 10 + u;
+    const double e0 = tE[p];
+    const double es[6] = {tE[p - 1] + e0, e0 + tE[p + 1], tE[p - 10] + e0, e0 + tE[p + 10], tE[p - 100] + e0, e0 + tE[p + 100]};
+    const int st[3] = {1, 10, 100};
+    double out[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        double acc = 0.0;
+        bool first = true;
+        const double *Bc = tB + c * S::CS + p;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            if (a == c) continue;
+            double tl, th;  // T of the low and the high face along a, component c (Eq. 10)
+            if constexpr (ZERO) {
+                const double *Ba = tB + a * S::CS + p;
+                tl = th = Ba[st[c]] - Ba[-st[c]];
+            } else {
+                // (u, v) of the face cross-section are the two other axes in ascending order
+                const int cu = a == 0 ? v : u, cv = a == 2 ? v : w, fn = a == 0 ? ic : (a == 1 ? j : kl);
+                const int NV = a == 2 ? 10 : NZ + 2;
+                const int du = (a == 0 ? c == 1 : c == 0) ? 1 : 10;
+                const double *Pa = P + a * S::PXY + (fn * NV + cv) * 10 + cu;
+                tl = Pa[du] - Pa[-du];
+                th = Pa[NV * 10 + du] - Pa[NV * 10 - du];
+            }
+            const double fl = fma(0.25, tl, Bc[-st[a]]), fh = fma(-0.25, th, Bc[st[a]]);
+            acc = first ? es[2 * a] * fl : fma(es[2 * a], fl, acc);
+            acc = fma(es[2 * a + 1], fh, acc);
+            first = false;
+        }
+        const double rc = odd ? rp[c].y : rp[c].x, ivc = odd ? ip[c].y : ip[c].x;
+        const double tt = fma(coef, acc, rc);
+        const double ec = Bc[0];
+        if (ZERO) {
+            out[c] = ivc * tt;
+        } else if (om1 != 0.0) {
+            out[c] = fma(ivc, tt, om1 * ec);
+        } else {  // Gauss-Seidel: the old value has no weight, but a NaN or infinity in it stays visible
+            out[c] = ivc * tt;
+            if (nonfinite_bits(ec)) out[c] = ec - ec;
+        }
+        const double eo = Bc[odd ? -1 : 1];  // the pair's other cell
+        *reinterpret_cast<double2 *>(e_out + cpair + c * B3) = odd ? make_double2(eo, out[c]) : make_double2(out[c], eo);
+    }
+}
+
+template <int NZ, bool ZERO>
+static cudaError_t launch_smooth_slab(const GridDev &g, const double *e_in, double *e_out, const double *r,
+                                      const double *eta, const double *inv, const double *Ge, const double *Geta,
+                                      double lamdt, int colour, cudaStream_t s) {
+    using S = SlabD<NZ>;
+    // set once per process (thread-safe static initialisation)
+    static const bool attr = (cudaFuncSetAttribute(k_smooth_d<NZ, ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES), true);
+    (void)attr;
+    k_smooth_d<NZ, ZERO><<<g.nblk * (8 / NZ), S::NT, ZERO ? 4 * S::CS * sizeof(double) : S::BYTES, s>>>(
+        g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt / (2.0 * g.h * g.h), 1.0 - g.omega, colour);
     return cudaGetLastError();
 }
-template cudaError_t launch_smooth<double>(const GridDev &, const double *, double *, const double *, const double *,
-                                           const double *, const double *, const double *, double, int, cudaStream_t);
-template cudaError_t launch_smooth<float>(const GridDev &, const float *, float *, const float *, const float *,
-                                          const float *, const float *, const float *, double, int, cudaStream_t);
+
+// Slab height by the number of blocks: whole blocks do the least work, but a grid should give
+// every SM several thread blocks of equal share
+constexpr int SLAB2_BLOCKS = 256, SLAB4_BLOCKS = 2048;
+template <bool ZERO>
+static cudaError_t launch_smooth_d(const GridDev &g, const double *e_in, double *e_out, const double *r, const double *eta,
+                                   const double *inv, const double *Ge, const double *Geta, double lamdt, int colour,
+                                   cudaStream_t s) {
+    if (g.nblk == 0) return cudaSuccess;
+    if (g.nblk <= SLAB2_BLOCKS) return launch_smooth_slab<2, ZERO>(g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt, colour, s);
+    if (g.nblk <= SLAB4_BLOCKS) return launch_smooth_slab<4, ZERO>(g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt, colour, s);
+    return launch_smooth_slab<8, ZERO>(g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt, colour, s);
+}
+
+template <>
+cudaError_t launch_smooth<double>(const GridDev &g, const double *e_in, double *e_out, const double *r, const double *eta,
+                                  const double *inv, const double *Ge, const double *Geta, double lamdt, int colour,
+                                  cudaStream_t s) {
+    return launch_smooth_d<false>(g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt, colour, s);
+}
+template <>
+cudaError_t launch_smooth<float>(const GridDev &g, const float *e_in, float *e_out, const float *r, const float *eta,
+                                 const float *inv, const float *Ge, const float *Geta, double lamdt, int colour,
+                                 cudaStream_t s) {
+    if (g.nblk == 0) return cudaSuccess;
+    k_smooth<float><<<g.nblk, 256, 0, s>>>(g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
+    return cudaGetLastError();
+}
+cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
+                               const double *Geta, double lamdt, cudaStream_t s) {
+    return launch_smooth_d<true>(g, nullptr, e_out, r, eta, inv, nullptr, Geta, lamdt, 1, s);
+}
 
 // ------------------------------------------------------------------ fused red + black sweep
 // One full red-black sweep in one launch, for grids whose blocks have every neighbour (no

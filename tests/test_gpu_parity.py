@@ -144,6 +144,30 @@ def test_grid_smooth_relaxed(ohm, orc, colour):
     assert np.array_equal(got[:, ~moved], e[:, ~moved])
 
 
+@pytest.mark.parametrize("dims", [(64, 64, 64), (104, 104, 104)])
+def test_float64_sweeps_on_taller_slabs(ohm, orc, dims):
+    """Grids of more blocks give a thread block more planes of an 8^3 block (4 above 256 blocks, 8
+    above 2048): both colours of a pass, and the sweeps from zero inside a V-cycle."""
+    h = W.uniform(*dims, 1.0 / dims[0])
+    o = orc.Oracle(h, 0.5)
+    g = make(ohm, h, nu_pre=2, nu_post=1, n_coarse=3)
+    _, nb, ijk = ohm.ohm_mg_grid_info(g, 0)
+    rng = np.random.default_rng(31)
+    e, r = (rng.standard_normal((3,) + dims[::-1]) for _ in range(2))
+    eta = 10 ** rng.uniform(-1, 1, (1,) + dims[::-1])
+    dt = 5.0 * h.dx0 ** 2
+    for colour in (0, 1):
+        et = dev(grid_of_dense(e, ijk))
+        ohm.ohm_op_grid_smooth(g, 0, et, dev(grid_of_dense(r, ijk)), dev(grid_of_dense(eta, ijk)), dt, colour)
+        assert rel_err(dense_of_grid(host(et).reshape(nb, 3, 8, 8, 8), ijk, dims, 3), o.grid_smooth(0, e, r, eta, dt, colour)) < TOL64
+    B, etab = rand_fields(h, 32)
+    o = orc.Oracle(h, 0.5, etab)
+    ohm.ohm_set_eta(g, dev(etab))
+    out = torch.empty_like(dev(B))
+    ohm.ohm_op_vcycle(g, dev(B), dt, out)
+    assert rel_err(host(out), o.vcycle(B, dt, 2, 1, 3)) < TOL64
+
+
 @pytest.mark.parametrize("m", [0, 1])
 def test_grid_residual_restrict_prolong(ohm, orc, m):
     """a4 (level residual), a6 restriction, a7 prolongation on base multigrid grid m."""
