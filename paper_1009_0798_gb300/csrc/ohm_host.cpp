@@ -21,9 +21,6 @@ using namespace ohm;
 namespace {
 
 constexpr int MAX_LEVELS = 8;
-// lexicographic grids of more cells than this are stepped by grid-wide launches; the rest, down
-// to the coarsest, by the one-block solver (k_bottom: one thread block per instance)
-constexpr int MAX_BOTTOM_CELLS = 16384;
 // mixed precision: coarse grids of at most this many cells (16^3), with power-of-two extents, are
 // not blocked; the coarsest-grid solver runs them in shared memory
 constexpr int64_t MIN_BLOCKED_CELLS = 4096;
@@ -126,6 +123,7 @@ struct ohm_hier {
     std::vector<double> cur_scale;
     bool eta_dirty = false;
     InstRanges ranges;
+    int tail_m = 0;               // blocked base grid from which on launch_tail takes every grid (0: none)
     int smoother = 0;             // 0: fused red+black sweep where possible, 1: two colour passes
     const uint8_t *cmask = nullptr;  // compute mask of batched iterations (null: every instance)
     double active_frac = 1.0;        // share of instances the compute mask lets through (timing)
@@ -724,6 +722,32 @@ SmallDev<T> small_dev(ohm_hier *H) {
     return sm;
 }
 
+// grids s0 .. of sm as a table of their own
+template <typename T>
+SmallDev<T> small_from(const SmallDev<T> &sm, int s0) {
+    SmallDev<T> v = sm;
+    v.n = sm.n - s0;
+    for (int q = 0; q < v.n; q++) {
+        for (int a = 0; a < 3; a++) v.dims[q][a] = sm.dims[s0 + q][a];
+        v.h[q] = sm.h[s0 + q];
+        v.e[q] = sm.e[s0 + q];
+        v.r[q] = sm.r[s0 + q];
+        v.t[q] = sm.t[s0 + q];
+        v.eta[q] = sm.eta[s0 + q];
+        v.inv[q] = sm.inv[s0 + q];
+        v.origin[q] = sm.origin[s0 + q];
+    }
+    return v;
+}
+
+// the first lexicographic grid from which on launch_tail takes the rest (their number if none)
+template <typename T>
+int tail_first(const SmallDev<T> &sm) {
+    int s0 = 0;
+    while (s0 < sm.n && !tail_fits(small_from(sm, s0))) s0++;
+    return s0;
+}
+
 // eta: level ghosts, the multigrid copies and the eta chain below level 0
 template <typename T>
 int eta_derive(ohm_hier *H) {
@@ -776,8 +800,7 @@ int prepare_dt(ohm_hier *H, double dt) {
     SmallDev<T> sm = small_dev<T>(H);
     bool small_lean = false;
     if constexpr (std::is_same<T, float>::value)
-        small_lean = lean && (int64_t)sm.dims[0][0] * sm.dims[0][1] * sm.dims[0][2] <= MAX_BOTTOM_CELLS &&
-                     bottom_in_shared(sm);
+        small_lean = lean && tail_first(sm) == 0;
     if (!small_lean) CK(launch_small_inv<T>(sm, lamdt, s));
     H->inv_dt = dt;
     H->inv_all = !lean;
@@ -860,17 +883,50 @@ int sweeps(ohm_hier *H, const GridRef &G, int n, double lamdt, bool zero = false
     }
     return OHM_OK;
 }
+// The tail's grids from blocked base grid m (>= 1) on: the blocked ones, then the lexicographic ones.
+// False when they do not all fit into launch_tail.
+template <typename T>
+bool tail_from_blocked(ohm_hier *H, int m, SmallDev<T> &sm) {
+    const int nb = (int)H->mg.size() - (m - 1), ns = (int)H->small.size();
+    if (nb + ns > MAX_SMALL) return false;
+    const SmallDev<T> lex = small_dev<T>(H);
+    sm = lex;
+    sm.n = nb + ns;
+    for (int q = 0; q < nb; q++) {
+        const HGrid &g = H->mg[m - 1 + q];
+        const Buffers &b = H->mgbuf[m - 1 + q];
+        for (int a = 0; a < 3; a++) sm.dims[q][a] = g.dims[a];
+        sm.h[q] = g.h;
+        sm.e[q] = (T *)b.e;
+        sm.r[q] = (T *)b.r;
+        sm.t[q] = (T *)b.e2;
+        sm.eta[q] = (T *)b.eta;
+        sm.inv[q] = (T *)b.inv;
+        sm.origin[q] = g.dev.origin;
+    }
+    for (int q = 0; q < ns; q++) {
+        for (int a = 0; a < 3; a++) sm.dims[nb + q][a] = lex.dims[q][a];
+        sm.h[nb + q] = lex.h[q];
+        sm.e[nb + q] = lex.e[q];
+        sm.r[nb + q] = lex.r[q];
+        sm.t[nb + q] = lex.t[q];
+        sm.eta[nb + q] = lex.eta[q];
+        sm.inv[nb + q] = lex.inv[q];
+        sm.origin[nb + q] = nullptr;
+    }
+    return tail_fits(sm);
+}
+
 // The V-cycle over the lexicographic grids below the last blocked one, for the restricted
-// residual already in r of small grid 0.  Grids of more than MAX_BOTTOM_CELLS cells take
-// grid-wide launches (the same arithmetic as the one-block solver); the one-block solver runs
-// the remaining grids, or the coarsest grid gets its sweeps grid-wide when even that is large.
+// residual already in r of small grid 0.  Grids too large for the cluster solver take grid-wide
+// launches; it runs the remaining grids, or the coarsest grid gets its sweeps grid-wide when even
+// that is too large.
 template <typename T>
 int small_vcycle(ohm_hier *H, double lamdt, int npre, int npost, int ncoarse) {
     SmallDev<T> sm = small_dev<T>(H);
-    int s0 = 0;
-    while (s0 < sm.n && (int64_t)sm.dims[s0][0] * sm.dims[s0][1] * sm.dims[s0][2] > MAX_BOTTOM_CELLS) s0++;
+    const int s0 = tail_first(sm);
     if (s0 == 0) {
-        LAUNCH(H, OHM_K_BOTTOM, 0, launch_bottom<T>(sm, lamdt, npre, npost, ncoarse, H->s));
+        LAUNCH(H, OHM_K_BOTTOM, 0, launch_tail<T>(sm, lamdt, npre, npost, ncoarse, H->s));
         return OHM_OK;
     }
     const size_t cells0 = (size_t)sm.dims[0][0] * sm.dims[0][1] * sm.dims[0][2];
@@ -880,22 +936,10 @@ int small_vcycle(ohm_hier *H, double lamdt, int npre, int npost, int ncoarse) {
         LAUNCH(H, OHM_K_BOTTOM, 0, launch_lex_sweeps<T>(sm, g, lamdt, npre, H->s));
         LAUNCH(H, OHM_K_BOTTOM, 0, launch_lex_resid_restrict<T>(sm, g, lamdt, H->s));
     }
-    if (s0 < sm.n) {
-        SmallDev<T> v = sm;  // grids s0 .. n-1
-        v.n = sm.n - s0;
-        for (int q = 0; q < v.n; q++) {
-            for (int a = 0; a < 3; a++) v.dims[q][a] = sm.dims[s0 + q][a];
-            v.h[q] = sm.h[s0 + q];
-            v.e[q] = sm.e[s0 + q];
-            v.r[q] = sm.r[s0 + q];
-            v.t[q] = sm.t[s0 + q];
-            v.eta[q] = sm.eta[s0 + q];
-            v.inv[q] = sm.inv[s0 + q];
-        }
-        LAUNCH(H, OHM_K_BOTTOM, 0, launch_bottom<T>(v, lamdt, npre, npost, ncoarse, H->s));
-    } else {
+    if (s0 < sm.n)
+        LAUNCH(H, OHM_K_BOTTOM, 0, launch_tail<T>(small_from(sm, s0), lamdt, npre, npost, ncoarse, H->s));
+    else
         LAUNCH(H, OHM_K_BOTTOM, 0, launch_lex_sweeps<T>(sm, sm.n - 1, lamdt, ncoarse, H->s));
-    }
     for (int g = top - 1; g >= 0; g--) {
         LAUNCH(H, OHM_K_BOTTOM, 0, launch_lex_prolong<T>(sm, g, H->s));
         LAUNCH(H, OHM_K_BOTTOM, 0, launch_lex_sweeps<T>(sm, g, lamdt, npost, H->s));
@@ -924,6 +968,14 @@ int base_vcycle(ohm_hier *H, int m, double lamdt) {
     // level 0 takes nu_pre / nu_post, its coarsenings the coarse-grid counts when those are set
     const bool cs = m >= 1 && (d.nu_coarse_pre || d.nu_coarse_post);
     const int npre = cs ? d.nu_coarse_pre : d.nu_pre, npost = cs ? d.nu_coarse_post : d.nu_post;
+    if (m >= 1 && H->tail_m == m && (std::is_same<T, double>::value || H->smoother == 0)) {
+        // this grid and all below it fit into the cluster solver
+        SmallDev<T> sm;
+        if (tail_from_blocked<T>(H, m, sm)) {
+            LAUNCH(H, OHM_K_BOTTOM, 0, launch_tail<T>(sm, lamdt, npre, npost, d.n_coarse, H->s));
+            return OHM_OK;
+        }
+    }
     if ((st = sweeps<T>(H, G, npre, lamdt, true))) return st;  // the level's correction starts at 0
     const bool next_blocked = m < (int)H->mg.size();
     if (next_blocked) {
@@ -1921,6 +1973,11 @@ int ohm_create_hierarchy(const ohm_hier_desc *d, ohm_hier **out) {
         g_last_error = err;
         ohm_destroy(H);
         return st;
+    }
+    for (int m = 1; m <= (int)H->mg.size() && H->tail_m == 0; m++) {
+        SmallDev<float> sf;
+        SmallDev<double> sd;
+        if (H->mixed ? tail_from_blocked<float>(H, m, sf) : tail_from_blocked<double>(H, m, sd)) H->tail_m = m;
     }
     *out = H;
     return OHM_OK;

@@ -39,18 +39,20 @@ struct GridDev {
     double omega = 1.0;             // relaxation factor of the red-black sweeps (1 = Gauss-Seidel)
 };
 
-// Lexicographic coarse grids below the last blocked grid (solved in one thread block).
+// Coarse grids of the V-cycle's tail: the lexicographic grids below the last blocked grid, and above
+// them blocked grids small enough for launch_tail (origin set).
 constexpr int MAX_SMALL = 12;
 template <typename T>
 struct SmallDev {
     int n = 0;                      // number of small grids
     int ninst = 1;                  // instances; the arrays of grid s hold them one after another
                                     // (instance q at q * ncomp * cells(s)), one thread block each
-    const uint8_t *imask = nullptr; // k_bottom skips instances whose flag is 0
+    const uint8_t *imask = nullptr; // instances whose flag is 0 are skipped
     double omega = 1.0;             // relaxation factor folded into inv (1 = Gauss-Seidel)
     int dims[MAX_SMALL][3];
     double h[MAX_SMALL];
     T *e[MAX_SMALL], *r[MAX_SMALL], *t[MAX_SMALL], *eta[MAX_SMALL], *inv[MAX_SMALL];
+    const int *origin[MAX_SMALL] = {};  // blocked grids: [blocks][3] block coordinates of one instance
 };
 
 // ------------------------------------------------------------------ kernel launchers
@@ -185,16 +187,15 @@ constexpr size_t NORM_SCRATCH_BYTES = 128 * 3 * sizeof(double) + 16;
 cudaError_t launch_norm_reduce(const double *partials, int nblocks, double *scratch, double *out, cudaStream_t s,
                                double *host_out = nullptr, const int *err = nullptr);
 
+// The V-cycle over all grids of sm (grid 0's r set, its e the result) in one launch, a cluster of
+// thread blocks per instance with the grids in shared memory.  tail_fits: whether they fit.  In
+// float32 the inverse diagonals are not read (the diagonal is formed from eta).
 template <typename T>
-cudaError_t launch_bottom(const SmallDev<T> &sm, double lamdt, int nu_pre, int nu_post,
-                          int n_coarse, cudaStream_t s);
-// whether launch_bottom runs these float32 grids in the shared-memory solver (every extent a
-// power of two, the grids within its shared memory), which forms the diagonal from eta and does
-// not read the grids' inverse diagonals
-bool bottom_in_shared(const SmallDev<float> &sm);
+bool tail_fits(const SmallDev<T> &sm);
+template <typename T>
+cudaError_t launch_tail(const SmallDev<T> &sm, double lamdt, int nu_pre, int nu_post, int n_coarse, cudaStream_t s);
 
-// Grid-wide steps on lexicographic grid s of every instance (grids too large for the one-block
-// coarsest solver): nsweep red-black sweeps (e -> t -> e), residual into t and its restriction
+// Grid-wide steps on lexicographic grid s of every instance (grids too large for launch_tail): nsweep red-black sweeps (e -> t -> e), residual into t and its restriction
 // into r of grid s + 1 (e of grid s + 1 zeroed), prolongation e_s += P e_{s+1}.
 template <typename T>
 cudaError_t launch_lex_sweeps(const SmallDev<T> &sm, int s, double lamdt, int nsweep, cudaStream_t st);

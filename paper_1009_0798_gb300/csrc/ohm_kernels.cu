@@ -8,6 +8,7 @@
 //   Phi_a^b = (eta_lo + eta_hi) * (T/4 - N),  N = B_b(hi) - B_b(lo)                 (Eq. 9)
 //   T = B_a(lo+e_b) + B_a(hi+e_b) - B_a(lo-e_b) - B_a(hi-e_b)                         (Eq. 10)
 // and the flux divergence (Eq. 8) is sum_a (Phi_a(+) - Phi_a(-)) / (2 h^2).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -2659,8 +2660,8 @@ cudaError_t launch_maxpy_inst(float *dst, const float *src, const VecSet &V, con
 }
 
 // ------------------------------------------------------------------ coarsest grids
-// Lexicographic periodic grids below the last blocked grid, all handled by one thread block per
-// instance with a barrier between phases.  Face flux and divergence as above, with periodic wrap.
+// Lexicographic periodic grids below the last blocked grid.  Face flux and divergence as above, with
+// periodic wrap.
 template <typename T>
 struct LexGrid {
     int nx, ny, nz;
@@ -2706,129 +2707,29 @@ __device__ __forceinline__ void lex_div(const LexGrid<T> &G, const T *B, const T
     dv[2] = (xh2 - xl2) + (yh2 - yl2);
 }
 
+// The V-cycle over the coarsest grids in one launch: a cluster of CS thread blocks per instance.
+// A grid of more than tail_divide cells is divided over the cluster in z-planes: every block keeps the
+// grid's arrays at full size in its own shared memory but holds only its planes and the ones beside
+// them, and writes its new values into the neighbours' copies through distributed shared memory, so
+// that every read of a pass is a local one and a pass costs two cluster barriers.  Smaller grids are
+// stepped by every block for itself, without any exchange, and the coarsest one with its stencil
+// coefficients in registers.  What bounds these grids is latency and one SM's arithmetic (float64
+// above all: 1.7 operations per clock and SM, a quarter of that for one warp scheduler), not bytes.
+// Measured against one thread block per instance (which float32 had in shared memory, float64 in
+// global memory): float32 16^3 .. 2^3, V(1,0), 2 coarsest sweeps, 46 -> 29 us; float64 below 32^3, V(2,2), 16
+// coarsest sweeps, 470 -> 140 us (with the launches for 16^3 and 8^3 that it takes in); steps: 32^3
+// float64 4.63 -> 2.35 ms, half-refined box 10.2 -> 7.9, 64^3 mixed 1.75 -> 1.63.
 template <typename T>
-__device__ void lex_sweeps(const SmallDev<T> &sm, int s, double lamdt, int nsweep) {
-    LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
-    const int n = G.nx * G.ny * G.nz;
-    const T coef = (T)(lamdt / (2.0 * sm.h[s] * sm.h[s]));
-    T *e = sm.e[s], *d = sm.t[s];
-    const T *r = sm.r[s], *E = sm.eta[s], *inv = sm.inv[s];
-    for (int sw = 0; sw < nsweep; sw++)
-        for (int colour = 0; colour < 2; colour++) {
-            for (int q = threadIdx.x; q < n; q += blockDim.x) {
-                int x = q % G.nx, y = (q / G.nx) % G.ny, z = q / (G.nx * G.ny);
-                if (((x + y + z) & 1) != colour) continue;
-                T dv[3];
-                lex_div(G, e, E, x, y, z, dv);
-                for (int c = 0; c < 3; c++) {
-                    size_t id = (size_t)c * n + q;
-                    d[id] = (r[id] - e[id] - coef * dv[c]) * inv[id];
-                }
-            }
-            __syncthreads();
-            for (int q = threadIdx.x; q < n; q += blockDim.x) {
-                int x = q % G.nx, y = (q / G.nx) % G.ny, z = q / (G.nx * G.ny);
-                if (((x + y + z) & 1) != colour) continue;
-                for (int c = 0; c < 3; c++) e[(size_t)c * n + q] += d[(size_t)c * n + q];
-            }
-            __syncthreads();
-        }
-}
-
-// the grids of instance blockIdx.x
-template <typename T>
-__device__ __forceinline__ SmallDev<T> small_instance(const SmallDev<T> &in) {
-    SmallDev<T> sm = in;
-    const size_t q = blockIdx.x;
-    for (int s = 0; s < sm.n; s++) {
-        const size_t cells = (size_t)sm.dims[s][0] * sm.dims[s][1] * sm.dims[s][2];
-        sm.e[s] += q * 3 * cells;
-        sm.r[s] += q * 3 * cells;
-        sm.t[s] += q * 3 * cells;
-        sm.inv[s] += q * 3 * cells;
-        sm.eta[s] += q * cells;
-    }
-    return sm;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_bottom(SmallDev<T> sm_all, double lamdt, int nu1, int nu2, int nc) {
-    if (sm_all.imask && !sm_all.imask[blockIdx.x]) return;
-    const SmallDev<T> sm = small_instance(sm_all);
-    // e on the first small grid starts from zero
-    {
-        const int n0 = sm.dims[0][0] * sm.dims[0][1] * sm.dims[0][2];
-        for (int q = threadIdx.x; q < 3 * n0; q += blockDim.x) sm.e[0][q] = T(0);
-        __syncthreads();
-    }
-    int s = 0;
-    for (; s < sm.n - 1; s++) {
-        lex_sweeps(sm, s, lamdt, nu1);
-        LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
-        LexGrid<T> C{sm.dims[s + 1][0], sm.dims[s + 1][1], sm.dims[s + 1][2]};
-        const int n = G.nx * G.ny * G.nz, nc_ = C.nx * C.ny * C.nz;
-        const T coef = (T)(lamdt / (2.0 * sm.h[s] * sm.h[s]));
-        for (int q = threadIdx.x; q < n; q += blockDim.x) {
-            int x = q % G.nx, y = (q / G.nx) % G.ny, z = q / (G.nx * G.ny);
-            T dv[3];
-            lex_div(G, sm.e[s], sm.eta[s], x, y, z, dv);
-            for (int c = 0; c < 3; c++) {
-                size_t id = (size_t)c * n + q;
-                sm.t[s][id] = sm.r[s][id] - sm.e[s][id] - coef * dv[c];
-            }
-        }
-        __syncthreads();
-        for (int q = threadIdx.x; q < 3 * nc_; q += blockDim.x) {
-            int c = q / nc_, cq = q % nc_;
-            int x = cq % C.nx, y = (cq / C.nx) % C.ny, z = cq / (C.nx * C.ny);
-            T acc = 0;
-            for (int dk = 0; dk < 2; dk++)
-                for (int dj = 0; dj < 2; dj++)
-                    for (int di = 0; di < 2; di++) acc += sm.t[s][G.id(c, 2 * x + di, 2 * y + dj, 2 * z + dk)];
-            sm.r[s + 1][q] = acc / T(8);
-            sm.e[s + 1][q] = T(0);
-        }
-        __syncthreads();
-    }
-    lex_sweeps(sm, s, lamdt, nc);
-    for (s = sm.n - 2; s >= 0; s--) {
-        LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
-        LexGrid<T> C{sm.dims[s + 1][0], sm.dims[s + 1][1], sm.dims[s + 1][2]};
-        const int n = G.nx * G.ny * G.nz;
-        for (int q = threadIdx.x; q < 3 * n; q += blockDim.x) {
-            int c = q / n, fq = q % n;
-            int x = fq % G.nx, y = (fq / G.nx) % G.ny, z = fq / (G.nx * G.ny);
-            int px = x >> 1, py = y >> 1, pz = z >> 1;
-            int sx = (x & 1) ? 1 : -1, sy = (y & 1) ? 1 : -1, sz = (z & 1) ? 1 : -1;
-            T v = 0;
-            for (int ak = 0; ak < 2; ak++)
-                for (int aj = 0; aj < 2; aj++)
-                    for (int ai = 0; ai < 2; ai++) {
-                        T wt = (ai ? T(0.25) : T(0.75)) * (aj ? T(0.25) : T(0.75)) * (ak ? T(0.25) : T(0.75));
-                        v += wt * sm.e[s + 1][C.id(c, px + ai * sx, py + aj * sy, pz + ak * sz)];
-                    }
-            sm.e[s][q] += v;
-        }
-        __syncthreads();
-        lex_sweeps(sm, s, lamdt, nu2);
-    }
-}
-
-// The same V-cycle over the lexicographic grids (float32) with the grids held in shared memory: e, r, t and eta of every grid are staged once (r of the first grid
-// and eta from global memory, e from zero), every pass of the cycle runs between two block
-// barriers, and only e of the first grid is written back.  The point update is the fused sweeps'
-// (face_pair flux divergence, Eqs. 8-10, and the relaxed diagonal formed from eta, Eqs. 21-23)
-// through an accessor whose periodic neighbour offsets are formed once per cell.
 struct LexAcc {
-    const float *fB, *fE;
+    const T *fB, *fE;
     int n;                    // cells of the grid (component stride)
     int xo[3], yo[3], zo[3];  // offsets of the cells at -1, 0, +1 along x, y, z (wrapped)
     template <int C, int DX, int DY, int DZ>
-    __device__ __forceinline__ float B() const {
+    __device__ __forceinline__ T B() const {
         return fB[C * n + zo[DZ + 1] + yo[DY + 1] + xo[DX + 1]];
     }
     template <int DX, int DY, int DZ>
-    __device__ __forceinline__ float E() const {
+    __device__ __forceinline__ T E() const {
         return fE[zo[DZ + 1] + yo[DY + 1] + xo[DX + 1]];
     }
 };
@@ -2851,8 +2752,25 @@ struct LexDims {
             y = t - z * ny;
         }
     }
-    __device__ __forceinline__ LexAcc acc(const float *B, const float *E, int x, int y, int z) const {
-        LexAcc a;
+    // the slots of a colour's cells: (nx + 1) / 2 per row; x may come out as nx on odd extents (no cell)
+    __host__ __device__ __forceinline__ int slots() const { return ((nx + 1) >> 1) * ny * nz; }
+    __device__ __forceinline__ void colour_cell(int i, int colour, int &x, int &y, int &z) const {
+        int h;
+        if (p2 && nx > 1) {
+            h = i & ((nx >> 1) - 1);
+            y = (i >> (lx - 1)) & (ny - 1);
+            z = i >> (lx - 1 + ly);
+        } else {
+            const int hx = (nx + 1) >> 1, t = i / hx;
+            h = i - t * hx;
+            z = t / ny;
+            y = t - z * ny;
+        }
+        x = 2 * h + ((y + z + colour) & 1);
+    }
+    template <typename T>
+    __device__ __forceinline__ LexAcc<T> acc(const T *B, const T *E, int x, int y, int z) const {
+        LexAcc<T> a;
         a.fB = B;
         a.fE = E;
         a.n = n();
@@ -2870,166 +2788,503 @@ struct LexDims {
     }
 };
 
-struct BottomSm {  // no default member initialisers: a __shared__ copy is filled by one thread
+constexpr int TAIL_LUT = 64;                  // blocks of the blocked grids of a tail, all together
+constexpr size_t TAIL_SMEM_MAX = 220 * 1024;
+// grids of more cells are divided over the cluster: a pass over fewer takes one block less than the
+// barriers of the division
+template <typename T>
+constexpr int tail_divide() {
+    return sizeof(T) == 8 ? 64 : 512;
+}
+// threads: an instance on one thread block (large batches) in float32 wants 32 warps to hide latency
+template <typename T, int CS>
+struct TailThreads {
+    static constexpr int N = CS == 1 && sizeof(T) == 4 ? 1024 : 512;
+};
+// coarsest grids of at most this many cells per colour keep their coefficients in registers (six
+// threads per cell: components x the two axes of each)
+constexpr int TAIL_REG_SLOTS = 18;
+
+template <typename T>
+struct TailP {  // no default member initialisers: the kernel keeps a __shared__ copy
     int n;
+    T om1;                        // 1 - omega
     LexDims d[MAX_SMALL];
-    int base[MAX_SMALL];          // float offset of grid s in shared memory: e[3n], r[3n], t[3n], eta[n]
-    RbK<float> K[MAX_SMALL];      // update constants of grid s (the sweeps' relaxed diagonal, Eqs. 21-23)
+    int oe[MAX_SMALL], oE[MAX_SMALL], orr[MAX_SMALL], oi[MAX_SMALL];  // element offsets in shared memory: e[3n],
+                                  // eta[n], r (first grid, divided: the own cells by colour, else [3n]) and, in
+                                  // float64, the own cells' inverse diagonals by colour
+    bool own;                     // the own cells' values are kept (else read from global memory in each pass)
+    int ot;                       // new values of one pass
+    int hz[MAX_SMALL];            // divided grids: planes per block (1, or even where the grid is restricted)
+    int lut[MAX_SMALL], nbx[MAX_SMALL], nby[MAX_SMALL], nblk[MAX_SMALL];  // blocked grids: table offset, blocks
+    bool divided[MAX_SMALL], blocked[MAX_SMALL];
+    RbK<T> K[MAX_SMALL];
+    const T *inv[MAX_SMALL], *eta[MAX_SMALL];
+    const int *origin[MAX_SMALL];
+    const T *r0;
+    T *e0;
+    const uint8_t *imask;
 };
 
-// the i-th cell of colour `colour` ((x + y + z) & 1) of a power-of-two grid with at least 2
-// cells along x
-__device__ __forceinline__ void colour_cell(const LexDims &D, int i, int colour, int &x, int &y, int &z) {
-    const int hx = D.lx - 1;
-    y = (i >> hx) & (D.ny - 1);
-    z = i >> (hx + D.ly);
-    x = 2 * (i & ((1 << hx) - 1)) + ((y + z + colour) & 1);
+template <int CS>
+__device__ __forceinline__ void tail_sync(bool cluster) {
+    if (CS > 1 && cluster)
+        cooperative_groups::this_cluster().sync();
+    else
+        __syncthreads();
+}
+template <int CS>
+__device__ __forceinline__ int tail_rank() {
+    return CS > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
 }
 
-// one colour pass of grid s (Jacobi within the colour): t = (r - L e) / den on the colour's cells,
-// then e += t
-__device__ __forceinline__ void bsm_colour(const BottomSm &P, float *sh, int s, int colour) {
+// stores v at element offset o of the shared memory of every block of the cluster (or only here)
+template <int CS, typename T>
+__device__ __forceinline__ void tail_store_all(T *sh, int o, T v, bool cluster) {
+    if (CS > 1 && cluster) {
+        auto cl = cooperative_groups::this_cluster();
+#pragma unroll
+        for (int k = 0; k < CS; k++) cl.map_shared_rank(sh, k)[o] = v;
+    } else {
+        sh[o] = v;
+    }
+}
+
+// stores the three components of a cell of plane z of grid s (offsets o, o + n, o + 2 n) here and in
+// the blocks that read that plane: the owners of the planes within `reach` of it (1 where blocks own
+// whole octets, 2 where a block owns one plane and reads its octet's other one)
+template <int CS, typename T>
+__device__ __forceinline__ void tail_store_cell(const TailP<T> &P, T *sh, int s, int z, int o, int n, const T v[3], int rank) {
+#pragma unroll
+    for (int c = 0; c < 3; c++) sh[o + c * n] = v[c];
+    if (CS > 1 && P.divided[s]) {
+        auto cl = cooperative_groups::this_cluster();
+        const int hz = P.hz[s], nz = P.d[s].nz, reach = hz == 1 ? 2 : 1;
+        int last = rank;
+        for (int dz = -reach; dz <= reach; dz++) {
+            int zz = z + dz;
+            zz = zz < 0 ? zz + nz : (zz >= nz ? zz - nz : zz);
+            const int k = zz / hz;
+            if (k == rank || k == last) continue;
+            last = k;
+            T *rem = cl.map_shared_rank(sh, k);
+#pragma unroll
+            for (int c = 0; c < 3; c++) rem[o + c * n] = v[c];
+        }
+    }
+}
+
+// index of cell (x, y, z) of grid s in global memory: component stride cst for ncomp components
+template <typename T>
+__device__ __forceinline__ size_t tail_gidx(const TailP<T> &P, const int *lut, int s, int x, int y, int z, int ncomp, int &cst) {
+    if (P.blocked[s]) {
+        const int b = lut[P.lut[s] + ((z >> 3) * P.nby[s] + (y >> 3)) * P.nbx[s] + (x >> 3)];
+        cst = B3;
+        return (size_t)b * ncomp * B3 + ((z & 7) * 8 + (y & 7)) * 8 + (x & 7);
+    }
+    cst = P.d[s].n();
+    return P.d[s].id(x, y, z);
+}
+
+// the planes of grid s that this block owns
+template <int CS, typename T>
+__device__ __forceinline__ void tail_planes(const TailP<T> &P, int s, int rank, int &z0, int &z1) {
+    const int nz = P.d[s].nz;
+    if (CS > 1 && P.divided[s]) {
+        z0 = min(nz, rank * P.hz[s]);
+        z1 = min(nz, z0 + P.hz[s]);
+    } else {
+        z0 = 0;
+        z1 = nz;
+    }
+}
+
+// the off-diagonal part of -2 h^2 divF of component C through its two faces along AX in float64, added
+// to acc: es_lo (B_lo + T_lo / 4) + es_hi (B_hi - T_hi / 4) (k_smooth_d's form, the tangential
+// differences formed per cell)
+template <int AX, int C, class A>
+__device__ __forceinline__ double offdiag_pair(const A &a, double acc) {
+    constexpr int AXX = AX == 0, AXY = AX == 1, AXZ = AX == 2;
+    constexpr int CX = C == 0, CY = C == 1, CZ = C == 2;
+    const double e0 = a.template E<0, 0, 0>();
+    const double d0 = a.template B<AX, CX, CY, CZ>() - a.template B<AX, -CX, -CY, -CZ>();
+    const double dp = a.template B<AX, AXX + CX, AXY + CY, AXZ + CZ>() - a.template B<AX, AXX - CX, AXY - CY, AXZ - CZ>();
+    const double dm = a.template B<AX, CX - AXX, CY - AXY, CZ - AXZ>() - a.template B<AX, -CX - AXX, -CY - AXY, -CZ - AXZ>();
+    acc = fma(a.template E<-AXX, -AXY, -AXZ>() + e0, fma(0.25, d0 + dm, a.template B<C, -AXX, -AXY, -AXZ>()), acc);
+    return fma(a.template E<AXX, AXY, AXZ>() + e0, fma(-0.25, dp + d0, a.template B<C, AXX, AXY, AXZ>()), acc);
+}
+// new value of component C of a cell in float64; zero: e = 0 everywhere (only r matters)
+template <int C, class A>
+__device__ __forceinline__ double tail_update_d(const A &a, double coef, double om1, double r, double inv, bool zero) {
+    constexpr int A1 = C == 0 ? 1 : 0, A2 = C == 2 ? 1 : 2;
+    const double acc = zero ? 0.0 : offdiag_pair<A2, C>(a, offdiag_pair<A1, C>(a, 0.0));
+    return fma(inv, fma(coef, acc, r), om1 * a.template B<C, 0, 0, 0>());
+}
+// new values of a cell in float32 (the point update of the fused sweeps)
+__device__ __forceinline__ void tail_update_f(const LexAcc<float> &a, const RbK<float> &K, const float rr[3], bool zero, float out[3]) {
+    float es[6], den[3], dv[3] = {0.f, 0.f, 0.f};
+    rb_faces_den<float>(a, K, es, den);
+    if (!zero) cell_divergence<float>(a, es, dv);
+    const float ev[3] = {a.template B<0, 0, 0, 0>(), a.template B<1, 0, 0, 0>(), a.template B<2, 0, 0, 0>()};
+#pragma unroll
+    for (int c = 0; c < 3; c++) out[c] = v_add(ev[c], rb_relax(0.f, v_mad(K.ncoef, dv[c], v_sub(rr[c], ev[c])), den[c]));
+}
+
+// one colour pass of grid s (Jacobi within the colour: every new value is formed before any is stored).
+// float64 takes a thread per cell and component: its arithmetic is spread over the four schedulers of
+// the SM, each of which has a quarter of the float64 rate.
+template <typename T, int CS>
+__device__ __forceinline__ void tail_colour(const TailP<T> &P, T *sh, const int *lut, size_t inst3, int s, int colour, bool zero) {
+    constexpr int NT = TailThreads<T, CS>::N;
     const LexDims D = P.d[s];
-    const int n = D.n();
-    float *e = sh + P.base[s], *r = e + 3 * n, *t = r + 3 * n, *E = t + 3 * n;
-    const RbK<float> K = P.K[s];
-    // power-of-two grids at least 2 cells wide in x enumerate the colour's cells; other grids
-    // visit every cell and skip the other colour
-    const bool half = D.p2 && D.nx >= 2;
-    const int ncol = half ? n / 2 : n;
-    for (int i = threadIdx.x; i < ncol; i += blockDim.x) {
+    const int n = D.n(), row = D.slots() / D.nz, rank = tail_rank<CS>();
+    const bool dv = P.divided[s];
+    int z0, z1;
+    tail_planes<CS>(P, s, rank, z0, z1);
+    const int lo = z0 * row, own = (z1 - z0) * row;
+    const T *e = sh + P.oe[s], *E = sh + P.oE[s];
+    T *t = sh + P.ot;
+    constexpr int NC = sizeof(T) == 8 ? 3 : 1;
+    for (int i = threadIdx.x; i < NC * own; i += NT) {
+        const int cc = NC == 1 ? 0 : i / own, il = i - cc * own;
         int x, y, z;
-        if (half) {
-            colour_cell(D, i, colour, x, y, z);
+        D.colour_cell(lo + il, colour, x, y, z);
+        if (x >= D.nx) continue;
+        const int q = D.id(x, y, z), o = 3 * colour * own + il;
+        size_t id = 0;
+        int cst = 0;
+        if (!P.own) id = inst3 * n + tail_gidx(P, lut, s, x, y, z, 3, cst);
+        auto rhs = [&](int c) { return s > 0 || (P.own && !dv) ? sh[P.orr[s] + c * n + q] : (P.own ? sh[P.orr[0] + o + c * own] : P.r0[id + (size_t)c * cst]); };
+        const LexAcc<T> acc = D.acc(e, E, x, y, z);
+        if constexpr (sizeof(T) == 8) {
+            const double rv = rhs(cc), iv = P.own ? sh[P.oi[s] + o + cc * own] : P.inv[s][id + (size_t)cc * cst];
+            const double coef = -P.K[s].ncoef;
+            t[cc * own + il] = cc == 0 ? tail_update_d<0>(acc, coef, P.om1, rv, iv, zero)
+                                       : (cc == 1 ? tail_update_d<1>(acc, coef, P.om1, rv, iv, zero)
+                                                  : tail_update_d<2>(acc, coef, P.om1, rv, iv, zero));
         } else {
-            D.cell(i, x, y, z);
-            if (((x + y + z) & 1) != colour) continue;
-        }
-        const int q = D.id(x, y, z);
-        const LexAcc a = D.acc(e, E, x, y, z);
-        float es[6], den[3], dv[3];
-        rb_faces_den<float>(a, K, es, den);
-        cell_divergence<float>(a, es, dv);
+            const T rr[3] = {rhs(0), rhs(1), rhs(2)};
+            T out[3];
+            tail_update_f(acc, P.K[s], rr, zero, out);
 #pragma unroll
-        for (int c = 0; c < 3; c++)
-            t[c * n + q] = rb_relax(0.f, v_mad(K.ncoef, dv[c], v_sub(r[c * n + q], e[c * n + q])), den[c]);
+            for (int c = 0; c < 3; c++) t[c * own + il] = out[c];
+        }
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < ncol; i += blockDim.x) {
+    tail_sync<CS>(dv);
+    for (int il = threadIdx.x; il < own; il += NT) {
         int x, y, z;
-        if (half) {
-            colour_cell(D, i, colour, x, y, z);
-        } else {
-            D.cell(i, x, y, z);
-            if (((x + y + z) & 1) != colour) continue;
-        }
-        const int q = D.id(x, y, z);
-#pragma unroll
-        for (int c = 0; c < 3; c++) e[c * n + q] = v_add(e[c * n + q], t[c * n + q]);
+        D.colour_cell(lo + il, colour, x, y, z);
+        if (x >= D.nx) continue;
+        const T v[3] = {t[il], t[own + il], t[2 * own + il]};
+        tail_store_cell<CS>(P, sh, s, z, P.oe[s] + D.id(x, y, z), n, v, rank);
     }
-    __syncthreads();
+    tail_sync<CS>(dv);
 }
 
-__global__ void __launch_bounds__(1024) k_bottom_sm(SmallDev<float> sm_all, BottomSm P_arg, int nu1, int nu2, int nc) {
-    if (sm_all.imask && !sm_all.imask[blockIdx.x]) return;
-    extern __shared__ __align__(16) float sh[];
-    // the grid table and this instance's global arrays in shared memory (indexed by grid below;
-    // kernel parameters are only read at compile-time indices)
-    __shared__ BottomSm P;
-    if (threadIdx.x == 0) P = P_arg;
-    // stage r of grid 0 and eta of every grid; e of grid 0 starts from zero
+template <typename T, int CS>
+__device__ __forceinline__ void tail_sweeps(const TailP<T> &P, T *sh, const int *lut, size_t inst3, int s, int nsweep, bool zero) {
+    for (int k = 0; k < nsweep; k++) {
+        tail_colour<T, CS>(P, sh, lut, inst3, s, 0, zero && k == 0);
+        tail_colour<T, CS>(P, sh, lut, inst3, s, 1, false);
+    }
+}
+
+// float64 sweeps of a coarsest grid of at most TAIL_REG_SLOTS cells per colour: a colour update is linear
+// in e with fixed coefficients, e_c <- (1 - omega) e_c + inv r + sum_k w_k e_k over 16 neighbour values
+// (8 through each axis' two faces), so a thread keeps the 8 weights and offsets of one (cell,
+// component, axis) for each colour in registers and a pass is 8 multiply-adds, one exchange between
+// the two lanes of a component and one barrier pair (warp-wide when 32 threads hold the grid: 2^3).
+__device__ __forceinline__ void tail_coarsest(const TailP<double> &P, double *sh, const int *lut, size_t inst3, int s, int nsweep) {
+    const LexDims D = P.d[s];
+    const int n = D.n(), slots = D.slots(), nthr = 6 * slots;
+    double *e = sh + P.oe[s];
+    const double *E = sh + P.oE[s];
+    const bool one_warp = nthr <= 32;
+    if (threadIdx.x < (one_warp ? 32 : 128)) {
+        double w[2][8], base[2];
+        int off[2][8], oc[2];
+        const int half = threadIdx.x & 1, c = (threadIdx.x >> 1) % 3, il = threadIdx.x / 6;
+        const int ax = c == 0 ? 1 + half : (c == 1 ? 2 * half : half);
 #pragma unroll
-    for (int g = 0; g < MAX_SMALL; g++) {
-        if (g >= P_arg.n) break;
-        const int n = P_arg.d[g].n();
-        float *e = sh + P_arg.base[g], *r = e + 3 * n, *E = r + 6 * n;
-        const float *eta = sm_all.eta[g] + (size_t)blockIdx.x * n;
-        for (int q = threadIdx.x; q < n; q += blockDim.x) E[q] = eta[q];
-        if (g == 0) {
-            const float *r0 = sm_all.r[0] + (size_t)blockIdx.x * 3 * n;
-            for (int q = threadIdx.x; q < 3 * n; q += blockDim.x) {
-                r[q] = r0[q];
-                e[q] = 0.f;
+        for (int colour = 0; colour < 2; colour++) {
+            int x = 0, y = 0, z = 0;
+            if (il < slots) D.colour_cell(il, colour, x, y, z);
+            const bool live = il < slots && x < D.nx;
+            if (!live) x = y = z = 0;
+            const int q = D.id(x, y, z);
+            const LexAcc<double> a = D.acc(e, E, x, y, z);
+            // offsets of the cells at +-1 along ax, along c and along both
+            auto at = [&](int da, int dc) {
+                int dx = 1 + (ax == 0 ? da : 0) + (c == 0 ? dc : 0), dy = 1 + (ax == 1 ? da : 0) + (c == 1 ? dc : 0),
+                    dz = 1 + (ax == 2 ? da : 0) + (c == 2 ? dc : 0);
+                const int px = dx == 0 ? a.xo[0] : (dx == 1 ? a.xo[1] : a.xo[2]);
+                const int py = dy == 0 ? a.yo[0] : (dy == 1 ? a.yo[1] : a.yo[2]);
+                const int pz = dz == 0 ? a.zo[0] : (dz == 1 ? a.zo[1] : a.zo[2]);
+                return px + py + pz;
+            };
+            const double es_lo = E[q] + E[at(-1, 0)], es_hi = E[q] + E[at(1, 0)];
+            int cst;
+            const size_t id = inst3 * n + tail_gidx(P, lut, s, x, y, z, 3, cst) + (size_t)c * cst;
+            const double rv = s == 0 ? P.r0[id] : sh[P.orr[s] + c * n + q];
+            const double inv = P.inv[s][id];
+            const double k_lo = -P.K[s].ncoef * es_lo * inv, k_hi = -P.K[s].ncoef * es_hi * inv;
+            const double m_lo = 0.25 * k_lo, m_hi = 0.25 * k_hi, m_0 = m_lo - m_hi;
+            w[colour][0] = k_lo; off[colour][0] = c * n + at(-1, 0);
+            w[colour][1] = k_hi; off[colour][1] = c * n + at(1, 0);
+            w[colour][2] = m_0; off[colour][2] = ax * n + at(0, 1);
+            w[colour][3] = -m_0; off[colour][3] = ax * n + at(0, -1);
+            w[colour][4] = m_lo; off[colour][4] = ax * n + at(-1, 1);
+            w[colour][5] = -m_lo; off[colour][5] = ax * n + at(-1, -1);
+            w[colour][6] = -m_hi; off[colour][6] = ax * n + at(1, 1);
+            w[colour][7] = m_hi; off[colour][7] = ax * n + at(1, -1);
+            base[colour] = inv * rv;
+            oc[colour] = live ? c * n + q : -1;
+        }
+        for (int k = 0; k < nsweep; k++) {
+#pragma unroll
+            for (int colour = 0; colour < 2; colour++) {
+                double v = half == 0 && oc[colour] >= 0 ? P.om1 * e[oc[colour]] + base[colour] : 0.0, u = 0.0;
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    v += w[colour][j] * e[off[colour][j]];
+                    u += w[colour][4 + j] * e[off[colour][4 + j]];
+                }
+                v += u;
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                if (one_warp)
+                    __syncwarp();
+                else
+                    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four warps of this branch
+                if (half == 0 && oc[colour] >= 0) e[oc[colour]] = v;
+                if (one_warp)
+                    __syncwarp();
+                else
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
             }
         }
     }
     __syncthreads();
-    int s = 0;
-    for (; s < P.n - 1; s++) {
-        for (int k = 0; k < nu1; k++) {
-            bsm_colour(P, sh, s, 0);
-            bsm_colour(P, sh, s, 1);
-        }
-        const LexDims D = P.d[s], C = P.d[s + 1];
-        const int n = D.n(), ncs = C.n();
-        float *e = sh + P.base[s], *r = e + 3 * n, *t = r + 3 * n, *E = t + 3 * n;
-        for (int q = threadIdx.x; q < n; q += blockDim.x) {  // residual t = r - L e
-            int x, y, z;
-            D.cell(q, x, y, z);
-            const LexAcc a = D.acc(e, E, x, y, z);
-            float es[6], dv[3];
-            face_sums<float>(a, es);
-            cell_divergence<float>(a, es, dv);
-#pragma unroll
-            for (int c = 0; c < 3; c++) t[c * n + q] = v_mad(P.K[s].ncoef, dv[c], v_sub(r[c * n + q], e[c * n + q]));
-        }
-        __syncthreads();
-        float *ec = sh + P.base[s + 1], *rc = ec + 3 * ncs;
-        for (int q = threadIdx.x; q < 3 * ncs; q += blockDim.x) {  // mean of the 8 children; e = 0
-            const int c = q / ncs, cq = q - c * ncs;
-            int x, y, z;
-            C.cell(cq, x, y, z);
-            float acc = 0.f;
-            for (int dk = 0; dk < 2; dk++)
-                for (int dj = 0; dj < 2; dj++)
-                    for (int di = 0; di < 2; di++)
-                        acc = v_add(acc, t[c * n + D.id(2 * x + di, 2 * y + dj, 2 * z + dk)]);
-            rc[q] = v_mul(acc, 0.125f);
-            ec[q] = 0.f;
-        }
-        __syncthreads();
-    }
-    for (int k = 0; k < nc; k++) {
-        bsm_colour(P, sh, s, 0);
-        bsm_colour(P, sh, s, 1);
-    }
-    for (s = P.n - 2; s >= 0; s--) {
-        const LexDims D = P.d[s], C = P.d[s + 1];
-        const int n = D.n(), ncs = C.n();
-        float *e = sh + P.base[s];
-        const float *ec = sh + P.base[s + 1];
-
-        for (int q = threadIdx.x; q < 3 * n; q += blockDim.x) {  // trilinear prolongation (weights 3/4, 1/4)
-            const int c = q / n, fq = q - c * n;
-            int x, y, z;
-            D.cell(fq, x, y, z);
-            const int px = x >> 1, py = y >> 1, pz = z >> 1;
-            const int sx = (x & 1) ? 1 : -1, sy = (y & 1) ? 1 : -1, sz = (z & 1) ? 1 : -1;
-            float v = 0.f;
-            for (int ak = 0; ak < 2; ak++)
-                for (int aj = 0; aj < 2; aj++)
-                    for (int ai = 0; ai < 2; ai++) {
-                        const float wt = (ai ? 0.25f : 0.75f) * (aj ? 0.25f : 0.75f) * (ak ? 0.25f : 0.75f);
-                        int cx = px + ai * sx, cy = py + aj * sy, cz = pz + ak * sz;  // periodic wrap
-                        cx = cx < 0 ? cx + C.nx : (cx >= C.nx ? cx - C.nx : cx);
-                        cy = cy < 0 ? cy + C.ny : (cy >= C.ny ? cy - C.ny : cy);
-                        cz = cz < 0 ? cz + C.nz : (cz >= C.nz ? cz - C.nz : cz);
-                        v = v_mad(wt, ec[c * ncs + C.id(cx, cy, cz)], v);
-                    }
-            e[q] = v_add(e[q], v);
-        }
-        __syncthreads();
-        for (int k = 0; k < nu2; k++) {
-            bsm_colour(P, sh, s, 0);
-            bsm_colour(P, sh, s, 1);
-        }
-    }
-    const int n0 = P.d[0].n();
-    float *e0 = sm_all.e[0] + (size_t)blockIdx.x * 3 * n0;
-    for (int q = threadIdx.x; q < 3 * n0; q += blockDim.x) e0[q] = sh[P.base[0] + q];
 }
 
-constexpr size_t BOTTOM_SMEM_MAX = 200 * 1024;
+// Contribution of one outer face of an octet's cell (octet_face's terms): along axis a at offset os
+// from the cell at o0, component strides and the +-1 offsets of component c in the cell's own plane
+// (p, m) and in the face neighbour's (ps, ms); qs = +-1/4
+template <typename T>
+__device__ __forceinline__ T tail_face(const T *Ba, const T *Bc, int o0, int os, int p, int m, int ps, int ms, T qs, T es) {
+    const T d0 = v_sub(Ba[p], Ba[m]), dn = v_sub(Ba[ps], Ba[ms]);
+    return v_mul(es, v_mad(v_add(dn, d0), qs, v_sub(Bc[o0], Bc[os])));
+}
+
+template <typename T, int CS>
+__global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_constant__ TailP<T> P_arg, int nu1, int nu2, int nc) {
+    constexpr int NT = TailThreads<T, CS>::N;
+    const int inst = blockIdx.x / CS;
+    if (P_arg.imask && !P_arg.imask[inst]) return;  // the whole cluster
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *sh = reinterpret_cast<T *>(smem_raw);
+    __shared__ TailP<T> P;  // indexed by grid below: kernel parameters are only read at fixed indices
+    __shared__ int lut[TAIL_LUT];
+    static_assert(sizeof(TailP<T>) % sizeof(int) == 0, "copied as ints");
+    for (int q = threadIdx.x; q < (int)(sizeof(TailP<T>) / sizeof(int)); q += NT)
+        reinterpret_cast<int *>(&P)[q] = reinterpret_cast<const int *>(&P_arg)[q];
+    __syncthreads();
+    bool any = false;
+    for (int s = 0; s < P.n; s++) {
+        if (!P.blocked[s]) continue;
+        any = true;
+        for (int b = threadIdx.x; b < P.nblk[s]; b += NT) {
+            const int *o = P.origin[s] + 3 * b;
+            lut[P.lut[s] + (o[2] * P.nby[s] + o[1]) * P.nbx[s] + o[0]] = b;
+        }
+    }
+    if (any) __syncthreads();
+    const int rank = tail_rank<CS>();
+    // eta of every grid (divided ones: the planes read here), e = 0 on the first; the own cells' r
+    // (first grid) and inverse diagonals (float64)
+    for (int s = 0; s < P.n; s++) {
+        const LexDims D = P.d[s];
+        const int n = D.n(), pl = D.nx * D.ny;
+        const T *eta = P.eta[s] + (size_t)inst * n;
+        int z0, z1;
+        tail_planes<CS>(P, s, rank, z0, z1);
+        const bool part = CS > 1 && P.divided[s] && z1 - z0 + 4 < D.nz;
+        const int za = part ? z0 - 2 : 0, np = z0 < z1 ? (part ? z1 - z0 + 4 : D.nz) : 0;
+        if (!part && !P.blocked[s]) {
+            for (int q = threadIdx.x; q < np * pl; q += NT) sh[P.oE[s] + q] = eta[q];
+        } else
+#pragma unroll 4
+        for (int q = threadIdx.x; q < np * pl; q += NT) {
+            int x, y, z, cst;
+            D.cell(q, x, y, z);
+            z += za;
+            z = z < 0 ? z + D.nz : (z >= D.nz ? z - D.nz : z);
+            sh[P.oE[s] + D.id(x, y, z)] = eta[tail_gidx(P, lut, s, x, y, z, 1, cst)];
+        }
+        if (s == 0)
+            for (int q = threadIdx.x; q < 3 * n; q += NT) sh[P.oe[0] + q] = T(0);
+        if (!P.own || (s > 0 && sizeof(T) == 4)) continue;
+        const bool full = s == 0 && !P.divided[0];  // r as it lies
+        if (full && !P.blocked[0]) {
+            const T *r0 = P.r0 + (size_t)inst * 3 * n;
+            for (int q = threadIdx.x; q < 3 * n; q += NT) sh[P.orr[0] + q] = r0[q];
+            if (sizeof(T) == 4) continue;
+        }
+        const int row = D.slots() / D.nz, lo = z0 * row, own = (z1 - z0) * row;
+        for (int colour = 0; colour < 2; colour++)
+#pragma unroll 2
+            for (int i = threadIdx.x; i < own; i += NT) {
+                int x, y, z, cst;
+                D.colour_cell(lo + i, colour, x, y, z);
+                if (x >= D.nx) continue;
+                const size_t id = (size_t)inst * 3 * n + tail_gidx(P, lut, s, x, y, z, 3, cst);
+                const int o = 3 * colour * own + i;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    if (s == 0 && !full) sh[P.orr[0] + o + c * own] = P.r0[id + (size_t)c * cst];
+                    if (full && P.blocked[0]) sh[P.orr[0] + c * n + D.id(x, y, z)] = P.r0[id + (size_t)c * cst];
+                    if (sizeof(T) == 8) sh[P.oi[s] + o + c * own] = P.inv[s][id + (size_t)c * cst];
+                }
+            }
+    }
+    tail_sync<CS>(true);  // every block of the cluster runs before its shared memory is written
+    const size_t inst3 = 3 * (size_t)inst;
+    int s = 0;
+    for (; s < P.n - 1; s++) {
+        tail_sweeps<T, CS>(P, sh, lut, inst3, s, nu1, true);
+        // residual and its restriction, 8 lanes per coarse cell: in float64 each with the three outer
+        // faces of its child (k_pair_op's octet form: the fluxes between the children cancel in their
+        // sum).  A block takes the coarse cells of its planes, or half of a coarse plane where it owns
+        // one fine plane.
+        const LexDims D = P.d[s], C = P.d[s + 1];
+        const int n = D.n(), ncs = C.n(), cpl = C.nx * C.ny;
+        const bool dv = P.divided[s];
+        const T *e = sh + P.oe[s], *E = sh + P.oE[s];
+        for (int q = threadIdx.x; q < 3 * ncs; q += NT) sh[P.oe[s + 1] + q] = T(0);
+        int z0, z1, lo, hi;
+        tail_planes<CS>(P, s, rank, z0, z1);
+        if (z1 - z0 == 1) {
+            const int mid = (z0 >> 1) * cpl + cpl / 2;
+            lo = (z0 & 1) ? mid : (z0 >> 1) * cpl;
+            hi = (z0 & 1) ? ((z0 >> 1) + 1) * cpl : mid;
+        } else {
+            lo = (z0 >> 1) * cpl;
+            hi = (z1 >> 1) * cpl;
+        }
+        for (int w0 = 8 * lo + (threadIdx.x & ~31); w0 < 8 * hi; w0 += NT) {
+            const int w = min(w0 + (int)(threadIdx.x & 31), 8 * hi - 1);  // the tail lanes repeat the last child
+            const int cq = w >> 3, ch = w & 7;
+            int x, y, z, cst;
+            C.cell(cq, x, y, z);
+            x = 2 * x + (ch & 1);
+            y = 2 * y + ((ch >> 1) & 1);
+            z = 2 * z + (ch >> 2);
+            const int q = D.id(x, y, z);
+            const LexAcc<T> a = D.acc(e, E, x, y, z);
+            T o[3];
+            if constexpr (sizeof(T) == 8) {
+                const int X = a.xo[1], Y = a.yo[1], Z = a.zo[1];
+                const int xs = (x & 1) ? a.xo[2] : a.xo[0], ys = (y & 1) ? a.yo[2] : a.yo[0], zs = (z & 1) ? a.zo[2] : a.zo[0];
+                const T qx = (x & 1) ? T(0.25) : T(-0.25), qy = (y & 1) ? T(0.25) : T(-0.25), qz = (z & 1) ? T(0.25) : T(-0.25);
+                const T eta0 = E[q];
+                const T esx = v_add(eta0, E[Z + Y + xs]), esy = v_add(eta0, E[Z + ys + X]), esz = v_add(eta0, E[zs + Y + X]);
+                const T *Bx = e, *By = e + n, *Bz = e + 2 * n;
+                o[0] = v_add(tail_face(By, Bx, q, Z + ys + X, Z + Y + a.xo[2], Z + Y + a.xo[0], Z + ys + a.xo[2], Z + ys + a.xo[0], qy, esy),
+                             tail_face(Bz, Bx, q, zs + Y + X, Z + Y + a.xo[2], Z + Y + a.xo[0], zs + Y + a.xo[2], zs + Y + a.xo[0], qz, esz));
+                o[1] = v_add(tail_face(Bx, By, q, Z + Y + xs, Z + a.yo[2] + X, Z + a.yo[0] + X, Z + a.yo[2] + xs, Z + a.yo[0] + xs, qx, esx),
+                             tail_face(Bz, By, q, zs + Y + X, Z + a.yo[2] + X, Z + a.yo[0] + X, zs + a.yo[2] + X, zs + a.yo[0] + X, qz, esz));
+                o[2] = v_add(tail_face(Bx, Bz, q, Z + Y + xs, a.zo[2] + Y + X, a.zo[0] + Y + X, a.zo[2] + Y + xs, a.zo[0] + Y + xs, qx, esx),
+                             tail_face(By, Bz, q, Z + ys + X, a.zo[2] + Y + X, a.zo[0] + Y + X, a.zo[2] + ys + X, a.zo[0] + ys + X, qy, esy));
+            } else {
+                T es[6];
+                face_sums<T>(a, es);
+                cell_divergence<T>(a, es, o);
+            }
+            size_t id = 0;
+            if (s == 0) id = inst3 * n + tail_gidx(P, lut, 0, x, y, z, 3, cst);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const T rv = s == 0 && (dv || !P.own) ? P.r0[id + (size_t)c * cst] : sh[P.orr[s] + c * n + q];
+                T v = v_mad(P.K[s].ncoef, o[c], v_sub(rv, e[c * n + q]));
+                if constexpr (sizeof(T) == 8) {
+                    v = v_add(v, __shfl_xor_sync(0xffffffffu, v, 1));
+                    v = v_add(v, __shfl_xor_sync(0xffffffffu, v, 2));
+                    v = v_add(v, __shfl_xor_sync(0xffffffffu, v, 4));
+                } else {  // the children in memory order
+                    const T t = v;
+                    v = __shfl_sync(0xffffffffu, t, threadIdx.x & 24);
+#pragma unroll
+                    for (int k = 1; k < 8; k++) v = v_add(v, __shfl_sync(0xffffffffu, t, (threadIdx.x & 24) + k));
+                }
+                if (ch == c) tail_store_all<CS>(sh, P.orr[s + 1] + c * ncs + cq, v_mul(v, T(0.125)), dv);
+            }
+        }
+        tail_sync<CS>(dv);
+    }
+    bool done = false;
+    if constexpr (sizeof(T) == 8) {
+        if (!P.divided[s] && P.d[s].slots() <= TAIL_REG_SLOTS) {
+            tail_coarsest(P, sh, lut, inst3, s, nc);
+            done = true;
+        }
+    }
+    if (!done) tail_sweeps<T, CS>(P, sh, lut, inst3, s, nc, true);
+    for (s = P.n - 2; s >= 0; s--) {
+        const LexDims D = P.d[s], C = P.d[s + 1];
+        const int n = D.n(), ncs = C.n(), pl = D.nx * D.ny;
+        int z0, z1;
+        if (CS > 1 && P.divided[s + 1]) {  // every block reads the coarse correction: hand out the own planes
+            const int cpl = C.nx * C.ny;
+            tail_planes<CS>(P, s + 1, rank, z0, z1);
+            for (int i = threadIdx.x; i < 3 * (z1 - z0) * cpl; i += NT) {
+                const int c = i / ((z1 - z0) * cpl), o = P.oe[s + 1] + c * ncs + z0 * cpl + i - c * (z1 - z0) * cpl;
+                tail_store_all<CS>(sh, o, sh[o], true);
+            }
+            tail_sync<CS>(true);
+        }
+        const T *ec = sh + P.oe[s + 1];
+        tail_planes<CS>(P, s, rank, z0, z1);
+        for (int i = threadIdx.x; i < (z1 - z0) * pl; i += NT) {  // trilinear prolongation (weights 3/4, 1/4)
+            int x, y, z;
+            D.cell(z0 * pl + i, x, y, z);
+            const int px = x >> 1, py = y >> 1, pz = z >> 1;
+            int nx = px + ((x & 1) ? 1 : -1), ny = py + ((y & 1) ? 1 : -1), nz = pz + ((z & 1) ? 1 : -1);  // periodic wrap
+            nx = nx < 0 ? nx + C.nx : (nx >= C.nx ? nx - C.nx : nx);
+            ny = ny < 0 ? ny + C.ny : (ny >= C.ny ? ny - C.ny : ny);
+            nz = nz < 0 ? nz + C.nz : (nz >= C.nz ? nz - C.nz : nz);
+            T v[3] = {T(0), T(0), T(0)};
+#pragma unroll
+            for (int ak = 0; ak < 2; ak++)
+#pragma unroll
+                for (int aj = 0; aj < 2; aj++)
+#pragma unroll
+                    for (int ai = 0; ai < 2; ai++) {
+                        const T wt = (ai ? T(0.25) : T(0.75)) * (aj ? T(0.25) : T(0.75)) * (ak ? T(0.25) : T(0.75));
+                        const int o = C.id(ai ? nx : px, aj ? ny : py, ak ? nz : pz);
+#pragma unroll
+                        for (int c = 0; c < 3; c++) v[c] = v_mad(wt, ec[c * ncs + o], v[c]);
+                    }
+            const int o = P.oe[s] + z0 * pl + i;
+#pragma unroll
+            for (int c = 0; c < 3; c++) v[c] = v_add(sh[o + c * n], v[c]);
+            tail_store_cell<CS>(P, sh, s, z, o, n, v, rank);  // no other block reads this cell in the pass
+        }
+        tail_sync<CS>(P.divided[s]);
+        tail_sweeps<T, CS>(P, sh, lut, inst3, s, nu2, false);
+    }
+    // e of the first grid: the own planes, or a share of the whole copy
+    const LexDims D = P.d[0];
+    const int n = D.n(), pl = D.nx * D.ny;
+    int z0, z1;
+    tail_planes<CS>(P, 0, rank, z0, z1);
+    const int step = CS > 1 && !P.divided[0] ? CS * NT : NT;
+    for (int q = z0 * pl + threadIdx.x + (CS > 1 && !P.divided[0] ? rank * NT : 0); q < z1 * pl; q += step) {
+        int x, y, z, cst;
+        D.cell(q, x, y, z);
+        const size_t id = inst3 * n + tail_gidx(P, lut, 0, x, y, z, 3, cst);
+#pragma unroll
+        for (int c = 0; c < 3; c++) P.e0[id + (size_t)c * cst] = sh[P.oe[0] + c * n + q];
+    }
+}
 
 static int ilog2_exact(int v) {
     int l = 0;
@@ -3037,52 +3292,139 @@ static int ilog2_exact(int v) {
     return (1 << l) == v ? l : -1;
 }
 
-// the shared-memory solver's grid table and its shared-memory bytes; false when the grids do
-// not fit
-static bool bottom_table(const SmallDev<float> &sm, double lamdt, BottomSm &P, size_t &bytes) {
-    P.n = sm.n;
-    size_t off = 0;
-    for (int q = 0; q < sm.n; q++) {
-        const int lx = ilog2_exact(sm.dims[q][0]), ly = ilog2_exact(sm.dims[q][1]), lz = ilog2_exact(sm.dims[q][2]);
-        P.d[q] = LexDims{sm.dims[q][0], sm.dims[q][1], sm.dims[q][2], lx, ly, lx >= 0 && ly >= 0 && lz >= 0};
-        P.base[q] = (int)off;
-        P.K[q] = rb_constants<float>(lamdt, sm.h[q], sm.omega);
-        off += 10 * (size_t)sm.dims[q][0] * sm.dims[q][1] * sm.dims[q][2];
-        off = (off + 3) & ~(size_t)3;
-    }
-    bytes = off * sizeof(float);
-    return bytes <= BOTTOM_SMEM_MAX;
+// cluster size: enough thread blocks per instance to use the SMs, and no more than one wave of them.
+// float64 takes 16 (the largest the hardware forms, beyond the portable 8) for few instances: its
+// passes are bound by the SMs' float64 units.
+static bool tail_16();
+template <typename T>
+static int tail_cluster(int ninst) {
+    if (sizeof(T) == 8 && ninst <= 8 && tail_16()) return 16;
+    return ninst <= 19 ? 8 : (ninst <= 38 ? 4 : (ninst <= 76 ? 2 : 1));
 }
 
-bool bottom_in_shared(const SmallDev<float> &sm) {
-    BottomSm P;
+// the solver's table and shared-memory bytes; false when the grids do not fit
+template <typename T>
+static bool tail_plan(const SmallDev<T> &sm, double lamdt, int cs, bool own, TailP<T> &P, size_t &bytes) {
+    P.n = sm.n;
+    P.own = own;
+    P.om1 = (T)(1.0 - sm.omega);
+    P.imask = sm.imask;
+    P.r0 = sm.r[0];
+    P.e0 = sm.e[0];
+    size_t off = 0, tmax = 0;
+    int lut = 0;
+    auto take = [&](size_t n) {
+        const size_t o = off;
+        off = (off + n + 3) & ~(size_t)3;
+        return (int)o;
+    };
+    for (int s = 0; s < sm.n; s++) {
+        const int lx = ilog2_exact(sm.dims[s][0]), ly = ilog2_exact(sm.dims[s][1]), lz = ilog2_exact(sm.dims[s][2]);
+        const LexDims d{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2], lx, ly, lx >= 0 && ly >= 0 && lz >= 0};
+        const size_t n = (size_t)d.nx * d.ny * d.nz;
+        if (n > 16384) return false;
+        P.d[s] = d;
+        P.divided[s] = cs > 1 && n > (size_t)tail_divide<T>();
+        // planes per block: one, or an even number (whole octets) where the grid is restricted
+        P.hz[s] = P.divided[s] ? (d.nz + cs - 1) / cs : d.nz;
+        if (P.divided[s] && P.hz[s] > 1) P.hz[s] += P.hz[s] & 1;
+        const size_t per = (size_t)(d.slots() / d.nz) * P.hz[s];
+        P.oe[s] = take(3 * n);
+        P.oE[s] = take(n);
+        P.orr[s] = take(s > 0 || (own && !P.divided[s]) ? 3 * n : (own ? 6 * per : 0));
+        P.oi[s] = sizeof(T) == 8 && own ? take(6 * per) : 0;
+        tmax = std::max(tmax, 3 * per);
+        P.K[s] = rb_constants<T>(lamdt, sm.h[s], sm.omega);
+        P.inv[s] = sm.inv[s];
+        P.eta[s] = sm.eta[s];
+        P.blocked[s] = sm.origin[s] != nullptr;
+        P.origin[s] = sm.origin[s];
+        P.lut[s] = lut;
+        P.nbx[s] = d.nx / BS;
+        P.nby[s] = d.ny / BS;
+        P.nblk[s] = P.blocked[s] ? (int)(n / B3) : 0;
+        lut += P.nblk[s];
+    }
+    P.ot = take(tmax);
+    bytes = off * sizeof(T);
+    return bytes <= TAIL_SMEM_MAX && lut <= TAIL_LUT;
+}
+
+// decided for one thread block per instance, so that an instance takes the same grids (and gives the
+// same bits) alone and in any batch
+template <typename T>
+bool tail_fits(const SmallDev<T> &sm) {
+    TailP<T> P;
     size_t bytes = 0;
-    return sm.n > 0 && bottom_table(sm, 1.0, P, bytes);
+    return sm.n > 0 && tail_plan(sm, 1.0, 1, false, P, bytes);
+}
+template bool tail_fits<double>(const SmallDev<double> &);
+template bool tail_fits<float>(const SmallDev<float> &);
+
+template <typename T, int CS>
+static void tail_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, int ninst, size_t bytes, cudaStream_t s) {
+    static const bool attr = (cudaFuncSetAttribute(k_tail<T, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_MAX),
+                              CS > 8 ? cudaFuncSetAttribute(k_tail<T, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess,
+                              true);
+    (void)attr;
+    cfg = {};
+    cfg.gridDim = dim3((unsigned)(ninst * CS));
+    cfg.blockDim = dim3(TailThreads<T, CS>::N);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CS;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = CS > 1 ? 1 : 0;
+}
+
+template <typename T, int CS>
+static cudaError_t launch_tail_cs(const TailP<T> &P, int ninst, size_t bytes, int nu_pre, int nu_post, int n_coarse,
+                                  cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    tail_config<T, CS>(cfg, at, ninst, bytes, s);
+    return cudaLaunchKernelEx(&cfg, k_tail<T, CS>, P, nu_pre, nu_post, n_coarse);
+}
+
+// whether the device can hold a cluster of 16 of the float64 solver's blocks (asked once)
+static bool tail_16() {
+    static const bool ok = [] {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        tail_config<double, 16>(cfg, at, 1, TAIL_SMEM_MAX, nullptr);
+        int n = 0;
+        const bool fits = cudaOccupancyMaxActiveClusters(&n, k_tail<double, 16>, &cfg) == cudaSuccess && n > 0;
+        cudaGetLastError();
+        return fits;
+    }();
+    return ok;
 }
 
 template <typename T>
-cudaError_t launch_bottom(const SmallDev<T> &sm, double lamdt, int nu_pre, int nu_post, int n_coarse, cudaStream_t s) {
+cudaError_t launch_tail(const SmallDev<T> &sm, double lamdt, int nu_pre, int nu_post, int n_coarse, cudaStream_t s) {
     if (sm.n == 0) return cudaSuccess;
-    if constexpr (std::is_same<T, float>::value) {
-        // shared-memory solver when the grids fit
-        BottomSm P;
-        size_t bytes = 0;
-        if (bottom_table(sm, lamdt, P, bytes)) {
-            static const bool attr =
-                (cudaFuncSetAttribute(k_bottom_sm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BOTTOM_SMEM_MAX), true);
-            (void)attr;
-            k_bottom_sm<<<sm.ninst, 1024, bytes, s>>>(sm, P, nu_pre, nu_post, n_coarse);
-            return cudaGetLastError();
-        }
+    TailP<T> P;
+    size_t bytes = 0;
+    const int cs = tail_cluster<T>(sm.ninst);
+    if (!tail_plan(sm, lamdt, cs, true, P, bytes) && !tail_plan(sm, lamdt, cs, false, P, bytes))
+        return cudaErrorInvalidValue;  // callers ask tail_fits first
+    if constexpr (sizeof(T) == 8) {
+        if (cs == 16) return launch_tail_cs<T, 16>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
     }
-    k_bottom<T><<<sm.ninst, 1024, 0, s>>>(sm, lamdt, nu_pre, nu_post, n_coarse);
-    return cudaGetLastError();
+    switch (cs) {
+        case 8: return launch_tail_cs<T, 8>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
+        case 4: return launch_tail_cs<T, 4>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
+        case 2: return launch_tail_cs<T, 2>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
+        default: return launch_tail_cs<T, 1>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
+    }
 }
-template cudaError_t launch_bottom<double>(const SmallDev<double> &, double, int, int, int, cudaStream_t);
-template cudaError_t launch_bottom<float>(const SmallDev<float> &, double, int, int, int, cudaStream_t);
+template cudaError_t launch_tail<double>(const SmallDev<double> &, double, int, int, int, cudaStream_t);
+template cudaError_t launch_tail<float>(const SmallDev<float> &, double, int, int, int, cudaStream_t);
 
-// Lexicographic grids too large for the one-block solver, stepped by grid-wide launches over
-// all instances (thread per instance and cell): the same arithmetic as k_bottom, one kernel per
+// Lexicographic grids too large for the cluster solver, stepped by grid-wide launches over
+// all instances (thread per instance and cell), one kernel per
 // colour pass (e_in -> e_out, the other colour copied), per residual, per restriction and per
 // prolongation.
 template <typename T>

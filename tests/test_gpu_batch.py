@@ -338,3 +338,31 @@ def test_fgmres_batch_takes_fewer_cycles(ohm):
         assert status == ohm.OHM_OK
         cyc[kr] = [x["cycles"] for x in st]
     assert all(a < b for a, b in zip(cyc[6], cyc[0])), cyc
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("base", [(32, 32, 32), (48, 16, 32), (16, 24, 40)])
+def test_coarse_solver_clusters_give_same_bits_and_match_oracle(ohm, orc, base, precision):
+    """The coarsest-grid solver runs an instance on 8, 4, 2 or 1 thread blocks by the number of
+    instances (up to 19, 38, 76, more): blocked grids among its own (16^3, 24x8x16), extents that are no
+    powers of two, odd ones (2x3x5).  The first instance gives the same bits in every batch, and in
+    float64 the fixed schedule's result is the oracle's."""
+    h = W.uniform(*base, 1.0 / base[0])
+    bs, etas = instances(h, 2, 300)
+    dts = [6.0 * h.dx0 ** 2, 9.0 * h.dx0 ** 2]
+    got = []
+    for K in (1, 20, 40, 80):
+        pick = [0] + [1] * (K - 1)
+        g = make(ohm, h, K, precision=precision, nu_pre=2, nu_post=1, n_coarse=5, max_outer=2)
+        ohm.ohm_set_eta(g, dev(stack(h, [etas[q] for q in pick])))
+        B = dev(stack(h, [bs[q] for q in pick]))
+        ohm.ohm_cn_step_batch(g, B, [dts[q] for q in pick], -1.0)
+        out = unstack(h, host(B).reshape(-1, 3, 8, 8, 8), K)
+        got.append(out[0])
+        assert np.array_equal(out[0], got[0])
+        if precision == 0:
+            for q in {0, K - 1}:
+                o = orc.Oracle(h, 0.5, etas[pick[q]])
+                want, _ = o.cn_step(bs[pick[q]], dts[pick[q]], -1.0, 2, 1, 5, 2)
+                assert rel_err(out[q], want) < 1e-12
+        g.close()
