@@ -984,9 +984,12 @@ int base_vcycle(ohm_hier *H, int m, double lamdt) {
                resid_restrict_base<T>(H, *G.g, (const T *)G.e, (const T *)G.r, (const T *)G.eta, lamdt, nullptr, (T *)C.r,
                                       nullptr, nullptr));
         if ((st = base_vcycle<T>(H, m + 1, lamdt))) return st;
-        if (G.g->octet)
-            LAUNCH(H, OHM_K_PROLONG, G.g->n(), launch_prolong_add8<T>(gdev(H, *C.g), (const T *)C.e, (T *)G.e, H->s));
-        else
+        bool octet = false;
+        if constexpr (std::is_same<T, float>::value) {
+            octet = G.g->octet;
+            if (octet) LAUNCH(H, OHM_K_PROLONG, G.g->n(), launch_prolong_add8<T>(gdev(H, *C.g), (const T *)C.e, (T *)G.e, H->s));
+        }
+        if (!octet)
             LAUNCH(H, OHM_K_PROLONG, G.g->n(), launch_prolong_add<T>(gdev(H, *G.g), &C.g->dev, (const T *)C.e, nullptr, nullptr, (T *)G.e, H->d_err, H->s));
     } else {
         LAUNCH(H, OHM_K_RESID_RESTRICT, G.g->n(), launch_resid_restrict<T>(gdev(H, *G.g), (const T *)G.e, (const T *)G.r, (const T *)G.eta, nullptr, nullptr, lamdt,

@@ -1886,6 +1886,125 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 4 : 1) k_resid_restrict(
     }
 }
 
+// float64 residual and its restriction without the fine residual.  Bound by the float64 pipe: the
+// octet sums of the flux divergence need only the fluxes through the octets' outer faces
+// (k_pair_op's octet form), every one of which bounds two octets, so a thread takes one side of an
+// octet (2 x 2 faces) and forms sum es (T/4 - N) over it for both flux components, from pair sums as
+// in k_smooth_d, once for the two octets it separates: about 27 operations per cell instead of 66.
+// Slabs of NZ planes as there.  t = r - e + kc divF summed over an octet and divided by 8 goes to the
+// coarser grid.
+template <int NZ>
+struct OctD {
+    static constexpr int NT = 32 * NZ, NP = NZ + 2, NZO = NZ / 2;
+    static constexpr int CS = 100 * NP;
+    static constexpr int PXY = 50 * NP;                        // 5 face planes of 10 NP sums
+    static constexpr int SUMS = 2 * PXY + 100 * (NZO + 1);
+    static constexpr int SXY = 5 * 4 * NZO, SZ = (NZO + 1) * 16, SIDES = 2 * SXY + SZ;
+    static constexpr size_t BYTES = (4 * CS + SUMS + 2 * SIDES) * sizeof(double);
+};
+
+template <int NZ, int NF, int NV>
+__device__ __forceinline__ void octet_sums_axis(const double *__restrict__ Ba, double *__restrict__ P, int sa, int su, int sv) {
+    constexpr int FULL = 10 * NV - 4;
+    for (int e = threadIdx.x; e < NF * FULL; e += OctD<NZ>::NT) {
+        const int f = e / FULL;
+        int u, v;
+        cross_pos<NV>(e - f * FULL, u, v);
+        const double *p = Ba + 2 * f * sa + u * su + v * sv;
+        P[(f * NV + v) * 10 + u] = p[sa] + p[0];
+    }
+}
+
+template <int NZ>
+__global__ void __launch_bounds__(32 * NZ) k_resid_restrict_d(GridDev g, const double *__restrict__ e, const double *__restrict__ r,
+                                                              const double *__restrict__ eta, const double *__restrict__ Ge,
+                                                              const double *__restrict__ Geta, double kc, double *__restrict__ coarse,
+                                                              double *__restrict__ lex, int3 ld) {
+    using S = OctD<NZ>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS, *side = P + S::SUMS;
+    __shared__ int snb[27];
+    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
+    if (skip_block(g, b)) return;
+    const int slot = g.gslot ? g.gslot[b] : -1, t = threadIdx.x;
+    if (NZ == 2 || t < 32) stage_nbr(snb, g.nbr, b);
+    __syncthreads();
+    stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
+    stage_slab<NZ, 3>(tB, e, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr, z0);
+    __syncthreads();
+    octet_sums_axis<NZ, 5, NZ + 2>(tB, P, 1, 10, 100);
+    octet_sums_axis<NZ, 5, NZ + 2>(tB + S::CS, P + S::PXY, 10, 1, 100);
+    octet_sums_axis<NZ, S::NZO + 1, 10>(tB + 2 * S::CS, P + 2 * S::PXY, 100, 1, 10);
+    __syncthreads();
+    // sides: face plane f (tile cell 2f and the next along the axis), octet (m, n) of the cross-section
+    for (int q = t; q < S::SIDES; q += S::NT) {
+        const int ax = q < S::SXY ? 0 : (q < 2 * S::SXY ? 1 : 2);
+        const int h = q - ax * S::SXY;
+        const int per = ax == 2 ? 16 : 4 * S::NZO, f = h / per, m = (h - f * per) & 3, n = (h - f * per) >> 2;
+        const int sa = ax == 0 ? 1 : (ax == 1 ? 10 : 100), su = ax == 0 ? 10 : 1, sv = ax == 2 ? 10 : 100;
+        const int NV = ax == 2 ? 10 : NZ + 2;
+        const double *B1 = tB + (ax == 0 ? 1 : 0) * S::CS, *B2 = tB + (ax == 2 ? 1 : 2) * S::CS;
+        double s1 = 0.0, s2 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int u = 2 * m + 1 + (k & 1), v = 2 * n + 1 + (k >> 1), p = 2 * f * sa + u * su + v * sv;
+            const double *Pa = P + ax * S::PXY + (f * NV + v) * 10 + u;
+            const double es = tE[p] + tE[p + sa];
+            const double g1 = fma(0.25, Pa[1] - Pa[-1], B1[p] - B1[p + sa]);
+            const double g2 = fma(0.25, Pa[10] - Pa[-10], B2[p] - B2[p + sa]);
+            s1 = k ? fma(es, g1, s1) : es * g1;
+            s2 = k ? fma(es, g2, s2) : es * g2;
+        }
+        side[q] = s1;
+        side[S::SIDES + q] = s2;
+    }
+    __syncthreads();
+    // one thread per octet and component
+    for (int q = t; q < 48 * S::NZO; q += S::NT) {
+        const int c = q / (16 * S::NZO), w = q - c * (16 * S::NZO), ci = w & 3, cj = (w >> 2) & 3, ck = w >> 4;
+        // the two axes of the component's fluxes: its own flux component index on them
+        auto net = [&](int ax) {
+            const int comp = ax == 0 ? (c == 1 ? 0 : 1) : (ax == 1 ? (c == 0 ? 0 : 1) : c);
+            const int m = ax == 0 ? cj : ci, n = ax == 2 ? cj : ck, f = ax == 0 ? ci : (ax == 1 ? cj : ck);
+            const int per = ax == 2 ? 16 : 4 * S::NZO;
+            const double *sd = side + comp * S::SIDES + ax * S::SXY + f * per + n * 4 + m;
+            return sd[per] - sd[0];
+        };
+        const double div = c == 0 ? net(1) + net(2) : (c == 1 ? net(0) + net(2) : net(0) + net(1));
+        double sum = 0.0;
+        const double *tc = tB + c * S::CS;
+        const double *rc = r + ((size_t)b * 3 + c) * B3;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const int x = 2 * ci + (k & 1), y = 2 * cj + ((k >> 1) & 1), z = 2 * ck + (k >> 2);
+            const double d = rc[((z0 + z) * 8 + y) * 8 + x] - tc[(z + 1) * 100 + (y + 1) * 10 + x + 1];
+            sum = k ? sum + d : d;
+        }
+        const double v = 0.125 * fma(kc, div, sum);
+        const int cz = (z0 >> 1) + ck;
+        if (coarse) {
+            const int pb = g.parent[b], o = g.octant[b];
+            const int x = 4 * (o & 1) + ci, y = 4 * ((o >> 1) & 1) + cj, z = 4 * (o >> 2) + cz;
+            coarse[((size_t)pb * 3 + c) * B3 + (z * 8 + y) * 8 + x] = v;
+        } else {
+            const int x = 4 * g.origin[b * 3 + 0] + ci, y = 4 * g.origin[b * 3 + 1] + cj, z = 4 * g.origin[b * 3 + 2] + cz;
+            double *lx = lex + lex_inst_offset(g, b, 3, ld);
+            lx[(((size_t)c * ld.z + z) * ld.y + y) * ld.x + x] = v;
+        }
+    }
+}
+
+template <int NZ>
+static cudaError_t launch_resid_restrict_slab(const GridDev &g, const double *e, const double *r, const double *eta,
+                                              const double *Ge, const double *Geta, double kc, double *coarse, double *lex,
+                                              int3 ld, cudaStream_t s) {
+    using S = OctD<NZ>;
+    static const bool attr = (cudaFuncSetAttribute(k_resid_restrict_d<NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES), true);
+    (void)attr;
+    k_resid_restrict_d<NZ><<<g.nblk * (8 / NZ), S::NT, S::BYTES, s>>>(g, e, r, eta, Ge, Geta, kc, coarse, lex, ld);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_resid_restrict(const GridDev &g, const T *e, const T *r, const T *eta, const T *Ge, const T *Geta,
                                   double lamdt, T *t_out, T *coarse, T *lex, const int *ldims, cudaStream_t s) {
@@ -1895,6 +2014,14 @@ cudaError_t launch_resid_restrict(const GridDev &g, const T *e, const T *r, cons
     static const bool attr = (cudaFuncSetAttribute(k_resid_restrict<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
     (void)attr;
     int3 ld = make_int3(ldims ? ldims[0] : 0, ldims ? ldims[1] : 0, ldims ? ldims[2] : 0);
+    if constexpr (std::is_same<T, double>::value) {
+        if (!t_out && (coarse || lex)) {  // slab height as for the colour passes
+            const double kc = -lamdt / (2.0 * g.h * g.h);
+            if (g.nblk <= SLAB2_BLOCKS) return launch_resid_restrict_slab<2>(g, e, r, eta, Ge, Geta, kc, coarse, lex, ld, s);
+            if (g.nblk <= SLAB4_BLOCKS) return launch_resid_restrict_slab<4>(g, e, r, eta, Ge, Geta, kc, coarse, lex, ld, s);
+            return launch_resid_restrict_slab<8>(g, e, r, eta, Ge, Geta, kc, coarse, lex, ld, s);
+        }
+    }
     k_resid_restrict<T><<<g.nblk, 512, sm, s>>>(g, e, r, eta, Ge, Geta, (T)(lamdt / (2.0 * g.h * g.h)), t_out, coarse,
                                                 lex, ld);
     return cudaGetLastError();
@@ -1994,13 +2121,84 @@ __global__ void __launch_bounds__(512) k_prolong_add(GridDev g, GridDev gc, cons
     }
 }
 
+// float64 prolongation.  Bound by the float64 pipe (8 multiply-adds per value above), so the
+// interpolation is separable: along x over the window's 6 x 6 rows, along y over 6 planes, along z
+// into the cells, each intermediate value formed once in shared memory: 12 operations per cell
+// instead of 27, and a thread block per fine block also where one coarse block's 8 children fill the
+// grid.  128^3: 134 us with the one-pass form on coarse blocks, one coarse block alone 36 us.
+__global__ void __launch_bounds__(256) k_prolong_add_d(GridDev g, GridDev gc, const double *__restrict__ coarse,
+                                                       const double *__restrict__ lex, int3 ld, double *__restrict__ fine,
+                                                       int *__restrict__ err) {
+    __shared__ double win[3 * 216], wx8[3 * 288], wy8[3 * 384];  // [6][6][6], [6][6][8], [6][8][8] per component
+    const int b = blockIdx.x;
+    if (skip_block(g, b)) return;
+    const int o = lex ? 0 : g.octant[b];
+    const int pb = lex ? 0 : g.parent[b];
+    const int t = threadIdx.x;
+    for (int q = t; q < 216; q += 256) {
+        const int wx = q % 6, wy = (q / 6) % 6, wz = q / 36;
+        if (lex) {
+            int x = 4 * g.origin[b * 3 + 0] - 1 + wx, y = 4 * g.origin[b * 3 + 1] - 1 + wy, z = 4 * g.origin[b * 3 + 2] - 1 + wz;
+            x = (x + ld.x) % ld.x; y = (y + ld.y) % ld.y; z = (z + ld.z) % ld.z;
+            const double *lx = lex + lex_inst_offset(g, b, 3, ld);
+            for (int c = 0; c < 3; c++) win[c * 216 + q] = lx[(((size_t)c * ld.z + z) * ld.y + y) * ld.x + x];
+        } else {
+            const int cx = 4 * (o & 1) - 1 + wx, cy = 4 * ((o >> 1) & 1) - 1 + wy, cz = 4 * (o >> 2) - 1 + wz;
+            const int dx = cx < 0 ? -1 : (cx > 7 ? 1 : 0), dy = cy < 0 ? -1 : (cy > 7 ? 1 : 0), dz = cz < 0 ? -1 : (cz > 7 ? 1 : 0);
+            const int src = gc.nbr[pb * 27 + (dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)];
+            if (src < 0) {
+                if (err) *err = 1;
+                for (int c = 0; c < 3; c++) win[c * 216 + q] = 0.0;
+            } else {
+                const int lx = cx - 8 * dx, ly = cy - 8 * dy, lz = cz - 8 * dz;
+                for (int c = 0; c < 3; c++) win[c * 216 + q] = coarse[((size_t)src * 3 + c) * B3 + (lz * 8 + ly) * 8 + lx];
+            }
+        }
+    }
+    double old[2][3];  // the fine values come in while the window is interpolated
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int c = 0; c < 3; c++) old[h][c] = fine[((size_t)b * 3 + c) * B3 + t + 256 * h];
+    __syncthreads();
+    // fine cells 2w - 2 and 2w - 1 from window cell w = 1 .. 4 and its neighbours: (3 f0 + f-)/4, (3 f0 + f+)/4
+    for (int q = t; q < 3 * 144; q += 256) {
+        const int row = q >> 2, w = (q & 3) + 1;  // row: component and (z, y) of the window
+        const double *p = win + row * 6 + w;
+        const double m = 0.75 * p[0];
+        wx8[row * 8 + 2 * w - 2] = fma(0.25, p[-1], m);
+        wx8[row * 8 + 2 * w - 1] = fma(0.25, p[1], m);
+    }
+    __syncthreads();
+    for (int q = t; q < 3 * 6 * 32; q += 256) {
+        const int x = q & 7, w = ((q >> 3) & 3) + 1, cz = q >> 5;  // cz: component and z of the window
+        const double *p = wx8 + (cz * 6 + w) * 8 + x;
+        const double m = 0.75 * p[0];
+        wy8[(cz * 8 + 2 * w - 2) * 8 + x] = fma(0.25, p[-8], m);
+        wy8[(cz * 8 + 2 * w - 1) * 8 + x] = fma(0.25, p[8], m);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int q = t + 256 * h, k = q >> 6, w = (k >> 1) + 1, sz = (k & 1) ? 64 : -64;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const double *p = wy8 + (c * 6 + w) * 64 + (q & 63);
+            fine[((size_t)b * 3 + c) * B3 + q] = fma(0.25, p[sz], fma(0.75, p[0], old[h][c]));
+        }
+    }
+}
+
 template <typename T>
 cudaError_t launch_prolong_add(const GridDev &g, const GridDev *gc, const T *coarse, const T *lex, const int *ldims,
                                T *fine, int *err, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
     int3 ld = make_int3(ldims ? ldims[0] : 0, ldims ? ldims[1] : 0, ldims ? ldims[2] : 0);
     GridDev c = gc ? *gc : GridDev();
-    k_prolong_add<T><<<g.nblk, 512, 0, s>>>(g, c, coarse, lex, ld, fine, err);
+    if constexpr (std::is_same<T, double>::value)
+        k_prolong_add_d<<<g.nblk, 256, 0, s>>>(g, c, coarse, lex, ld, fine, err);
+    else
+        k_prolong_add<T><<<g.nblk, 512, 0, s>>>(g, c, coarse, lex, ld, fine, err);
     return cudaGetLastError();
 }
 template cudaError_t launch_prolong_add<double>(const GridDev &, const GridDev *, const double *, const double *,
@@ -2052,7 +2250,6 @@ cudaError_t launch_prolong_add8(const GridDev &gc, const T *coarse, T *fine, cud
     k_prolong_add8<T><<<gc.nblk, 512, 0, s>>>(gc, coarse, fine);
     return cudaGetLastError();
 }
-template cudaError_t launch_prolong_add8<double>(const GridDev &, const double *, double *, cudaStream_t);
 template cudaError_t launch_prolong_add8<float>(const GridDev &, const float *, float *, cudaStream_t);
 
 // ------------------------------------------------------------------ coarse-fine ghosts
