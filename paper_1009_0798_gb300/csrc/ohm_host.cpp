@@ -472,7 +472,9 @@ int allocate(ohm_hier *H, std::string &err, int64_t *dry_bytes = nullptr) {
     want((void **)&H->ghostB, (size_t)H->nslot * 3 * T3 * 8);
     want((void **)&H->ghostEta64, (size_t)H->nslot * T3 * 8);
     want((void **)&H->reg, (size_t)H->nreg * 128 * 8);
-    want((void **)&H->partials, n * 3 * 8);
+    size_t parts = 0;  // norm partials: the float64 composite writes several entries per block of a small level
+    for (auto &g : H->amr) parts += (size_t)g.n() * composite_parts(g.n());
+    want((void **)&H->partials, parts * 3 * 8);
     want((void **)&H->dnorm, 64);
     want((void **)&H->redscr, NORM_SCRATCH_BYTES);
     want(&H->ghostE, (size_t)H->nslot * 3 * T3 * tsz);
@@ -1043,14 +1045,36 @@ int fill_ghosts_B(ohm_hier *H, const double *B) {
     return OHM_OK;
 }
 
+// Where the composite's norm partials lie: several unscaled entries per block of a small level from the
+// float64 kernel, one scaled entry per block from the others
+PartRanges part_ranges(const ohm_hier *H, bool f64) {
+    PartRanges R;
+    R.nlev = H->nlev;
+    int base = 0;
+    for (int l = 0; l < H->nlev; l++) {
+        const HGrid &g = H->amr[l];
+        R.off[l] = g.off;
+        R.n[l] = H->batched ? H->ranges.n[l] : g.n();
+        R.base[l] = base;
+        R.parts[l] = f64 ? composite_parts(g.n()) : 1;
+        R.vol[l] = f64 ? g.h * g.h * g.h : 1.0;
+        base += g.n() * R.parts[l];
+    }
+    return R;
+}
+
 // out = a X + c divF(X) + d Y on leaf blocks of every level (finest first, so refluxed
 // fine fluxes are in the registers before the coarser level reads them), computed in TC.
 template <typename TC, typename TO>
 int composite_t(ohm_hier *H, const TC *X, const TC *Y, const TC *eta, const TC *Gx, const TC *Geta, double a, double c,
-                double dcoef, TO *out, TO *out2, bool norms, double *outS = nullptr, double c2 = 0.0, bool ff64 = false) {
+                double dcoef, TO *out, TO *out2, bool norms, double *outS = nullptr, double c2 = 0.0, bool ff64 = false,
+                bool keep_ss = false) {
+    const bool f64 = std::is_same<TC, double>::value && !ff64 && !(H->ff && std::is_same<TO, float>::value);
+    const PartRanges R = part_ranges(H, f64);
     for (int l = H->nlev - 1; l >= 0; l--) {
         const HGrid &g = H->amr[l];
-        double vol = g.h * g.h * g.h;
+        const double vol = g.h * g.h * g.h;
+        double *part = norms ? H->partials + (size_t)R.base[l] * 3 : nullptr;
         const size_t o3 = (size_t)g.off * 3 * B3;
         if constexpr (std::is_same<TC, double>::value && std::is_same<TO, float>::value) {
           if (ff64) {
@@ -1058,7 +1082,7 @@ int composite_t(ohm_hier *H, const TC *X, const TC *Y, const TC *eta, const TC *
             LAUNCH(H, OHM_K_COMPOSITE, g.n(),
                    launch_composite_df(gdev(H, g), X + o3, Y ? Y + o3 : nullptr, eta + (size_t)g.off * B3, Gx, Geta, a,
                                        c, dcoef, out + o3, out2 ? out2 + o3 : nullptr, H->reg, H->d_rsrc,
-                                       norms ? H->partials + (size_t)g.off * 3 : nullptr, vol, H->s));
+                                       part, vol, H->s));
             continue;
           }
           if (H->ff) {
@@ -1068,7 +1092,7 @@ int composite_t(ohm_hier *H, const TC *X, const TC *Y, const TC *eta, const TC *
                    (launch_composite_df(gdev(H, g), X + o3, Y ? reinterpret_cast<const dfloat *>(Y) + o3 : nullptr,
                                         eta + (size_t)g.off * B3, Gx, Geta, a, c, dcoef, out + o3,
                                         out2 ? out2 + o3 : nullptr, H->reg, H->d_rsrc,
-                                        norms ? H->partials + (size_t)g.off * 3 : nullptr, vol, H->s,
+                                        part, vol, H->s,
                                         outS ? reinterpret_cast<dfloat *>(outS) + o3 : nullptr, c2)));
             continue;
           }
@@ -1084,19 +1108,21 @@ int composite_t(ohm_hier *H, const TC *X, const TC *Y, const TC *eta, const TC *
                 continue;
             }
         }
-        {
+        if constexpr (std::is_same<TC, double>::value)
             LAUNCH(H, OHM_K_COMPOSITE, g.n(),
-                   (launch_composite<TC, TO>(gdev(H, g), X + o3, Y ? Y + o3 : nullptr, eta + (size_t)g.off * B3, Gx, Geta,
-                                             a, c, dcoef, out + o3, out2 ? out2 + o3 : nullptr, H->reg, H->d_rsrc,
-                                             norms ? H->partials + (size_t)g.off * 3 : nullptr, vol, H->s,
-                                             outS ? outS + o3 : nullptr, c2)));
-        }
+                   launch_composite<TO>(gdev(H, g), X + o3, Y ? Y + o3 : nullptr, eta + (size_t)g.off * B3, Gx, Geta, a, c, dcoef,
+                                        out + o3, out2 ? out2 + o3 : nullptr, H->reg, H->d_rsrc, part, H->s,
+                                        outS ? outS + o3 : nullptr, c2, keep_ss));
+        else
+            LAUNCH(H, OHM_K_COMPOSITE, g.n(),
+                   launch_composite(gdev(H, g), X + o3, Y ? Y + o3 : nullptr, eta + (size_t)g.off * B3, Gx, Geta, a, c, dcoef,
+                                    out + o3, out2 ? out2 + o3 : nullptr, H->reg, H->d_rsrc, part, vol, H->s));
     }
     if (norms) {
         if (H->batched)
-            LAUNCH(H, OHM_K_NORM, 0, launch_norm_inst(H->partials, H->ranges, H->K, H->dnormK, H->s));
+            LAUNCH(H, OHM_K_NORM, 0, launch_norm_inst(H->partials, R, H->K, H->dnormK, H->s));
         else
-            LAUNCH(H, OHM_K_NORM, 0, launch_norm_reduce(H->partials, (int)H->nblocks, H->redscr, H->dnorm, H->s,
+            LAUNCH(H, OHM_K_NORM, 0, launch_norm_reduce(H->partials, R, (int)H->nblocks, H->redscr, H->dnorm, H->s,
                                                         H->hnorm_dev, H->d_err));
     }
     return OHM_OK;
@@ -1105,9 +1131,9 @@ int composite_t(ohm_hier *H, const TC *X, const TC *Y, const TC *eta, const TC *
 // float64 composite operator on B-like fields (eta and ghosts of the state)
 template <typename TO>
 int composite(ohm_hier *H, const double *X, const double *Y, double a, double c, double dcoef, TO *out, bool norms,
-              TO *out2 = nullptr, bool ff64 = false) {
+              TO *out2 = nullptr, bool ff64 = false, bool keep_ss = false) {
     return composite_t<double, TO>(H, X, Y, H->eta64, H->ghostB, H->ghostEta64, a, c, dcoef, out, out2, norms, nullptr,
-                                   0.0, ff64);
+                                   0.0, ff64, keep_ss);
 }
 
 // The first residual of a step and its source from one flux divergence of b (Eqs. 14, 20):
@@ -1187,8 +1213,8 @@ int cn_step_impl(ohm_hier *H, double *B, double dt, double tol, ohm_step_stats *
     for (;;) {
         // the first residual comes with the source S from one flux divergence of b
         if ((st = it == 0 ? source_and_residual<T>(H, B, lam, dt, (T *)H->amrbuf.r, (T *)nullptr)
-                          : composite<T>(H, B, H->S, -1.0, -lamdt, 1.0, (T *)H->amrbuf.r, true)))
-            return st;
+                          : composite<T>(H, B, H->S, -1.0, -lamdt, 1.0, (T *)H->amrbuf.r, true, (T *)nullptr, false, true)))
+            return st;  // (later residuals keep sum S^2 of the first: nothing else wrote the partials)
         int ef = 0;
         if ((st = read_norms(H, nr, &ef))) return st;
         if (ef) return OHM_ERR_INVALID;
@@ -1467,9 +1493,13 @@ int cn_step_mixed(ohm_hier *H, double *B, double dt, double tol, ohm_step_stats 
     // bring below tol only sets the next inner solve's right-hand side, and is evaluated in
     // float-float (error about 2^-48 of the operands, far below any tol it is compared with).  A
     // float-float residual that meets tol is confirmed in float64.
+    // sum S^2 stays in the partials of the first residual unless the inner solve or a float-float
+    // residual has written its own there
+    bool keep = H->d.krylov > 0;
     auto outer_residual = [&](int outer, bool ff) -> int {
+        if (ff) keep = false;
         int s2 = outer == 0 ? source_and_residual<T>(H, B, lam, dt, r, rout)
-                            : composite<T>(H, B, H->S, -1.0, -lamdt, 1.0, r, true, rout, ff);
+                            : composite<T>(H, B, H->S, -1.0, -lamdt, 1.0, r, true, rout, ff, keep && !ff);
         if (s2) return s2;
         int ef = 0;
         if ((s2 = read_norms(H, nr, &ef))) return s2;
@@ -1801,7 +1831,7 @@ int cn_step_batch_t(ohm_hier *H, double *B, const double *dt, double tol, const 
     for (int outer = 0;; outer++) {
         T *r2 = H->mixed ? rout : (T *)nullptr;
         if ((st = outer == 0 ? source_and_residual<T>(H, B, lam, 1.0, r, r2)
-                             : composite<T>(H, B, H->S, -1.0, -lamdt, 1.0, r, true, r2)))
+                             : composite<T>(H, B, H->S, -1.0, -lamdt, 1.0, r, true, r2, false, !H->mixed || H->d.krylov > 0)))
             return st;
         if ((st = enqueue_norm_copy(H))) return st;
         int ef = 0;

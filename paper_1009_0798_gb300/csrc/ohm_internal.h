@@ -57,19 +57,25 @@ struct SmallDev {
 
 // ------------------------------------------------------------------ kernel launchers
 // Every launcher enqueues on `s` and returns cudaGetLastError().
-// Composite operator on AMR level g (float64): out = a X + c divF(X) + d Y on leaf blocks,
+// Composite operator on AMR level g: out = a X + c divF(X) + d Y on leaf blocks,
 // reading ghosts from Gx (level ghost slots) and eta ghosts from Geta; writes face fluxes to
 // registers for faces without a same-level neighbour and reads refluxed fluxes from the
-// finer level for faces next to covered blocks; optional per-block norm partials.
-// Computed in TC; out (and out2 when not null) receive the result as TO.
-// With outS (first residual of a step, Eqs. 14 and 20 from one flux divergence of X = b):
-// outS = a X + c divF(X) (the source S) and out = out2 = c2 divF(X) = S - L X for c2 = -dt;
-// the norm partials are then those of out against S.
-template <typename TC, typename TO>
-cudaError_t launch_composite(const GridDev &g, const TC *X, const TC *Y, const TC *eta, const TC *Gx,
-                             const TC *Geta, double a, double c, double d, TO *out, TO *out2,
-                             double *reg, const int *rsrc_tab, double *partials, double vol,
-                             cudaStream_t s, double *outS = nullptr, double c2 = 0.0);
+// finer level for faces next to covered blocks; optional norm partials (sum out^2, sum Y^2, max |out|).
+// out (and out2 when not null) receive the result as TO.
+// float64: composite_parts(g.nblk) unscaled entries of partials per block, to be added pairwise;
+// keep_ss leaves the entries of sum Y^2 as they are.  With outS (first residual of a step, Eqs. 14 and
+// 20 from one flux divergence of X = b): outS = a X + c divF(X) (the source S) and out = out2 =
+// c2 divF(X) = S - L X for c2 = -dt; the norm partials are then those of out against S.
+int composite_parts(int nblk);
+template <typename TO>
+cudaError_t launch_composite(const GridDev &g, const double *X, const double *Y, const double *eta, const double *Gx,
+                             const double *Geta, double a, double c, double d, TO *out, TO *out2, double *reg,
+                             const int *rsrc_tab, double *partials, cudaStream_t s, double *outS = nullptr,
+                             double c2 = 0.0, bool keep_ss = false);
+// float32: one entry per block, already scaled by the cell volume vol
+cudaError_t launch_composite(const GridDev &g, const float *X, const float *Y, const float *eta, const float *Gx,
+                             const float *Geta, double a, double c, double d, float *out, float *out2, double *reg,
+                             const int *rsrc_tab, double *partials, double vol, cudaStream_t s);
 
 // Float-float number: the unevaluated sum hi + lo of two float32 values (about 48 significant
 // bits).  The mixed-precision path evaluates its outer residual in this arithmetic on the
@@ -82,7 +88,7 @@ struct alignas(8) dfloat {
     constexpr explicit dfloat(float h = 0.f, float l = 0.f) : hi(h), lo(l) {}
 };
 
-// launch_composite for the outer residual of the mixed path: X, eta and the ghosts are float64
+// launch_composite for the outer residual of OHM_MIXED_FF (one scaled entry of partials per block): X, eta and the ghosts are float64
 // fields, split into float-float values when staged; Y and outS are the source in float-float
 // form; out / out2 are float32 (the inner solve's right-hand side).  Float-float arithmetic
 // keeps the error of R = S - L X near 2^-48 (1 + lambda dt |divF| / |X|) |X|, which bounds the
@@ -170,7 +176,14 @@ struct InstRanges {
     int off[MAX_LEVELS_DEV];
     int n[MAX_LEVELS_DEV];
 };
-cudaError_t launch_norm_inst(const double *partials, const InstRanges &R, int ninst, double *out, cudaStream_t s);
+// where a hierarchy's norm partials lie: level l owns blocks off[l] .. (n[l] per instance), its entries
+// start at base[l], parts[l] of them per block, to be scaled by vol[l]
+struct PartRanges {
+    int nlev = 0;
+    int off[MAX_LEVELS_DEV], n[MAX_LEVELS_DEV], base[MAX_LEVELS_DEV], parts[MAX_LEVELS_DEV];
+    double vol[MAX_LEVELS_DEV];
+};
+cudaError_t launch_norm_inst(const double *partials, const PartRanges &R, int ninst, double *out, cudaStream_t s);
 
 // dst[b][512] = src[b][512] * scale[b] (per-block scale of a block field)
 cudaError_t launch_scale_blocks(const double *src, double *dst, const double *scale, int nblk, cudaStream_t s);
@@ -184,8 +197,8 @@ constexpr size_t NORM_SCRATCH_BYTES = 128 * 3 * sizeof(double) + 16;
 // host_out (optional): pinned host memory mapped into the device that also receives the three
 // sums and, as an int at host_out + 4, the word *err (the caller reads them after synchronising,
 // without a copy)
-cudaError_t launch_norm_reduce(const double *partials, int nblocks, double *scratch, double *out, cudaStream_t s,
-                               double *host_out = nullptr, const int *err = nullptr);
+cudaError_t launch_norm_reduce(const double *partials, const PartRanges &R, int nblocks, double *scratch, double *out,
+                               cudaStream_t s, double *host_out = nullptr, const int *err = nullptr);
 
 // The V-cycle over all grids of sm (grid 0's r set, its e the result) in one launch, a cluster of
 // thread blocks per instance with the grids in shared memory.  tail_fits: whether they fit.  In

@@ -372,84 +372,6 @@ __device__ __forceinline__ void all_faces_512(const T *__restrict__ tB, const T 
     }
 }
 
-// float64 face fluxes with shared pair sums.  The tangential term of Eq. 10 is a difference of
-// two pair sums across the face, P_a(q) = B_a(q) + B_a(q + e_a), taken one cell apart along the
-// flux component's axis; every pair sum serves two faces, so computing the 2592 sums of a block
-// once (one float64 addition each) saves two additions per face flux, a fifth of the float64
-// work of the composite operator.  The sums are the same additions in the same order as in
-// face_phi_s, so the fluxes are bit-identical.  P holds, per axis a, [9 faces][10][10] sums over
-// the face's tile coordinates (u, v) along the two other axes in ascending order (corners unused).
-constexpr int PSUM = 3 * 900;
-__device__ __forceinline__ void pair_sums_512(const double *__restrict__ tB, double *__restrict__ P) {
-    using G = Geo<double>;
-    for (int e = threadIdx.x; e < PSUM; e += blockDim.x) {
-        const int a = e / 900, r = e - a * 900, fn = r / 100, v = (r / 10) % 10, u = r % 10;
-        if ((u == 0 || u == 9) && (v == 0 || v == 9)) continue;  // corners: never staged, never read
-        int p, sa;
-        if (a == 0) { p = G::at(fn, u, v) ; sa = 1; }           // x faces: (u, v) = (y, z)
-        else if (a == 1) { p = G::at(u, fn, v); sa = G::RS; }  // y faces: (u, v) = (x, z)
-        else { p = G::at(u, v, fn); sa = G::PS; }              // z faces: (u, v) = (x, y)
-        const double *Ba = tB + a * G::CS;
-        P[e] = Ba[p + sa] + Ba[p];
-    }
-}
-
-// Phi of the face with low tile cell p along axis a (tile tangential coordinates u0, v0), from
-// the pair sums; the normal differences and eta as in face_phi_s.
-__device__ __forceinline__ void face_phi_p(const double *__restrict__ tB, const double *__restrict__ tE,
-                                           const double *__restrict__ P, int p, int a, int fn, int u0, int v0,
-                                           double &phi1, double &phi2) {
-    using G = Geo<double>;
-    const int sa = a == 0 ? 1 : (a == 1 ? G::RS : G::PS);
-    const int b1 = a == 0 ? 1 : 0, b2 = a == 2 ? 1 : 2;
-    const double es = tE[p] + tE[p + sa];
-    const double *Pa = P + a * 900 + fn * 100;
-    const double *B1 = tB + b1 * G::CS;
-    const double *B2 = tB + b2 * G::CS;
-    const double n1 = B1[p + sa] - B1[p];
-    const double t1 = Pa[v0 * 10 + u0 + 1] - Pa[v0 * 10 + u0 - 1];
-    phi1 = es * (quarter(t1) - n1);
-    const double n2 = B2[p + sa] - B2[p];
-    const double t2 = Pa[(v0 + 1) * 10 + u0] - Pa[(v0 - 1) * 10 + u0];
-    phi2 = es * (quarter(t2) - n2);
-}
-
-// all_faces_512 for float64 with the pair sums (call after pair_sums_512 and a barrier)
-__device__ __forceinline__ void all_faces_512_p(const double *__restrict__ tB, const double *__restrict__ tE,
-                                                const double *__restrict__ P, double *__restrict__ phi) {
-    using G = Geo<double>;
-    const int t = threadIdx.x;
-    int i, j, k;
-    cell_of_thread<double>(t, i, j, k);
-    const int p = G::at(i + 1, j + 1, k + 1);
-    double p1, p2;
-    face_phi_p(tB, tE, P, p - 1, 0, i, j + 1, k + 1, p1, p2);
-    phi[G::xf(i, j, k)] = p1;
-    phi[G::PHI_X + G::xf(i, j, k)] = p2;
-    face_phi_p(tB, tE, P, p - G::RS, 1, j, i + 1, k + 1, p1, p2);
-    phi[phi_base<double>(1, 0) + (k * 9 + j) * 8 + i] = p1;
-    phi[phi_base<double>(1, 1) + (k * 9 + j) * 8 + i] = p2;
-    face_phi_p(tB, tE, P, p - G::PS, 2, k, i + 1, j + 1, p1, p2);
-    phi[phi_base<double>(2, 0) + G::zf(i, j, k)] = p1;
-    phi[phi_base<double>(2, 1) + G::zf(i, j, k)] = p2;
-    if (t < 192) {
-        const int ax = t >> 6, u = t & 7, v = (t >> 3) & 7;
-        if (ax == 0) {  // x = 8 plane: (j, k) = (u, v)
-            face_phi_p(tB, tE, P, G::at(8, u + 1, v + 1), 0, 8, u + 1, v + 1, p1, p2);
-            phi[G::xf(8, u, v)] = p1;
-            phi[G::PHI_X + G::xf(8, u, v)] = p2;
-        } else if (ax == 1) {  // y = 8 plane: (i, k) = (u, v)
-            face_phi_p(tB, tE, P, G::at(u + 1, 8, v + 1), 1, 8, u + 1, v + 1, p1, p2);
-            phi[phi_base<double>(1, 0) + (v * 9 + 8) * 8 + u] = p1;
-            phi[phi_base<double>(1, 1) + (v * 9 + 8) * 8 + u] = p2;
-        } else {  // z = 8 plane: (i, j) = (u, v)
-            face_phi_p(tB, tE, P, G::at(u + 1, v + 1, 8), 2, 8, u + 1, v + 1, p1, p2);
-            phi[phi_base<double>(2, 0) + G::zf(u, v, 8)] = p1;
-            phi[phi_base<double>(2, 1) + G::zf(u, v, 8)] = p2;
-        }
-    }
-}
-
 // sum_a (Phi_a(+) - Phi_a(-)) at cell (i,j,k) for the three components
 template <typename T>
 __device__ __forceinline__ void cell_div(const T *__restrict__ phi, int i, int j, int k, T &dx, T &dy, T &dz) {
@@ -505,9 +427,9 @@ __device__ __forceinline__ T block_max(T v, T *red) {
 }
 
 // ------------------------------------------------------------------ composite operator
-// Computed in TC: float64 for the outer residual and the source of the float64 path, float-float
-// (dfloat, from float64 fields) for those of the mixed path, float32 for the inner residual of
-// mixed precision; refluxed fluxes travel through float64 registers.
+// Computed in TC: float-float (dfloat, from float64 fields) for the outer residual and the source of
+// OHM_MIXED_FF, float32 for the inner residual of mixed precision (float64: k_composite_d below);
+// refluxed fluxes travel through float64 registers.
 template <typename TC>
 struct CompTypes {
     using In = TC;   // element type of X, eta and the ghosts
@@ -548,14 +470,7 @@ __global__ void __launch_bounds__(512, CompTypes<TC>::minb)
     stage_rows<TC, 3, 1, G::RS, G::OFF>(tB, X, snb, slot >= 0 && Gx ? Gx + (size_t)slot * 3 * T3 : nullptr);
     stage_rows<TC, 1, 1, G::RS, G::OFF>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr);
     __syncthreads();
-    if constexpr (std::is_same<TC, double>::value) {
-        double *P = phi + G::PHI;  // pair sums after the flux arrays
-        pair_sums_512(tB, P);
-        __syncthreads();
-        all_faces_512_p(tB, tE, P, phi);
-    } else {
-        all_faces_512(tB, tE, phi);
-    }
+    all_faces_512(tB, tE, phi);
     __syncthreads();
     // flux registers: faces with no same-level neighbour publish F = Phi / (2h) (inv2h = 1 / (2h)
     // and twoh = 2h come from the host: a float64 division here would cost the float32 kernels
@@ -654,7 +569,7 @@ static cudaError_t launch_composite_t(const GridDev &g, const typename CompTypes
                                      double *reg, const int *rsrc_tab, double *partials, double vol, cudaStream_t s,
                                      TC *outS, TC coef2, bool ymx) {
     if (g.nblk == 0) return cudaSuccess;
-    const size_t sm = (4 * Geo<TC>::CS + Geo<TC>::PHI + (std::is_same<TC, double>::value ? PSUM : 0)) * sizeof(TC);
+    const size_t sm = (4 * Geo<TC>::CS + Geo<TC>::PHI) * sizeof(TC);
     // set once per process (thread-safe static initialisation)
     static const bool attr = (cudaFuncSetAttribute(k_composite<TC, TO, true, YT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                               cudaFuncSetAttribute(k_composite<TC, TO, false, YT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
@@ -668,16 +583,6 @@ static cudaError_t launch_composite_t(const GridDev &g, const typename CompTypes
                                                                rsrc_tab, partials, vol, outS, coef2, 0.5 / g.h, 2.0 * g.h,
                                                                ymx);
     return cudaGetLastError();
-}
-
-template <typename TC, typename TO>
-cudaError_t launch_composite(const GridDev &g, const TC *X, const TC *Y, const TC *eta, const TC *Gx, const TC *Geta,
-                             double a, double c, double d, TO *out, TO *out2, double *reg, const int *rsrc_tab,
-                             double *partials, double vol, cudaStream_t s, double *outS, double c2) {
-    const double coef = c / (2.0 * g.h * g.h), coef2 = c2 / (2.0 * g.h * g.h);
-    // outS is set only for TC = float64 (the source of a step)
-    return launch_composite_t<TC, TO>(g, X, Y, eta, Gx, Geta, (TC)a, (TC)coef, (TC)d, out, out2, reg, rsrc_tab,
-                                      partials, vol, s, reinterpret_cast<TC *>(outS), (TC)coef2, a == -1.0 && d == 1.0);
 }
 
 // float64 coefficient as float-float (hi = nearest float32, lo = nearest float32 to the rest)
@@ -704,13 +609,12 @@ cudaError_t launch_composite_df(const GridDev &g, const double *X, const double 
                                                      df_from_host(d), out, out2, reg, rsrc_tab, partials, vol, s,
                                                      nullptr, dfloat(), a == -1.0 && d == 1.0);
 }
-#define INST_COMPOSITE(TC, TO)                                                                                        \
-    template cudaError_t launch_composite<TC, TO>(const GridDev &, const TC *, const TC *, const TC *, const TC *,     \
-                                                  const TC *, double, double, double, TO *, TO *, double *, const int *, \
-                                                  double *, double, cudaStream_t, double *, double);
-INST_COMPOSITE(double, double)
-INST_COMPOSITE(double, float)
-INST_COMPOSITE(float, float)
+cudaError_t launch_composite(const GridDev &g, const float *X, const float *Y, const float *eta, const float *Gx,
+                             const float *Geta, double a, double c, double d, float *out, float *out2, double *reg,
+                             const int *rsrc_tab, double *partials, double vol, cudaStream_t s) {
+    return launch_composite_t<float, float>(g, X, Y, eta, Gx, Geta, (float)a, (float)(c / (2.0 * g.h * g.h)), (float)d, out,
+                                            out2, reg, rsrc_tab, partials, vol, s, nullptr, 0.f, a == -1.0 && d == 1.0);
+}
 
 // ------------------------------------------------------------------ red-black smoothing
 // One colour pass (Eq. 19): colour cells get e + (r - e - lamdt divF(e)) * inv, the other
@@ -871,7 +775,7 @@ template <int NZ, bool ZERO>
 __global__ void __launch_bounds__(32 * NZ) k_smooth_d(GridDev g, const double *__restrict__ e_in, double *__restrict__ e_out,
                                                       const double *__restrict__ r, const double *__restrict__ eta,
                                                       const double *__restrict__ inv, const double *__restrict__ Ge,
-                                                      const double *__restrict__ Geta, double coef, double om1, int colour) {
+                                                      const double *__restrict__ Geta, double coef, double om1, bool relaxed, int colour) {
     using S = SlabD<NZ>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
@@ -957,7 +861,7 @@ __global__ void __launch_bounds__(32 * NZ) k_smooth_d(GridDev g, const double *_
         const double ec = Bc[0];
         if (ZERO) {
             out[c] = ivc * tt;
-        } else if (om1 != 0.0) {
+        } else if (relaxed) {
             out[c] = fma(ivc, tt, om1 * ec);
         } else {  // Gauss-Seidel: the old value has no weight, but a NaN or infinity in it stays visible
             out[c] = ivc * tt;
@@ -977,7 +881,7 @@ static cudaError_t launch_smooth_slab(const GridDev &g, const double *e_in, doub
     static const bool attr = (cudaFuncSetAttribute(k_smooth_d<NZ, ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES), true);
     (void)attr;
     k_smooth_d<NZ, ZERO><<<g.nblk * (8 / NZ), S::NT, ZERO ? 4 * S::CS * sizeof(double) : S::BYTES, s>>>(
-        g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt / (2.0 * g.h * g.h), 1.0 - g.omega, colour);
+        g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt / (2.0 * g.h * g.h), 1.0 - g.omega, g.omega != 1.0, colour);
     return cudaGetLastError();
 }
 
@@ -993,6 +897,262 @@ static cudaError_t launch_smooth_d(const GridDev &g, const double *e_in, double 
     if (g.nblk <= SLAB4_BLOCKS) return launch_smooth_slab<4, ZERO>(g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt, colour, s);
     return launch_smooth_slab<8, ZERO>(g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt, colour, s);
 }
+
+// ---- float64 composite operator: out = a X + c divF(X) + d Y on leaf blocks, the outer residual and
+// the source (launch_composite's rules).  Bound by the float64 pipe like the colour passes, and on slabs
+// of a block as they are: pair sums shared by the faces that read them, each face's G = T/4 - N and eta
+// sum once in shared memory, and the divergence as multiply-adds es G per cell (12) instead of flux
+// products (6.75) and their differences (9): about 51 operations per cell with norms, 59 before, and
+// the sum of squares of Y (of the source) is left out where the caller has it from the step's first
+// residual.  ohm_op_residual at 256^3 (all norms) 2.36 -> 2.19 ms, the operator of a 128^3 float64 FGMRES
+// step with it (and the colour passes without a comparison of doubles) 22.2 -> 21.6 ms.
+// Norms: the 128 threads of a plane pair are
+// folded in a fixed order, plane pairs pairwise, so that a block's sums do not depend on the slab height.
+template <int NZ>
+struct CompD {
+    static constexpr int NT = 64 * NZ, NP = NZ + 2;
+    static constexpr int CS = 100 * NP;
+    static constexpr int PXY = 90 * NP, SUMS = 2 * PXY + 100 * (NZ + 1);
+    static constexpr int FXY = 72 * NZ, FACES = 2 * FXY + 64 * (NZ + 1);
+    static constexpr size_t BYTES = (4 * CS + SUMS + 3 * FACES) * sizeof(double);
+};
+
+template <int NZ, int NF, int NV>
+__device__ __forceinline__ void all_sums_axis(const double *__restrict__ Ba, double *__restrict__ P, int sa, int su, int sv) {
+    constexpr int FULL = 10 * NV - 4;
+    for (int e = threadIdx.x; e < NF * FULL; e += CompD<NZ>::NT) {
+        const int f = e / FULL;
+        int u, v;
+        cross_pos<NV>(e - f * FULL, u, v);
+        const double *p = Ba + f * sa + u * su + v * sv;
+        P[(f * NV + v) * 10 + u] = p[sa] + p[0];
+    }
+}
+
+// index of the face with low tile cell f along ax at block coordinates (u, v) of the two other axes
+// (z slab-local)
+template <int NZ>
+__device__ __forceinline__ int slab_face(int ax, int f, int u, int v) {
+    return ax == 0 ? (v * 8 + u) * 9 + f : (ax == 1 ? CompD<NZ>::FXY + (v * 9 + f) * 8 + u : 2 * CompD<NZ>::FXY + (f * 8 + v) * 8 + u);
+}
+
+template <int NZ, typename TO, bool NORMS>
+__global__ void __launch_bounds__(64 * NZ, 16 / NZ)
+    k_composite_d(GridDev g, const double *__restrict__ X, const double *__restrict__ Y, const double *__restrict__ eta,
+                  const double *__restrict__ Gx, const double *__restrict__ Geta, double a, double coef, double d,
+                  TO *__restrict__ out, TO *__restrict__ out2, double *__restrict__ reg, const int *__restrict__ rsrc_tab,
+                  double *__restrict__ partials, double *__restrict__ outS, double coef2, double inv2h, double twoh,
+                  int mode, bool keep_ss) {
+    using S = CompD<NZ>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
+    double *G1 = P + S::SUMS, *G2 = G1 + S::FACES, *ES = G2 + S::FACES;
+    __shared__ int snb[27];
+    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ)), t = threadIdx.x;
+    if (skip_block(g, b)) return;
+    if (g.covered && g.covered[b]) {
+        if (NORMS && t < 3 && !(keep_ss && t == 1)) partials[(size_t)blockIdx.x * 3 + t] = 0.0;
+        return;
+    }
+    const int slot = g.gslot ? g.gslot[b] : -1;
+    if (t < 32) stage_nbr(snb, g.nbr, b);
+    __syncthreads();
+    stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
+    stage_slab<NZ, 3>(tB, X, snb, slot >= 0 && Gx ? Gx + (size_t)slot * 3 * T3 : nullptr, z0);
+    const int i = t & 7, j = (t >> 3) & 7, k = t >> 6;
+    const size_t cell = (size_t)b * 3 * B3 + ((z0 + k) * 8 + j) * 8 + i;
+    double yv[3] = {0.0, 0.0, 0.0};  // in flight through the face phases
+    if (Y) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) yv[c] = __ldg(Y + cell + c * B3);
+    }
+    __syncthreads();
+    all_sums_axis<NZ, 9, NZ + 2>(tB, P, 1, 10, 100);
+    all_sums_axis<NZ, 9, NZ + 2>(tB + S::CS, P + S::PXY, 10, 1, 100);
+    all_sums_axis<NZ, NZ + 1, 10>(tB + 2 * S::CS, P + 2 * S::PXY, 100, 1, 10);
+    __syncthreads();
+    for (int e = t; e < S::FACES; e += S::NT) {
+        int ax, f, u, v;
+        if (e < S::FXY) {
+            const int row = e / 9;
+            ax = 0;
+            f = e - 9 * row;
+            u = row & 7;
+            v = row >> 3;
+        } else if (e < 2 * S::FXY) {
+            const int h = e - S::FXY, row = h >> 3;
+            ax = 1;
+            u = h & 7;
+            v = row / 9;
+            f = row - 9 * v;
+        } else {
+            const int h = e - 2 * S::FXY;
+            ax = 2;
+            u = h & 7;
+            v = (h >> 3) & 7;
+            f = h >> 6;
+        }
+        const int sa = ax == 0 ? 1 : (ax == 1 ? 10 : 100), su = ax == 0 ? 10 : 1, sv = ax == 2 ? 10 : 100;
+        const int p = f * sa + (u + 1) * su + (v + 1) * sv;
+        const double *Pa = P + ax * S::PXY + (f * (ax == 2 ? 10 : NZ + 2) + v + 1) * 10 + u + 1;
+        const double *B1 = tB + (ax == 0 ? S::CS : 0) + p, *B2 = tB + (ax == 2 ? S::CS : 2 * S::CS) + p;
+        ES[e] = tE[p] + tE[p + sa];
+        G1[e] = fma(0.25, Pa[1] - Pa[-1], B1[0] - B1[sa]);
+        G2[e] = fma(0.25, Pa[10] - Pa[-10], B2[0] - B2[sa]);
+    }
+    __syncthreads();
+    // flux registers: faces with no same-level neighbour publish F = es G / (2h)
+    if (g.freg) {
+        for (int sd = 0; sd < 6; sd++) {
+            const int slotr = g.freg[b * 6 + sd], ax = sd >> 1, hi = sd & 1;
+            if (slotr < 0 || (ax == 2 && (hi ? z0 + NZ < 8 : z0 > 0))) continue;
+            const int nv = ax == 2 ? 8 : NZ;
+            for (int q = t; q < 16 * nv; q += S::NT) {
+                const int comp = q / (8 * nv), u = q & 7, v = (q >> 3) % nv;
+                const int e = slab_face<NZ>(ax, hi ? (ax == 2 ? NZ : 8) : 0, u, v);
+                reg[(size_t)slotr * 128 + comp * 64 + (ax == 2 ? v : z0 + v) * 8 + u] = ES[e] * (comp ? G2 : G1)[e] * inv2h;
+            }
+        }
+    }
+    // refluxing: faces next to a covered block take 2h * (mean of the four fine fluxes)
+    if (g.rsrc) {
+        for (int sd = 0; sd < 6; sd++) {
+            const int src = g.rsrc[b * 6 + sd], ax = sd >> 1, hi = sd & 1;
+            if (src < 0 || (ax == 2 && (hi ? z0 + NZ < 8 : z0 > 0))) continue;
+            const int nv = ax == 2 ? 8 : NZ;
+            for (int q = t; q < 16 * nv; q += S::NT) {
+                const int comp = q / (8 * nv), u = q & 7, vl = (q >> 3) % nv, v = ax == 2 ? vl : z0 + vl;
+                const int fslot = rsrc_tab[src * 4 + (v >> 2) * 2 + (u >> 2)];
+                const double *R = reg + (size_t)fslot * 128 + comp * 64;
+                const int fu = 2 * (u & 3), fv = 2 * (v & 3);
+                const double m = 0.25 * ((R[fv * 8 + fu] + R[fv * 8 + fu + 1]) + (R[(fv + 1) * 8 + fu] + R[(fv + 1) * 8 + fu + 1]));
+                const int e = slab_face<NZ>(ax, hi ? (ax == 2 ? NZ : 8) : 0, u, vl);
+                (comp ? G2 : G1)[e] = m * twoh;
+                if (comp == 0) ES[e] = 1.0;
+            }
+        }
+        __syncthreads();  // refluxed faces before the divergence (g.rsrc is uniform: legal)
+    }
+    double sr = 0.0, ss = 0.0;
+    unsigned long long mx = 0;  // bits of max |out|: ordered like the values; NaNs are left out
+    const int fx = (k * 8 + j) * 9 + i, fy = S::FXY + (k * 9 + j) * 8 + i, fz = 2 * S::FXY + (k * 8 + j) * 8 + i;
+    const double xl = ES[fx], xh = ES[fx + 1], yl = ES[fy], yh = ES[fy + 8], zl = ES[fz], zh = ES[fz + 64];
+    const double dv[3] = {
+        fma(-zl, G1[fz], fma(zh, G1[fz + 64], fma(-yl, G1[fy], yh * G1[fy + 8]))),
+        fma(-zl, G2[fz], fma(zh, G2[fz + 64], fma(-xl, G1[fx], xh * G1[fx + 1]))),
+        fma(-yl, G2[fy], fma(yh, G2[fy + 8], fma(-xl, G2[fx], xh * G2[fx + 1])))};
+    const int p = (k + 1) * 100 + (j + 1) * 10 + i + 1;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const size_t id = cell + c * B3;
+        const double x = tB[c * S::CS + p];
+        double y = yv[c], o;
+        // mode, from the host (a comparison of doubles here would be a float64 operation): 0 a residual (a =
+        // -1, d = 1), 1 the operator or the source (a = 1, no Y), 2 any coefficients
+        if (mode == 0)
+            o = fma(coef, dv[c], y - x);
+        else if (mode == 1)
+            o = fma(coef, dv[c], x);
+        else
+            o = fma(coef, dv[c], Y ? a * x + d * y : a * x);
+        if (outS) {  // o is the source; the residual of X against it is coef2 divF(X)
+            outS[id] = o;
+            y = o;
+            o = coef2 * dv[c];
+        }
+        const TO oo = (TO)o;
+        out[id] = oo;
+        if (out2) out2[id] = oo;
+        if constexpr (NORMS) {
+            sr = fma(o, o, sr);
+            if (!keep_ss) ss = fma(y, y, ss);
+            unsigned long long m;
+            if constexpr (sizeof(TO) == 8) {
+                m = (unsigned long long)__double_as_longlong(o) & 0x7fffffffffffffffull;
+                if (m > 0x7ff0000000000000ull) m = 0;
+            } else {
+                m = __float_as_uint(oo) & 0x7fffffffu;
+                if (m > 0x7f800000u) m = 0;
+            }
+            mx = m > mx ? m : mx;
+        }
+    }
+    if constexpr (NORMS) {
+        // the pair sums' memory is free: [plane pairs][2][64] sums, then the maxima
+        double *rs = P, *rp = rs + 128 * NZ;
+        unsigned long long *rm = reinterpret_cast<unsigned long long *>(rp + NZ);
+        const int pp = t >> 7;
+        rs[pp * 256 + (t & 127)] = sr;
+        rs[pp * 256 + 128 + (t & 127)] = ss;
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long w = __shfl_xor_sync(0xffffffffu, mx, o);
+            mx = w > mx ? w : mx;
+        }
+        if ((t & 31) == 0) rm[t >> 5] = mx;
+        __syncthreads();
+        if ((t & 96) == 0) {  // one warp per plane pair: lanes 0-15 the first sum, 16-31 the second
+            const int l = t & 15;
+            const double *src = rs + pp * 256 + (t & 16) * 8 + l;
+            double v = ((src[0] + src[16]) + (src[32] + src[48])) + ((src[64] + src[80]) + (src[96] + src[112]));
+            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (l == 0) rp[pp * 2 + ((t >> 4) & 1)] = v;
+        }
+        __syncthreads();
+        if (t < 2 && !(keep_ss && t == 1)) {
+            double v = rp[t];
+            if constexpr (NZ >= 4) v = v + rp[2 + t];
+            if constexpr (NZ == 8) v = v + (rp[4 + t] + rp[6 + t]);
+            partials[(size_t)blockIdx.x * 3 + t] = v;
+        } else if (t == 2) {
+            unsigned long long m = 0;
+#pragma unroll
+            for (int w = 0; w < 2 * NZ; w++) m = rm[w] > m ? rm[w] : m;
+            partials[(size_t)blockIdx.x * 3 + 2] = sizeof(TO) == 8 ? __longlong_as_double((long long)m) : (double)__uint_as_float((unsigned)m);
+        }
+    }
+}
+
+template <int NZ, typename TO>
+static cudaError_t launch_composite_slab(const GridDev &g, const double *X, const double *Y, const double *eta, const double *Gx,
+                                         const double *Geta, double a, double coef, double d, TO *out, TO *out2, double *reg,
+                                         const int *rsrc_tab, double *partials, cudaStream_t s, double *outS, double coef2,
+                                         bool keep_ss) {
+    using S = CompD<NZ>;
+    static const bool attr = (cudaFuncSetAttribute(k_composite_d<NZ, TO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES),
+                              cudaFuncSetAttribute(k_composite_d<NZ, TO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES),
+                              true);
+    (void)attr;
+    const int mode = Y && a == -1.0 && d == 1.0 ? 0 : (!Y && a == 1.0 ? 1 : 2);
+    const int grid = g.nblk * (8 / NZ);
+    if (partials)
+        k_composite_d<NZ, TO, true><<<grid, S::NT, S::BYTES, s>>>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
+                                                                  outS, coef2, 0.5 / g.h, 2.0 * g.h, mode, keep_ss);
+    else
+        k_composite_d<NZ, TO, false><<<grid, S::NT, S::BYTES, s>>>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
+                                                                   outS, coef2, 0.5 / g.h, 2.0 * g.h, mode, keep_ss);
+    return cudaGetLastError();
+}
+
+int composite_parts(int nblk) { return nblk <= SLAB2_BLOCKS ? 4 : (nblk <= SLAB4_BLOCKS ? 2 : 1); }
+
+template <typename TO>
+cudaError_t launch_composite(const GridDev &g, const double *X, const double *Y, const double *eta, const double *Gx,
+                             const double *Geta, double a, double c, double d, TO *out, TO *out2, double *reg,
+                             const int *rsrc_tab, double *partials, cudaStream_t s, double *outS, double c2, bool keep_ss) {
+    if (g.nblk == 0) return cudaSuccess;
+    const double coef = c / (2.0 * g.h * g.h), coef2 = c2 / (2.0 * g.h * g.h);
+    switch (composite_parts(g.nblk)) {
+        case 4: return launch_composite_slab<2, TO>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials, s, outS, coef2, keep_ss);
+        case 2: return launch_composite_slab<4, TO>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials, s, outS, coef2, keep_ss);
+        default: return launch_composite_slab<8, TO>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials, s, outS, coef2, keep_ss);
+    }
+}
+template cudaError_t launch_composite<double>(const GridDev &, const double *, const double *, const double *, const double *,
+                                              const double *, double, double, double, double *, double *, double *, const int *,
+                                              double *, cudaStream_t, double *, double, bool);
+template cudaError_t launch_composite<float>(const GridDev &, const double *, const double *, const double *, const double *,
+                                             const double *, double, double, double, float *, float *, double *, const int *,
+                                             double *, cudaStream_t, double *, double, bool);
 
 template <>
 cudaError_t launch_smooth<double>(const GridDev &g, const double *e_in, double *e_out, const double *r, const double *eta,
@@ -2469,49 +2629,96 @@ cudaError_t launch_zero_covered(const GridDev &g, double *x, cudaStream_t s) {
 // thread block folds a fixed contiguous chunk in a fixed order, and the last block to finish
 // (atomic ticket) folds the per-chunk results in chunk order.
 constexpr int NRED = 128;
-__global__ void __launch_bounds__(256) k_norm_reduce(const double *__restrict__ part, int n, double *__restrict__ chunk,
+
+// block i of level l: its entries added pairwise (as the kernel that wrote them adds the ones it
+// holds), times the level's scale
+__device__ __forceinline__ void norm_add(const double *__restrict__ part, const PartRanges &R, int l, int i, double &a, double &b,
+                                         double &m) {
+    const int ns = R.parts[l];
+    const double *p = part + ((size_t)R.base[l] + (size_t)(i - R.off[l]) * ns) * 3;
+    double x = p[0], y = p[1], z = p[2];
+    if (ns == 2) {
+        x = x + p[3];
+        y = y + p[4];
+        z = fmax(z, p[5]);
+    } else if (ns == 4) {
+        x = (x + p[3]) + (p[6] + p[9]);
+        y = (y + p[4]) + (p[7] + p[10]);
+        z = fmax(fmax(z, p[5]), fmax(p[8], p[11]));
+    }
+    a = fma(x, R.vol[l], a);
+    b = fma(y, R.vol[l], b);
+    m = fmax(m, z);
+}
+
+// sums of a and b and maximum of m over the thread block in a fixed order, valid in thread 0
+__device__ __forceinline__ void block_norms(double &a, double &b, double &m, double (*red)[3]) {
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+        m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
+    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        red[w][0] = a;
+        red[w][1] = b;
+        red[w][2] = m;
+    }
+    __syncthreads();
+    if (w == 0) {
+        a = threadIdx.x < nw ? red[threadIdx.x][0] : 0.0;
+        b = threadIdx.x < nw ? red[threadIdx.x][1] : 0.0;
+        m = threadIdx.x < nw ? red[threadIdx.x][2] : 0.0;
+        for (int o = 4; o > 0; o >>= 1) {  // 8 warps
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+            m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_norm_reduce(const double *__restrict__ part, PartRanges R, int n, double *__restrict__ chunk,
                                                      unsigned int *__restrict__ ticket, double *__restrict__ out,
                                                      double *__restrict__ host_out, const int *__restrict__ err) {
-    __shared__ double red[32];
+    __shared__ double red[8][3];
     __shared__ bool last;
     const int per = (n + gridDim.x - 1) / gridDim.x;
     const int lo = blockIdx.x * per, hi = min(n, lo + per);
     double a = 0.0, b = 0.0, m = 0.0;
+    int l = 0;
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        a += part[i * 3 + 0];
-        b += part[i * 3 + 1];
-        m = fmax(m, part[i * 3 + 2]);
+        while (l + 1 < R.nlev && i >= R.off[l + 1]) l++;
+        norm_add(part, R, l, i, a, b, m);
     }
-    double sa = block_sum(a, red);
-    double sb = block_sum(b, red);
-    double sm = block_max(m, red);
-    if (threadIdx.x == 0) {
-        chunk[blockIdx.x * 3 + 0] = sa;
-        chunk[blockIdx.x * 3 + 1] = sb;
-        chunk[blockIdx.x * 3 + 2] = sm;
+    block_norms(a, b, m, red);
+    if (gridDim.x > 1) {
+        if (threadIdx.x == 0) {
+            chunk[blockIdx.x * 3 + 0] = a;
+            chunk[blockIdx.x * 3 + 1] = b;
+            chunk[blockIdx.x * 3 + 2] = m;
+            __threadfence();
+            last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!last) return;
         __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        a = b = m = 0.0;
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+            a += __ldcg(chunk + i * 3 + 0);
+            b += __ldcg(chunk + i * 3 + 1);
+            m = fmax(m, __ldcg(chunk + i * 3 + 2));
+        }
+        block_norms(a, b, m, red);
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    a = b = m = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        a += __ldcg(chunk + i * 3 + 0);
-        b += __ldcg(chunk + i * 3 + 1);
-        m = fmax(m, __ldcg(chunk + i * 3 + 2));
-    }
-    sa = block_sum(a, red);
-    sb = block_sum(b, red);
-    sm = block_max(m, red);
     if (threadIdx.x == 0) {
-        out[0] = sa;
-        out[1] = sb;
-        out[2] = sm;
+        out[0] = a;
+        out[1] = b;
+        out[2] = m;
         if (host_out) {  // pinned host memory mapped into the device: no copy needed to read them
-            host_out[0] = sa;
-            host_out[1] = sb;
-            host_out[2] = sm;
+            host_out[0] = a;
+            host_out[1] = b;
+            host_out[2] = m;
             reinterpret_cast<volatile int *>(host_out + 4)[0] = err ? *err : 0;
         }
         *ticket = 0u;
@@ -2519,40 +2726,34 @@ __global__ void __launch_bounds__(256) k_norm_reduce(const double *__restrict__ 
 }
 
 // scratch: NRED * 3 doubles followed by one unsigned ticket (zero on first use)
-cudaError_t launch_norm_reduce(const double *partials, int nblocks, double *scratch, double *out, cudaStream_t s,
-                               double *host_out, const int *err) {
+cudaError_t launch_norm_reduce(const double *partials, const PartRanges &R, int nblocks, double *scratch, double *out,
+                               cudaStream_t s, double *host_out, const int *err) {
     int grid = nblocks < NRED * 64 ? (nblocks + 63) / 64 : NRED;
-    k_norm_reduce<<<grid, 256, 0, s>>>(partials, nblocks, scratch, (unsigned int *)(scratch + 3 * NRED), out, host_out, err);
+    if (nblocks <= 512) grid = 1;  // one thread block, no second stage
+    k_norm_reduce<<<grid, 256, 0, s>>>(partials, R, nblocks, scratch, (unsigned int *)(scratch + 3 * NRED), out, host_out, err);
     return cudaGetLastError();
 }
 
 // One thread block per instance; its level ranges are folded in level order, each range in a
 // fixed thread-strided order, so the result does not depend on the other instances.
-__global__ void __launch_bounds__(256) k_norm_inst(const double *__restrict__ part, InstRanges R,
-                                                   double *__restrict__ out) {
-    __shared__ double red[32];
+__global__ void __launch_bounds__(256) k_norm_inst(const double *__restrict__ part, PartRanges R, double *__restrict__ out) {
+    __shared__ double red[8][3];
     const int q = blockIdx.x;
     double a = 0.0, b = 0.0, m = 0.0;
     for (int l = 0; l < R.nlev; l++) {
         const int lo = R.off[l] + q * R.n[l], hi = lo + R.n[l];
-        for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-            a += part[i * 3 + 0];
-            b += part[i * 3 + 1];
-            m = fmax(m, part[i * 3 + 2]);
-        }
+        for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) norm_add(part, R, l, i, a, b, m);
     }
-    const double sa = block_sum(a, red);
-    const double sb = block_sum(b, red);
-    const double sm = block_max(m, red);
+    block_norms(a, b, m, red);
     if (threadIdx.x == 0) {
-        out[q * 4 + 0] = sa;
-        out[q * 4 + 1] = sb;
-        out[q * 4 + 2] = sm;
+        out[q * 4 + 0] = a;
+        out[q * 4 + 1] = b;
+        out[q * 4 + 2] = m;
         out[q * 4 + 3] = 0.0;
     }
 }
 
-cudaError_t launch_norm_inst(const double *partials, const InstRanges &R, int ninst, double *out, cudaStream_t s) {
+cudaError_t launch_norm_inst(const double *partials, const PartRanges &R, int ninst, double *out, cudaStream_t s) {
     if (ninst <= 0) return cudaSuccess;
     k_norm_inst<<<ninst, 256, 0, s>>>(partials, R, out);
     return cudaGetLastError();

@@ -35,7 +35,9 @@ constexpr int STATIC_MAX_BLOCKS = 4096;  // 4096 blocks = 2,097,152 cells (e.g. 
 constexpr size_t SO_IJK = 0;                                             // int32 [max][3]
 constexpr size_t SO_INDEX = SO_IJK + STATIC_MAX_BLOCKS * 3 * 4;          // int32 [max] coords -> block
 constexpr size_t SO_NBR = SO_INDEX + STATIC_MAX_BLOCKS * 4;              // int32 [max][27]
-constexpr size_t SO_PART = SO_NBR + (size_t)STATIC_MAX_BLOCKS * 27 * 4;  // double [max][3]
+// norm partials, double [max][3]: composite_parts entries per block, at most STATIC_MAX_BLOCKS in all
+// (4 up to 256 blocks, 2 up to 2048)
+constexpr size_t SO_PART = SO_NBR + (size_t)STATIC_MAX_BLOCKS * 27 * 4;
 constexpr size_t SO_RED = SO_PART + (size_t)STATIC_MAX_BLOCKS * 3 * 8;   // norm reduction scratch
 constexpr size_t SO_NORM = SO_RED + ((NORM_SCRATCH_BYTES + 255) / 256) * 256;  // double [4] + error word
 constexpr size_t SO_TOTAL = SO_NORM + 64;
@@ -138,10 +140,16 @@ extern "C" int ohm_residual_static(const int32_t base_cells[3], double dx, doubl
     g.dims[1] = base_cells[1];
     g.dims[2] = base_cells[2];
     g.nbr = nbr;
-    if (launch_composite<double, double>(g, B_dev, S_dev, eta_dev, nullptr, nullptr, -1.0, -lambda * dt, 1.0, R_dev,
-                                         nullptr, nullptr, nullptr, part, dx * dx * dx, s) != cudaSuccess)
+    if (launch_composite<double>(g, B_dev, S_dev, eta_dev, nullptr, nullptr, -1.0, -lambda * dt, 1.0, R_dev, nullptr,
+                                 nullptr, nullptr, part, s) != cudaSuccess)
         return OHM_ERR_CUDA;
-    if (launch_norm_reduce(part, n, red, dnorm, s) != cudaSuccess) return OHM_ERR_CUDA;
+    PartRanges R;
+    R.nlev = 1;
+    R.off[0] = R.base[0] = 0;
+    R.n[0] = n;
+    R.parts[0] = composite_parts(n);
+    R.vol[0] = dx * dx * dx;
+    if (launch_norm_reduce(part, R, n, red, dnorm, s) != cudaSuccess) return OHM_ERR_CUDA;
     double h[5];
     if (cudaMemcpyAsync(h, dnorm, 5 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess) return OHM_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return OHM_ERR_CUDA;
