@@ -15,12 +15,72 @@
 #include <cfloat>
 #include <cstdint>
 #include <type_traits>
+#include <utility>
 
 #include "ohm_internal.h"
 
 namespace ohm {
 
 __device__ __forceinline__ int tix(int i, int j, int k) { return (k * TS + j) * TS + i; }
+
+// Programmatic dependent launch.  The kernels of a step follow one another on one stream and many of
+// them are short (a 64^3 step: 150 launches of 2-10 us), so each is launched while the one before it
+// drains: its thread blocks come up, read the block tables (which never change) and wait for the
+// grid before them to complete: 64^3 mixed step 1.67 -> 1.53 ms, three-level mixed step 2.50 -> 2.33,
+// 128^3 float-float step 3.56 -> 3.43.  Every kernel launched through launch_pdl calls pdl_trigger() and,
+// before it touches anything that another kernel writes and before any return, pdl_wait().  A load
+// through a const __restrict__ parameter could be moved above the wait, so pdl_wait returns an opaque 0
+// that goes into the block (or element) index from which the addresses of such loads are formed; the
+// other loads follow a __syncthreads() in any case.
+// (The opaque 0 also keeps the index out of the uniform registers, which costs the instruction-bound
+// float32 stencils 2-6% on large grids: they have an instance without any of this, EARLY = false.)
+template <bool EARLY = true>
+__device__ __forceinline__ void pdl_trigger() {
+    if constexpr (EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <bool EARLY = true>
+__device__ __forceinline__ int pdl_wait() {
+    int z = 0;
+    if constexpr (EARLY) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("mov.b32 %0, 0;" : "=r"(z) : : "memory");
+    }
+    return z;
+}
+// Grids of more thread blocks are launched when the one before has drained: their own time hides the
+// launch, and blocks that come up beside a running grid are spread unevenly over the SMs (28 boxes of
+// 64^3: 13.7-13.9 ms per step launched early throughout, 13.4 with this bound).
+constexpr unsigned PDL_GRID = 1024;
+static bool pdl_small(unsigned grid) { return grid <= PDL_GRID; }
+template <typename... E, typename... A>
+static cudaError_t launch_as(bool early, void (*k)(E...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+template <typename... E, typename... A>
+static cudaError_t launch_pdl(void (*k)(E...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+    return launch_as(pdl_small(grid), k, grid, block, smem, s, std::forward<A>(args)...);
+}
+// kernels with an instance for each: the first for small grids, the second for large ones
+template <typename... E, typename... A>
+static cudaError_t launch_pdl2(void (*k)(E...), void (*kl)(E...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+    return launch_as(pdl_small(grid), pdl_small(grid) ? k : kl, grid, block, smem, s, std::forward<A>(args)...);
+}
+// So are the kernels bound by the float64 pipe, whatever their size: the SM with the most thread blocks
+// sets their time (half-refined float64 box: 6.5 ms per step, 7.2 launched early).
+template <typename... E, typename... A>
+static cudaError_t launch_full(void (*k)(E...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+    return launch_as(false, k, grid, block, smem, s, std::forward<A>(args)...);
+}
 
 // batched inner iterations: block b belongs to an instance that is not iterated
 __device__ __forceinline__ bool skip_block(const GridDev &g, int b) {
@@ -443,7 +503,7 @@ struct CompTypes<dfloat> {
     static constexpr int minb = 3;
 };
 
-template <typename TC, typename TO, bool NORMS, typename YT = TC>
+template <typename TC, typename TO, bool NORMS, typename YT = TC, bool EARLY = false>
 __global__ void __launch_bounds__(512, CompTypes<TC>::minb)
     k_composite(GridDev g, const typename CompTypes<TC>::In *__restrict__ X, const YT *__restrict__ Y,
                 const typename CompTypes<TC>::In *__restrict__ eta, const typename CompTypes<TC>::In *__restrict__ Gx,
@@ -458,14 +518,17 @@ __global__ void __launch_bounds__(512, CompTypes<TC>::minb)
     TC *tE = tB + 3 * G::CS;
     TC *phi = tE + G::CS;
     __shared__ int snb[27];
-    const int b = blockIdx.x;
-    if (skip_block(g, b)) return;
+    const int b0 = blockIdx.x;
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(g, b0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b0);
+    const int slot = g.gslot ? g.gslot[b0] : -1;
+    const int b = b0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(g, b)) return;
     if (g.covered && g.covered[b]) {
         if (NORMS && threadIdx.x < 3) partials[b * 3 + threadIdx.x] = 0.0;
         return;
     }
-    const int slot = g.gslot ? g.gslot[b] : -1;
-    stage_nbr(snb, g.nbr, b);
     __syncthreads();
     stage_rows<TC, 3, 1, G::RS, G::OFF>(tB, X, snb, slot >= 0 && Gx ? Gx + (size_t)slot * 3 * T3 : nullptr);
     stage_rows<TC, 1, 1, G::RS, G::OFF>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr);
@@ -571,18 +634,21 @@ static cudaError_t launch_composite_t(const GridDev &g, const typename CompTypes
     if (g.nblk == 0) return cudaSuccess;
     const size_t sm = (4 * Geo<TC>::CS + Geo<TC>::PHI) * sizeof(TC);
     // set once per process (thread-safe static initialisation)
-    static const bool attr = (cudaFuncSetAttribute(k_composite<TC, TO, true, YT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              cudaFuncSetAttribute(k_composite<TC, TO, false, YT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+    constexpr bool E = sizeof(TC) == 4;  // float32: inner residuals and operators of small grids are launched early
+    static const bool attr = (cudaFuncSetAttribute(k_composite<TC, TO, true, YT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_composite<TC, TO, false, YT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_composite<TC, TO, true, YT, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_composite<TC, TO, false, YT, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                               true);
     (void)attr;
+    auto go = [&](auto k, auto kl) {  // early on small grids
+        const bool early = E && pdl_small(g.nblk);
+        return launch_as(early, early ? k : kl, g.nblk, 512, sm, s, g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
+                         vol, outS, coef2, 0.5 / g.h, 2.0 * g.h, ymx);
+    };
     if (partials)  // with norm partials (the block reductions are compiled out otherwise)
-        k_composite<TC, TO, true, YT><<<g.nblk, 512, sm, s>>>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab,
-                                                              partials, vol, outS, coef2, 0.5 / g.h, 2.0 * g.h, ymx);
-    else
-        k_composite<TC, TO, false, YT><<<g.nblk, 512, sm, s>>>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg,
-                                                               rsrc_tab, partials, vol, outS, coef2, 0.5 / g.h, 2.0 * g.h,
-                                                               ymx);
-    return cudaGetLastError();
+        return go(k_composite<TC, TO, true, YT, E>, k_composite<TC, TO, true, YT, false>);
+    return go(k_composite<TC, TO, false, YT, E>, k_composite<TC, TO, false, YT, false>);
 }
 
 // float64 coefficient as float-float (hi = nearest float32, lo = nearest float32 to the rest)
@@ -629,10 +695,12 @@ __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__
     __shared__ __align__(16) T tB[3 * G::CS];
     __shared__ __align__(16) T tE[G::CS];
     __shared__ int snb[27];
-    const int b = blockIdx.x;
+    const int b0 = blockIdx.x;
+    pdl_trigger();
+    stage_nbr(snb, g.nbr, b0);
+    const int slot = g.gslot ? g.gslot[b0] : -1;
+    const int b = b0 + pdl_wait();
     if (skip_block(g, b)) return;
-    const int slot = g.gslot ? g.gslot[b] : -1;
-    stage_nbr(snb, g.nbr, b);
     __syncthreads();
     stage_rows<T, 3, 1, G::RS, G::OFF>(tB, e_in, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr);
     stage_rows<T, 1, 1, G::RS, G::OFF>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr);
@@ -780,10 +848,12 @@ __global__ void __launch_bounds__(32 * NZ) k_smooth_d(GridDev g, const double *_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
     __shared__ int snb[27];
-    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
-    if (skip_block(g, b)) return;
-    const int slot = g.gslot ? g.gslot[b] : -1;
-    if (NZ == 2 || threadIdx.x < 32) stage_nbr(snb, g.nbr, b);
+    const int b0 = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
+    pdl_trigger<false>();
+    if (skip_block(g, b0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b0);
+    const int slot = g.gslot ? g.gslot[b0] : -1;
+    const int b = b0 + pdl_wait<false>();
     __syncthreads();
     stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
     const int t = threadIdx.x, i2 = t & 3, j = (t >> 2) & 7, kl = t >> 5;
@@ -880,7 +950,7 @@ static cudaError_t launch_smooth_slab(const GridDev &g, const double *e_in, doub
     // set once per process (thread-safe static initialisation)
     static const bool attr = (cudaFuncSetAttribute(k_smooth_d<NZ, ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES), true);
     (void)attr;
-    k_smooth_d<NZ, ZERO><<<g.nblk * (8 / NZ), S::NT, ZERO ? 4 * S::CS * sizeof(double) : S::BYTES, s>>>(
+    launch_full(k_smooth_d<NZ, ZERO>, g.nblk * (8 / NZ), S::NT, ZERO ? 4 * S::CS * sizeof(double) : S::BYTES, s, 
         g, e_in, e_out, r, eta, inv, Ge, Geta, lamdt / (2.0 * g.h * g.h), 1.0 - g.omega, g.omega != 1.0, colour);
     return cudaGetLastError();
 }
@@ -902,7 +972,9 @@ static cudaError_t launch_smooth_d(const GridDev &g, const double *e_in, double 
 // the source (launch_composite's rules).  Bound by the float64 pipe like the colour passes, and on slabs
 // of a block as they are: pair sums shared by the faces that read them, each face's G = T/4 - N and eta
 // sum once in shared memory, and the divergence as multiply-adds es G per cell (12) instead of flux
-// products (6.75) and their differences (9): about 51 operations per cell with norms, 59 before, and
+// products (6.75) and their differences (9): about 51 operations per cell with norms, 59 before (FLUX,
+// for a float32 output, keeps the flux products: the residuals of the mixed path, whose inner solves
+// amplify a last-bit change to the size of the step's tolerance, round as they did), and
 // the sum of squares of Y (of the source) is left out where the caller has it from the step's first
 // residual.  ohm_op_residual at 256^3 (all norms) 2.36 -> 2.19 ms, the operator of a 128^3 float64 FGMRES
 // step with it (and the colour passes without a comparison of doubles) 22.2 -> 21.6 ms.
@@ -914,7 +986,8 @@ struct CompD {
     static constexpr int CS = 100 * NP;
     static constexpr int PXY = 90 * NP, SUMS = 2 * PXY + 100 * (NZ + 1);
     static constexpr int FXY = 72 * NZ, FACES = 2 * FXY + 64 * (NZ + 1);
-    static constexpr size_t BYTES = (4 * CS + SUMS + 3 * FACES) * sizeof(double);
+    template <typename TO>
+    static constexpr size_t bytes = (4 * CS + SUMS + (sizeof(TO) == 4 ? 2 : 3) * FACES) * sizeof(double);
 };
 
 template <int NZ, int NF, int NV>
@@ -936,33 +1009,39 @@ __device__ __forceinline__ int slab_face(int ax, int f, int u, int v) {
     return ax == 0 ? (v * 8 + u) * 9 + f : (ax == 1 ? CompD<NZ>::FXY + (v * 9 + f) * 8 + u : 2 * CompD<NZ>::FXY + (f * 8 + v) * 8 + u);
 }
 
-template <int NZ, typename TO, bool NORMS>
+// KIND (a branch on it in the kernel would be turned into selects that execute every case's float64
+// operations): 0 a residual (a = -1, d = 1), 1 the operator or the source (a = 1, no Y), 2 the source and
+// the first residual (outS), 3 any coefficients
+template <int NZ, typename TO, int KIND, bool NORMS>
 __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
     k_composite_d(GridDev g, const double *__restrict__ X, const double *__restrict__ Y, const double *__restrict__ eta,
                   const double *__restrict__ Gx, const double *__restrict__ Geta, double a, double coef, double d,
                   TO *__restrict__ out, TO *__restrict__ out2, double *__restrict__ reg, const int *__restrict__ rsrc_tab,
                   double *__restrict__ partials, double *__restrict__ outS, double coef2, double inv2h, double twoh,
-                  int mode, bool keep_ss) {
+                  bool keep_ss) {
     using S = CompD<NZ>;
+    constexpr bool FLUX = sizeof(TO) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
-    double *G1 = P + S::SUMS, *G2 = G1 + S::FACES, *ES = G2 + S::FACES;
+    double *G1 = P + S::SUMS, *G2 = G1 + S::FACES, *ES = G2 + S::FACES;  // ES: !FLUX only
     __shared__ int snb[27];
-    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ)), t = threadIdx.x;
-    if (skip_block(g, b)) return;
+    const int b0 = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ)), t = threadIdx.x;
+    pdl_trigger<false>();
+    if (skip_block(g, b0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b0);
+    const int slot = g.gslot ? g.gslot[b0] : -1;
+    const int b = b0 + pdl_wait<false>();
     if (g.covered && g.covered[b]) {
         if (NORMS && t < 3 && !(keep_ss && t == 1)) partials[(size_t)blockIdx.x * 3 + t] = 0.0;
         return;
     }
-    const int slot = g.gslot ? g.gslot[b] : -1;
-    if (t < 32) stage_nbr(snb, g.nbr, b);
     __syncthreads();
     stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
     stage_slab<NZ, 3>(tB, X, snb, slot >= 0 && Gx ? Gx + (size_t)slot * 3 * T3 : nullptr, z0);
     const int i = t & 7, j = (t >> 3) & 7, k = t >> 6;
     const size_t cell = (size_t)b * 3 * B3 + ((z0 + k) * 8 + j) * 8 + i;
     double yv[3] = {0.0, 0.0, 0.0};  // in flight through the face phases
-    if (Y) {
+    if (KIND == 0 || (KIND == 3 && Y)) {
 #pragma unroll
         for (int c = 0; c < 3; c++) yv[c] = __ldg(Y + cell + c * B3);
     }
@@ -996,9 +1075,17 @@ __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
         const int p = f * sa + (u + 1) * su + (v + 1) * sv;
         const double *Pa = P + ax * S::PXY + (f * (ax == 2 ? 10 : NZ + 2) + v + 1) * 10 + u + 1;
         const double *B1 = tB + (ax == 0 ? S::CS : 0) + p, *B2 = tB + (ax == 2 ? S::CS : 2 * S::CS) + p;
-        ES[e] = tE[p] + tE[p + sa];
-        G1[e] = fma(0.25, Pa[1] - Pa[-1], B1[0] - B1[sa]);
-        G2[e] = fma(0.25, Pa[10] - Pa[-10], B2[0] - B2[sa]);
+        const double es = tE[p] + tE[p + sa];
+        const double g1 = fma(0.25, Pa[1] - Pa[-1], B1[0] - B1[sa]);
+        const double g2 = fma(0.25, Pa[10] - Pa[-10], B2[0] - B2[sa]);
+        if constexpr (FLUX) {
+            G1[e] = es * g1;
+            G2[e] = es * g2;
+        } else {
+            ES[e] = es;
+            G1[e] = g1;
+            G2[e] = g2;
+        }
     }
     __syncthreads();
     // flux registers: faces with no same-level neighbour publish F = es G / (2h)
@@ -1010,7 +1097,8 @@ __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
             for (int q = t; q < 16 * nv; q += S::NT) {
                 const int comp = q / (8 * nv), u = q & 7, v = (q >> 3) % nv;
                 const int e = slab_face<NZ>(ax, hi ? (ax == 2 ? NZ : 8) : 0, u, v);
-                reg[(size_t)slotr * 128 + comp * 64 + (ax == 2 ? v : z0 + v) * 8 + u] = ES[e] * (comp ? G2 : G1)[e] * inv2h;
+                const double phi = FLUX ? (comp ? G2 : G1)[e] : ES[e] * (comp ? G2 : G1)[e];
+                reg[(size_t)slotr * 128 + comp * 64 + (ax == 2 ? v : z0 + v) * 8 + u] = phi * inv2h;
             }
         }
     }
@@ -1028,7 +1116,7 @@ __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
                 const double m = 0.25 * ((R[fv * 8 + fu] + R[fv * 8 + fu + 1]) + (R[(fv + 1) * 8 + fu] + R[(fv + 1) * 8 + fu + 1]));
                 const int e = slab_face<NZ>(ax, hi ? (ax == 2 ? NZ : 8) : 0, u, vl);
                 (comp ? G2 : G1)[e] = m * twoh;
-                if (comp == 0) ES[e] = 1.0;
+                if (!FLUX && comp == 0) ES[e] = 1.0;
             }
         }
         __syncthreads();  // refluxed faces before the divergence (g.rsrc is uniform: legal)
@@ -1036,26 +1124,30 @@ __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
     double sr = 0.0, ss = 0.0;
     unsigned long long mx = 0;  // bits of max |out|: ordered like the values; NaNs are left out
     const int fx = (k * 8 + j) * 9 + i, fy = S::FXY + (k * 9 + j) * 8 + i, fz = 2 * S::FXY + (k * 8 + j) * 8 + i;
-    const double xl = ES[fx], xh = ES[fx + 1], yl = ES[fy], yh = ES[fy + 8], zl = ES[fz], zh = ES[fz + 64];
-    const double dv[3] = {
-        fma(-zl, G1[fz], fma(zh, G1[fz + 64], fma(-yl, G1[fy], yh * G1[fy + 8]))),
-        fma(-zl, G2[fz], fma(zh, G2[fz + 64], fma(-xl, G1[fx], xh * G1[fx + 1]))),
-        fma(-yl, G2[fy], fma(yh, G2[fy + 8], fma(-xl, G2[fx], xh * G2[fx + 1])))};
+    double dv[3];
+    if constexpr (FLUX) {
+        dv[0] = (G1[fy + 8] - G1[fy]) + (G1[fz + 64] - G1[fz]);
+        dv[1] = (G1[fx + 1] - G1[fx]) + (G2[fz + 64] - G2[fz]);
+        dv[2] = (G2[fx + 1] - G2[fx]) + (G2[fy + 8] - G2[fy]);
+    } else {
+        const double xl = ES[fx], xh = ES[fx + 1], yl = ES[fy], yh = ES[fy + 8], zl = ES[fz], zh = ES[fz + 64];
+        dv[0] = fma(-zl, G1[fz], fma(zh, G1[fz + 64], fma(-yl, G1[fy], yh * G1[fy + 8])));
+        dv[1] = fma(-zl, G2[fz], fma(zh, G2[fz + 64], fma(-xl, G1[fx], xh * G1[fx + 1])));
+        dv[2] = fma(-yl, G2[fy], fma(yh, G2[fy + 8], fma(-xl, G2[fx], xh * G2[fx + 1])));
+    }
     const int p = (k + 1) * 100 + (j + 1) * 10 + i + 1;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         const size_t id = cell + c * B3;
         const double x = tB[c * S::CS + p];
         double y = yv[c], o;
-        // mode, from the host (a comparison of doubles here would be a float64 operation): 0 a residual (a =
-        // -1, d = 1), 1 the operator or the source (a = 1, no Y), 2 any coefficients
-        if (mode == 0)
+        if constexpr (KIND == 0)
             o = fma(coef, dv[c], y - x);
-        else if (mode == 1)
-            o = fma(coef, dv[c], x);
-        else
+        else if constexpr (KIND == 3)
             o = fma(coef, dv[c], Y ? a * x + d * y : a * x);
-        if (outS) {  // o is the source; the residual of X against it is coef2 divF(X)
+        else
+            o = FLUX ? __dadd_rn(x, __dmul_rn(coef, dv[c])) : fma(coef, dv[c], x);
+        if constexpr (KIND == 2) {  // o is the source; the residual of X against it is coef2 divF(X)
             outS[id] = o;
             y = o;
             o = coef2 * dv[c];
@@ -1112,25 +1204,39 @@ __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
     }
 }
 
+template <int NZ, typename TO, int KIND, bool NORMS>
+static cudaError_t launch_composite_kind(const GridDev &g, const double *X, const double *Y, const double *eta, const double *Gx,
+                                         const double *Geta, double a, double coef, double d, TO *out, TO *out2, double *reg,
+                                         const int *rsrc_tab, double *partials, cudaStream_t s, double *outS, double coef2,
+                                         bool keep_ss) {
+    using S = CompD<NZ>;
+    constexpr auto k = k_composite_d<NZ, TO, KIND, NORMS>;
+    constexpr size_t sm = S::template bytes<TO>;
+    static const bool attr = (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
+    (void)attr;
+    return launch_full(k, g.nblk * (8 / NZ), S::NT, sm, s, g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
+                       outS, coef2, 0.5 / g.h, 2.0 * g.h, keep_ss);
+}
+
 template <int NZ, typename TO>
 static cudaError_t launch_composite_slab(const GridDev &g, const double *X, const double *Y, const double *eta, const double *Gx,
                                          const double *Geta, double a, double coef, double d, TO *out, TO *out2, double *reg,
                                          const int *rsrc_tab, double *partials, cudaStream_t s, double *outS, double coef2,
                                          bool keep_ss) {
-    using S = CompD<NZ>;
-    static const bool attr = (cudaFuncSetAttribute(k_composite_d<NZ, TO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES),
-                              cudaFuncSetAttribute(k_composite_d<NZ, TO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES),
-                              true);
-    (void)attr;
-    const int mode = Y && a == -1.0 && d == 1.0 ? 0 : (!Y && a == 1.0 ? 1 : 2);
-    const int grid = g.nblk * (8 / NZ);
-    if (partials)
-        k_composite_d<NZ, TO, true><<<grid, S::NT, S::BYTES, s>>>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
-                                                                  outS, coef2, 0.5 / g.h, 2.0 * g.h, mode, keep_ss);
-    else
-        k_composite_d<NZ, TO, false><<<grid, S::NT, S::BYTES, s>>>(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
-                                                                   outS, coef2, 0.5 / g.h, 2.0 * g.h, mode, keep_ss);
-    return cudaGetLastError();
+    auto go = [&](auto f) { return f(g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials, s, outS, coef2, keep_ss); };
+    const bool resid = Y && a == -1.0 && d == 1.0;
+    if (partials) {  // norms: of residuals only
+        if (resid && !outS) return go(launch_composite_kind<NZ, TO, 0, true>);
+        if (!Y && a == 1.0 && outS) return go(launch_composite_kind<NZ, TO, 2, true>);
+        return cudaErrorInvalidValue;
+    }
+    if (outS) return cudaErrorInvalidValue;
+    if constexpr (sizeof(TO) == 8) {
+        if (resid) return go(launch_composite_kind<NZ, TO, 0, false>);
+        if (!Y && a == 1.0) return go(launch_composite_kind<NZ, TO, 1, false>);
+        return go(launch_composite_kind<NZ, TO, 3, false>);
+    }
+    return cudaErrorInvalidValue;  // float32 output: the outer residuals of the mixed path, always with norms
 }
 
 int composite_parts(int nblk) { return nblk <= SLAB2_BLOCKS ? 4 : (nblk <= SLAB4_BLOCKS ? 2 : 1); }
@@ -1165,7 +1271,7 @@ cudaError_t launch_smooth<float>(const GridDev &g, const float *e_in, float *e_o
                                  const float *inv, const float *Ge, const float *Geta, double lamdt, int colour,
                                  cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    k_smooth<float><<<g.nblk, 256, 0, s>>>(g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
+    launch_pdl(k_smooth<float>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
     return cudaGetLastError();
 }
 cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
@@ -1359,7 +1465,7 @@ __device__ __forceinline__ void rb_update(const T *__restrict__ tB, const T *__r
     rb_update_acc<T>(TileAcc<T, G>{tB, tE, p}, K, rr, out);
 }
 
-template <typename T>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(256) k_smooth_rb(GridDev g, const T *__restrict__ e_in, T *__restrict__ e_out,
                                                    const T *__restrict__ r, const T *__restrict__ eta, RbK<T> K) {
     using G = G12<T>;
@@ -1367,9 +1473,12 @@ __global__ void __launch_bounds__(256) k_smooth_rb(GridDev g, const T *__restric
     T *tB = reinterpret_cast<T *>(smem_raw);  // [3][12 planes][12 rows][RRS]
     T *tE = tB + 3 * G::CS;
     __shared__ int snb[27];
-    const int b = blockIdx.x;
-    if (skip_block(g, b)) return;
-    stage_nbr(snb, g.nbr, b);
+    const int b0 = blockIdx.x;
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(g, b0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b0);
+    const int b = b0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(g, b)) return;
     __syncthreads();
     stage_rows<T, 3, 2, G::RRS, G::OFF>(tB, e_in, snb, nullptr);
     stage_rows<T, 1, 2, G::RRS, G::OFF>(tE, eta, snb, nullptr);
@@ -1447,9 +1556,10 @@ cudaError_t launch_smooth_rb(const GridDev &g, const T *e_in, T *e_out, const T 
     if (g.nblk == 0) return cudaSuccess;
     const size_t sm = 4 * G12<T>::CS * sizeof(T);
     // set once per process (thread-safe static initialisation)
-    static const bool attr = (cudaFuncSetAttribute(k_smooth_rb<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
+    static const bool attr = (cudaFuncSetAttribute(k_smooth_rb<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_smooth_rb<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
     (void)attr;
-    k_smooth_rb<T><<<g.nblk, 256, sm, s>>>(g, e_in, e_out, r, eta, rb_constants<T>(lamdt, g.h, g.omega));
+    launch_pdl2(k_smooth_rb<T, true>, k_smooth_rb<T, false>, g.nblk, 256, sm, s, g, e_in, e_out, r, eta, rb_constants<T>(lamdt, g.h, g.omega));
     return cudaGetLastError();
 }
 template cudaError_t launch_smooth_rb<float>(const GridDev &, const float *, float *, const float *, const float *, double,
@@ -1517,7 +1627,7 @@ __device__ const Ring2 g_ring2 = make_ring2();
 
 // ZERO: the sweep starts from e = 0 (the first pre-smoothing sweep of a level): e_in is not read,
 // only eta is staged, the red pass is pointwise and the black pass reads only red values.
-template <bool ZERO>
+template <bool ZERO, bool EARLY>
 __global__ void __launch_bounds__(512, 3) k_smooth_rb2(GridDev g, const float *__restrict__ e_in, float *__restrict__ e_out,
                                                     const float *__restrict__ r, const float *__restrict__ eta,
                                                     RbK<float> K) {
@@ -1527,13 +1637,16 @@ __global__ void __launch_bounds__(512, 3) k_smooth_rb2(GridDev g, const float *_
     float *tE = tB + 3 * G::CS;
     // neighbourhood of the brick: block columns bx = -1, 0 (A), 1 (B), 2 along x, by dj, dk
     __shared__ int snb[36];
-    const int A = 2 * blockIdx.x;
-    if (skip_block(g, A)) return;
+    const int A0 = 2 * blockIdx.x;
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(g, A0)) return;  // (masked blocks return before they load anything)
     if (threadIdx.x < 36) {
         const int bx = threadIdx.x % 4 - 1, dj = (threadIdx.x / 4) % 3 - 1, dk = threadIdx.x / 12 - 1;
-        const int base = bx <= 1 ? A : A + 1, dx = bx <= 1 ? bx : 1;
+        const int base = bx <= 1 ? A0 : A0 + 1, dx = bx <= 1 ? bx : 1;
         snb[threadIdx.x] = __ldg(g.nbr + base * 27 + (dk + 1) * 9 + (dj + 1) * 3 + (dx + 1));
     }
+    const int A = A0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(g, A)) return;
     __syncthreads();
     // one task per (field component, tile row): the 20 values of the row (halo pair, 8 + 8
     // interior cells, halo pair) as five 16-byte stores; each quarter-warp takes 4 rows of 2
@@ -1622,15 +1735,17 @@ cudaError_t launch_smooth_rb2(const GridDev &g, const float *e_in, float *e_out,
                               double lamdt, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
     const size_t sm = 4 * G20::CS * sizeof(float);
-    static const bool attr = (cudaFuncSetAttribute(k_smooth_rb2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              cudaFuncSetAttribute(k_smooth_rb2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+    static const bool attr = (cudaFuncSetAttribute(k_smooth_rb2<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_smooth_rb2<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_smooth_rb2<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_smooth_rb2<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                               true);
     (void)attr;
     const RbK<float> K = rb_constants<float>(lamdt, g.h, g.omega);
     if (e_in)
-        k_smooth_rb2<false><<<g.nblk / 2, 512, sm, s>>>(g, e_in, e_out, r, eta, K);
+        launch_pdl2(k_smooth_rb2<false, true>, k_smooth_rb2<false, false>, g.nblk / 2, 512, sm, s, g, e_in, e_out, r, eta, K);
     else  // from e = 0
-        k_smooth_rb2<true><<<g.nblk / 2, 512, sm, s>>>(g, nullptr, e_out, r, eta, K);
+        launch_pdl2(k_smooth_rb2<true, true>, k_smooth_rb2<true, false>, g.nblk / 2, 512, sm, s, g, nullptr, e_out, r, eta, K);
     return cudaGetLastError();
 }
 
@@ -1676,23 +1791,26 @@ __device__ __forceinline__ float octet_face(const float *__restrict__ tB, int p,
 // where it is even); it computes those three faces instead of its six, and the octet sum of
 // (Y - X) + kc divF(X) is formed as before.  Equal to the full form in exact arithmetic (the
 // internal fluxes cancel); about 40% fewer operations and 30% fewer tile reads per cell.
-template <bool APPLY, bool RESTRICT, int NV = -1, bool OCT = false>
+template <bool APPLY, bool RESTRICT, int NV = -1, bool OCT = false, bool EARLY = false>
 __global__ void __launch_bounds__(512, NV >= 0 ? 3 : 4)
     k_pair_op(GridDev g, const float *__restrict__ X, const float *__restrict__ Y, const float *__restrict__ eta, float kc,
-              float *__restrict__ out, float *__restrict__ coarse, VecSet V = VecSet(), double wt = 0.0,
-              double *__restrict__ part = nullptr) {
+              float *__restrict__ out, float *__restrict__ coarse, VecSet V, double wt,
+              double *__restrict__ part) {
     using G = G18;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *tB = reinterpret_cast<float *>(smem_raw);  // [3][10 planes][10 rows][RRS]
     float *tE = tB + 3 * G::CS;
     __shared__ int snb[36];
-    const int A = 2 * blockIdx.x;
-    if (skip_block(g, A)) return;
+    const int A0 = 2 * blockIdx.x;
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(g, A0)) return;  // (masked blocks return before they load anything)
     if (threadIdx.x < 36) {
         const int bx = threadIdx.x % 4 - 1, dj = (threadIdx.x / 4) % 3 - 1, dk = threadIdx.x / 12 - 1;
-        const int base = bx <= 1 ? A : A + 1, dx = bx <= 1 ? bx : 1;
+        const int base = bx <= 1 ? A0 : A0 + 1, dx = bx <= 1 ? bx : 1;
         snb[threadIdx.x] = __ldg(g.nbr + base * 27 + (dk + 1) * 9 + (dj + 1) * 3 + (dx + 1));
     }
+    const int A = A0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(g, A)) return;
     __syncthreads();
     // one task per (field component, tile row): 1 + 8 + 8 + 1 values, the interiors as 16-byte words
     if (threadIdx.x < 400) {
@@ -1753,7 +1871,7 @@ __global__ void __launch_bounds__(512, NV >= 0 ? 3 : 4)
             if (!OCT && out) out[id] = o[c];
             if constexpr (NV >= 0) {
 #pragma unroll
-                for (int i = 0; i < NV; i++) dots[i] = fmaf(o[c], __ldg(V.v[i] + id), dots[i]);
+                for (int i = 0; i < NV; i++) dots[i] = fmaf(o[c], V.v[i][id], dots[i]);
                 dots[NV] = fmaf(o[c], o[c], dots[NV]);
             }
         }
@@ -1791,20 +1909,27 @@ cudaError_t launch_pair_op(const GridDev &g, const float *X, const float *Y, con
                            float *out, float *coarse, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
     const size_t sm = 4 * G18::CS * sizeof(float);
-    static const bool attr = (cudaFuncSetAttribute(k_pair_op<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              cudaFuncSetAttribute(k_pair_op<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              cudaFuncSetAttribute(k_pair_op<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              cudaFuncSetAttribute(k_pair_op<false, true, -1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              true);
+    static const bool attr = [=] {
+        auto set = [=](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); };
+        set(k_pair_op<true, false>);
+        set(k_pair_op<false, false>);
+        set(k_pair_op<false, true>);
+        set(k_pair_op<false, true, -1, true>);
+        set(k_pair_op<true, false, -1, false, true>);
+        set(k_pair_op<false, false, -1, false, true>);
+        set(k_pair_op<false, true, -1, false, true>);
+        set(k_pair_op<false, true, -1, true, true>);
+        return true;
+    }();
     (void)attr;
     if (apply)
-        k_pair_op<true, false><<<g.nblk / 2, 512, sm, s>>>(g, X, nullptr, eta, (float)kc, out, nullptr);
+        launch_pdl2(k_pair_op<true, false, -1, false, true>, k_pair_op<true, false>, g.nblk / 2, 512, sm, s, g, X, nullptr, eta, (float)kc, out, nullptr, VecSet(), 0.0, (double *)nullptr);
     else if (coarse && !out)  // only the octet means: outer faces of each octet
-        k_pair_op<false, true, -1, true><<<g.nblk / 2, 512, sm, s>>>(g, X, Y, eta, (float)kc, nullptr, coarse);
+        launch_pdl2(k_pair_op<false, true, -1, true, true>, k_pair_op<false, true, -1, true>, g.nblk / 2, 512, sm, s, g, X, Y, eta, (float)kc, nullptr, coarse, VecSet(), 0.0, (double *)nullptr);
     else if (coarse)
-        k_pair_op<false, true><<<g.nblk / 2, 512, sm, s>>>(g, X, Y, eta, (float)kc, out, coarse);
+        launch_pdl2(k_pair_op<false, true, -1, false, true>, k_pair_op<false, true>, g.nblk / 2, 512, sm, s, g, X, Y, eta, (float)kc, out, coarse, VecSet(), 0.0, (double *)nullptr);
     else
-        k_pair_op<false, false><<<g.nblk / 2, 512, sm, s>>>(g, X, Y, eta, (float)kc, out, nullptr);
+        launch_pdl2(k_pair_op<false, false, -1, false, true>, k_pair_op<false, false>, g.nblk / 2, 512, sm, s, g, X, Y, eta, (float)kc, out, nullptr, VecSet(), 0.0, (double *)nullptr);
     return cudaGetLastError();
 }
 
@@ -1812,6 +1937,8 @@ cudaError_t launch_pair_op(const GridDev &g, const float *X, const float *Y, con
 // One thread per instance: the steps of FGMRES(m) (Saad 1993) that the single-problem solver
 // takes on the host, in the same order and float64 arithmetic, for every instance of a batch.
 __global__ void __launch_bounds__(128) k_fg(FgState f, int op, int j) {
+    pdl_trigger();
+    pdl_wait();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= f.K) return;
     constexpr int KC = KMAX + 1;
@@ -1932,7 +2059,7 @@ __global__ void __launch_bounds__(128) k_fg(FgState f, int op, int j) {
 
 cudaError_t launch_fg(const FgState &f, FgOp op, int j, cudaStream_t s) {
     if (f.K == 0) return cudaSuccess;
-    k_fg<<<(f.K + 127) / 128, 128, 0, s>>>(f, (int)op, j);
+    launch_pdl(k_fg, (f.K + 127) / 128, 128, 0, s, f, (int)op, j);
     return cudaGetLastError();
 }
 
@@ -1987,7 +2114,7 @@ __device__ __forceinline__ bool inst_masked(const GridDev &g, const uint8_t *ima
 }
 
 // ------------------------------------------------------------------ residual + restriction
-template <typename T>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 4 : 1) k_resid_restrict(GridDev g, const T *__restrict__ e, const T *__restrict__ r,
                                                         const T *__restrict__ eta, const T *__restrict__ Ge,
                                                         const T *__restrict__ Geta, T coef, T *__restrict__ t_out,
@@ -1999,10 +2126,13 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 4 : 1) k_resid_restrict(
     T *phi = tE + G::CS;
     T *tt = phi + G::PHI;
     __shared__ int snb[27];
-    const int b = blockIdx.x;
-    if (skip_block(g, b)) return;
-    const int slot = g.gslot ? g.gslot[b] : -1;
-    stage_nbr(snb, g.nbr, b);
+    const int b0 = blockIdx.x;
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(g, b0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b0);
+    const int slot = g.gslot ? g.gslot[b0] : -1;
+    const int b = b0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(g, b)) return;
     __syncthreads();
     stage_rows<T, 3, 1, G::RS, G::OFF>(tB, e, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr);
     stage_rows<T, 1, 1, G::RS, G::OFF>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr);
@@ -2084,10 +2214,12 @@ __global__ void __launch_bounds__(32 * NZ) k_resid_restrict_d(GridDev g, const d
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS, *side = P + S::SUMS;
     __shared__ int snb[27];
-    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
-    if (skip_block(g, b)) return;
-    const int slot = g.gslot ? g.gslot[b] : -1, t = threadIdx.x;
-    if (NZ == 2 || t < 32) stage_nbr(snb, g.nbr, b);
+    const int b0 = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
+    pdl_trigger<false>();
+    if (skip_block(g, b0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b0);
+    const int slot = g.gslot ? g.gslot[b0] : -1, t = threadIdx.x;
+    const int b = b0 + pdl_wait<false>();
     __syncthreads();
     stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
     stage_slab<NZ, 3>(tB, e, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr, z0);
@@ -2161,7 +2293,7 @@ static cudaError_t launch_resid_restrict_slab(const GridDev &g, const double *e,
     using S = OctD<NZ>;
     static const bool attr = (cudaFuncSetAttribute(k_resid_restrict_d<NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::BYTES), true);
     (void)attr;
-    k_resid_restrict_d<NZ><<<g.nblk * (8 / NZ), S::NT, S::BYTES, s>>>(g, e, r, eta, Ge, Geta, kc, coarse, lex, ld);
+    launch_full(k_resid_restrict_d<NZ>, g.nblk * (8 / NZ), S::NT, S::BYTES, s, g, e, r, eta, Ge, Geta, kc, coarse, lex, ld);
     return cudaGetLastError();
 }
 
@@ -2171,7 +2303,9 @@ cudaError_t launch_resid_restrict(const GridDev &g, const T *e, const T *r, cons
     if (g.nblk == 0) return cudaSuccess;
     const size_t sm = (4 * Geo<T>::CS + Geo<T>::PHI + 3 * B3) * sizeof(T);
     // set once per process (thread-safe static initialisation)
-    static const bool attr = (cudaFuncSetAttribute(k_resid_restrict<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
+    constexpr bool E = sizeof(T) == 4;
+    static const bool attr = (cudaFuncSetAttribute(k_resid_restrict<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+                              cudaFuncSetAttribute(k_resid_restrict<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
     (void)attr;
     int3 ld = make_int3(ldims ? ldims[0] : 0, ldims ? ldims[1] : 0, ldims ? ldims[2] : 0);
     if constexpr (std::is_same<T, double>::value) {
@@ -2182,7 +2316,7 @@ cudaError_t launch_resid_restrict(const GridDev &g, const T *e, const T *r, cons
             return launch_resid_restrict_slab<8>(g, e, r, eta, Ge, Geta, kc, coarse, lex, ld, s);
         }
     }
-    k_resid_restrict<T><<<g.nblk, 512, sm, s>>>(g, e, r, eta, Ge, Geta, (T)(lamdt / (2.0 * g.h * g.h)), t_out, coarse,
+    launch_pdl2(k_resid_restrict<T, E>, k_resid_restrict<T, false>, g.nblk, 512, sm, s, g, e, r, eta, Ge, Geta, (T)(lamdt / (2.0 * g.h * g.h)), t_out, coarse,
                                                 lex, ld);
     return cudaGetLastError();
 }
@@ -2234,12 +2368,13 @@ template cudaError_t launch_restrict<float>(const GridDev &, const float *, int,
 // fine += trilinear interpolation (weights 3/4, 1/4 per axis) of the coarser grid, read
 // through a 6^3 window around the block's footprint in its parent (blocked) or with
 // periodic wrap (lexicographic coarse grid).
-template <typename T>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(512) k_prolong_add(GridDev g, GridDev gc, const T *__restrict__ coarse,
                                                      const T *__restrict__ lex, int3 ld, T *__restrict__ fine,
                                                      int *__restrict__ err) {
     __shared__ T win[3 * 216];
-    const int b = blockIdx.x;
+    pdl_trigger<EARLY>();
+    const int b = blockIdx.x + pdl_wait<EARLY>();
     if (skip_block(g, b)) return;
     const int o = lex ? 0 : g.octant[b];
     const int pb = lex ? 0 : g.parent[b];
@@ -2290,7 +2425,8 @@ __global__ void __launch_bounds__(256) k_prolong_add_d(GridDev g, GridDev gc, co
                                                        const double *__restrict__ lex, int3 ld, double *__restrict__ fine,
                                                        int *__restrict__ err) {
     __shared__ double win[3 * 216], wx8[3 * 288], wy8[3 * 384];  // [6][6][6], [6][6][8], [6][8][8] per component
-    const int b = blockIdx.x;
+    pdl_trigger<false>();
+    const int b = blockIdx.x + pdl_wait<false>();
     if (skip_block(g, b)) return;
     const int o = lex ? 0 : g.octant[b];
     const int pb = lex ? 0 : g.parent[b];
@@ -2356,9 +2492,9 @@ cudaError_t launch_prolong_add(const GridDev &g, const GridDev *gc, const T *coa
     int3 ld = make_int3(ldims ? ldims[0] : 0, ldims ? ldims[1] : 0, ldims ? ldims[2] : 0);
     GridDev c = gc ? *gc : GridDev();
     if constexpr (std::is_same<T, double>::value)
-        k_prolong_add_d<<<g.nblk, 256, 0, s>>>(g, c, coarse, lex, ld, fine, err);
+        launch_full(k_prolong_add_d, g.nblk, 256, 0, s, g, c, coarse, lex, ld, fine, err);
     else
-        k_prolong_add<T><<<g.nblk, 512, 0, s>>>(g, c, coarse, lex, ld, fine, err);
+        launch_pdl2(k_prolong_add<T, true>, k_prolong_add<T, false>, g.nblk, 512, 0, s, g, c, coarse, lex, ld, fine, err);
     return cudaGetLastError();
 }
 template cudaError_t launch_prolong_add<double>(const GridDev &, const GridDev *, const double *, const double *,
@@ -2371,14 +2507,17 @@ template cudaError_t launch_prolong_add<float>(const GridDev &, const GridDev *,
 // coarse block and its 1-cell halo once (10^3, as the stencil kernels do) and adds the
 // trilinear interpolant (3/4, 1/4 per axis, the weights of k_prolong_add) to all 4096 cells of
 // the 8 children, one child block per pass of its 512 threads.
-template <typename T>
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(512) k_prolong_add8(GridDev gc, const T *__restrict__ coarse, T *__restrict__ fine) {
     using G = Geo<T>;
     __shared__ __align__(16) T tC[3 * G::CS];
     __shared__ int snb[27];
-    const int c = blockIdx.x;
-    if (skip_block(gc, c)) return;
-    stage_nbr(snb, gc.nbr, c);
+    const int c0 = blockIdx.x;
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(gc, c0)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, gc.nbr, c0);
+    const int c = c0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(gc, c)) return;
     __syncthreads();
     stage_rows<T, 3, 1, G::RS, G::OFF>(tC, coarse, snb, nullptr);
     __syncthreads();
@@ -2407,7 +2546,7 @@ __global__ void __launch_bounds__(512) k_prolong_add8(GridDev gc, const T *__res
 template <typename T>
 cudaError_t launch_prolong_add8(const GridDev &gc, const T *coarse, T *fine, cudaStream_t s) {
     if (gc.nblk == 0) return cudaSuccess;
-    k_prolong_add8<T><<<gc.nblk, 512, 0, s>>>(gc, coarse, fine);
+    launch_pdl2(k_prolong_add8<T, true>, k_prolong_add8<T, false>, gc.nblk, 512, 0, s, gc, coarse, fine);
     return cudaGetLastError();
 }
 template cudaError_t launch_prolong_add8<float>(const GridDev &, const float *, float *, cudaStream_t);
@@ -2431,8 +2570,9 @@ __global__ void __launch_bounds__(512) k_ghost_fill(GridDev g, GridDev gc, const
     __shared__ int nunit;
     const int sl = blockIdx.x;
     const int b = g.slot_block[sl];
+    pdl_trigger();
+    const int o = g.octant[b], pb = g.parent[b] + pdl_wait();
     if (skip_block(g, b)) return;
-    const int pb = g.parent[b], o = g.octant[b];
     const int ox = 4 * (o & 1), oy = 4 * ((o >> 1) & 1), oz = 4 * (o >> 2);
     if (threadIdx.x < 32) {
         // direction l: face 2 axis + high, or edge 6 + 4 (free axis) + signs of the two others (ascending)
@@ -2531,7 +2671,7 @@ template <typename TS_, typename TD>
 cudaError_t launch_ghost_fill(const GridDev &g, const GridDev &gc, const TS_ *coarse, int ncomp, TD *ghost, int *err,
                               cudaStream_t s) {
     if (g.nslot == 0) return cudaSuccess;
-    k_ghost_fill<TS_, TD><<<g.nslot, 512, 0, s>>>(g, gc, coarse, ncomp, ghost + (size_t)g.slot0 * ncomp * T3, err);
+    launch_pdl(k_ghost_fill<TS_, TD>, g.nslot, 512, 0, s, g, gc, coarse, ncomp, ghost + (size_t)g.slot0 * ncomp * T3, err);
     return cudaGetLastError();
 }
 template cudaError_t launch_ghost_fill<double, double>(const GridDev &, const GridDev &, const double *, int, double *,
@@ -2544,7 +2684,8 @@ template cudaError_t launch_ghost_fill<float, float>(const GridDev &, const Grid
 // ------------------------------------------------------------------ sync down, update
 template <typename T>
 __global__ void __launch_bounds__(512) k_sync_down(GridDev gc, T *__restrict__ Bc, const T *__restrict__ Bf) {
-    const int b = blockIdx.x;
+    pdl_trigger();
+    const int b = blockIdx.x + pdl_wait();
     if (!gc.covered[b] || skip_block(gc, b)) return;
     const int t = threadIdx.x, i = t & 7, j = (t >> 3) & 7, k = t >> 6;
     const int oc = (i >> 2) | ((j >> 2) << 1) | ((k >> 2) << 2);
@@ -2564,7 +2705,7 @@ __global__ void __launch_bounds__(512) k_sync_down(GridDev gc, T *__restrict__ B
 template <typename T>
 cudaError_t launch_sync_down(const GridDev &gc, T *Bc, const T *Bf, cudaStream_t s) {
     if (gc.nblk == 0) return cudaSuccess;
-    k_sync_down<T><<<gc.nblk, 512, 0, s>>>(gc, Bc, Bf);
+    launch_pdl(k_sync_down<T>, gc.nblk, 512, 0, s, gc, Bc, Bf);
     return cudaGetLastError();
 }
 template cudaError_t launch_sync_down<double>(const GridDev &, double *, const double *, cudaStream_t);
@@ -2574,7 +2715,8 @@ template cudaError_t launch_sync_down<float>(const GridDev &, float *, const flo
 template <typename T>
 __global__ void __launch_bounds__(512) k_axpy_leaf(GridDev g, T *__restrict__ x, const T *__restrict__ y,
                                                    const uint8_t *__restrict__ imask) {
-    const int b = blockIdx.x;
+    pdl_trigger();
+    const int b = blockIdx.x + pdl_wait();
     if ((g.covered && g.covered[b]) || inst_masked(g, imask, b)) return;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
@@ -2586,7 +2728,7 @@ __global__ void __launch_bounds__(512) k_axpy_leaf(GridDev g, T *__restrict__ x,
 template <typename T>
 cudaError_t launch_axpy_leaf(const GridDev &g, T *x, const T *y, const uint8_t *imask, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    k_axpy_leaf<T><<<g.nblk, 512, 0, s>>>(g, x, y, imask);
+    launch_pdl(k_axpy_leaf<T>, g.nblk, 512, 0, s, g, x, y, imask);
     return cudaGetLastError();
 }
 template cudaError_t launch_axpy_leaf<float>(const GridDev &, float *, const float *, const uint8_t *, cudaStream_t);
@@ -2595,7 +2737,8 @@ template cudaError_t launch_axpy_leaf<double>(const GridDev &, double *, const d
 template <typename T>
 __global__ void __launch_bounds__(512) k_update(GridDev g, double *__restrict__ B, const T *__restrict__ e,
                                                 const uint8_t *__restrict__ imask) {
-    const int b = blockIdx.x;
+    pdl_trigger();
+    const int b = blockIdx.x + pdl_wait();
     if ((g.covered && g.covered[b]) || inst_masked(g, imask, b)) return;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
@@ -2607,7 +2750,7 @@ __global__ void __launch_bounds__(512) k_update(GridDev g, double *__restrict__ 
 template <typename T>
 cudaError_t launch_update(const GridDev &g, double *B, const T *e, const uint8_t *imask, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    k_update<T><<<g.nblk, 512, 0, s>>>(g, B, e, imask);
+    launch_pdl(k_update<T>, g.nblk, 512, 0, s, g, B, e, imask);
     return cudaGetLastError();
 }
 template cudaError_t launch_update<double>(const GridDev &, double *, const double *, const uint8_t *, cudaStream_t);
@@ -2683,8 +2826,10 @@ __global__ void __launch_bounds__(256) k_norm_reduce(const double *__restrict__ 
                                                      double *__restrict__ host_out, const int *__restrict__ err) {
     __shared__ double red[8][3];
     __shared__ bool last;
+    pdl_trigger();
+    const int z = pdl_wait();
     const int per = (n + gridDim.x - 1) / gridDim.x;
-    const int lo = blockIdx.x * per, hi = min(n, lo + per);
+    const int lo = blockIdx.x * per + z, hi = min(n, lo + per);
     double a = 0.0, b = 0.0, m = 0.0;
     int l = 0;
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
@@ -2719,7 +2864,7 @@ __global__ void __launch_bounds__(256) k_norm_reduce(const double *__restrict__ 
             host_out[0] = a;
             host_out[1] = b;
             host_out[2] = m;
-            reinterpret_cast<volatile int *>(host_out + 4)[0] = err ? *err : 0;
+            reinterpret_cast<volatile int *>(host_out + 4)[0] = err ? err[z] : 0;
         }
         *ticket = 0u;
     }
@@ -2730,7 +2875,7 @@ cudaError_t launch_norm_reduce(const double *partials, const PartRanges &R, int 
                                cudaStream_t s, double *host_out, const int *err) {
     int grid = nblocks < NRED * 64 ? (nblocks + 63) / 64 : NRED;
     if (nblocks <= 512) grid = 1;  // one thread block, no second stage
-    k_norm_reduce<<<grid, 256, 0, s>>>(partials, R, nblocks, scratch, (unsigned int *)(scratch + 3 * NRED), out, host_out, err);
+    launch_pdl(k_norm_reduce, grid, 256, 0, s, partials, R, nblocks, scratch, (unsigned int *)(scratch + 3 * NRED), out, host_out, err);
     return cudaGetLastError();
 }
 
@@ -2738,7 +2883,8 @@ cudaError_t launch_norm_reduce(const double *partials, const PartRanges &R, int 
 // fixed thread-strided order, so the result does not depend on the other instances.
 __global__ void __launch_bounds__(256) k_norm_inst(const double *__restrict__ part, PartRanges R, double *__restrict__ out) {
     __shared__ double red[8][3];
-    const int q = blockIdx.x;
+    pdl_trigger();
+    const int q = blockIdx.x + pdl_wait();
     double a = 0.0, b = 0.0, m = 0.0;
     for (int l = 0; l < R.nlev; l++) {
         const int lo = R.off[l] + q * R.n[l], hi = lo + R.n[l];
@@ -2755,7 +2901,7 @@ __global__ void __launch_bounds__(256) k_norm_inst(const double *__restrict__ pa
 
 cudaError_t launch_norm_inst(const double *partials, const PartRanges &R, int ninst, double *out, cudaStream_t s) {
     if (ninst <= 0) return cudaSuccess;
-    k_norm_inst<<<ninst, 256, 0, s>>>(partials, R, out);
+    launch_pdl(k_norm_inst, ninst, 256, 0, s, partials, R, out);
     return cudaGetLastError();
 }
 
@@ -2827,10 +2973,12 @@ __device__ __forceinline__ void warp_block_dots(const float *__restrict__ w, con
 template <int NV>
 __global__ void __launch_bounds__(256) k_mdot(const float *__restrict__ w, VecSet V, const double *__restrict__ wb,
                                               int nblk, double *__restrict__ part, const int *__restrict__ gate) {
-    if (gate && !*gate) return;
+    pdl_trigger();
+    const int z = pdl_wait();
+    if (gate && !gate[z]) return;
     __shared__ double sred[8][NV + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x * 8 + warp;
+    const int b = blockIdx.x * 8 + warp + z;
     double d[NV + 1];
     warp_block_dots<NV>(w, V, b < nblk ? b : 0, lane, b < nblk ? wb[b] : 0.0, d);
     if (lane == 0)
@@ -2846,9 +2994,11 @@ __global__ void __launch_bounds__(256) k_mdot(const float *__restrict__ w, VecSe
 // column sums of part[nrow][ncol] in a fixed order (one thread block per column)
 __global__ void __launch_bounds__(256) k_colsum(const double *__restrict__ part, int nrow, int ncol, double *__restrict__ out,
                                                 const int *__restrict__ gate, double *__restrict__ host_out) {
-    if (gate && !*gate) return;
+    pdl_trigger();
+    const int z = pdl_wait();
+    if (gate && !gate[z]) return;
     __shared__ double red[32];
-    const int c = blockIdx.x;
+    const int c = blockIdx.x + z;
     double a = 0.0;
     for (int b = threadIdx.x; b < nrow; b += blockDim.x) a += part[(size_t)b * ncol + c];
     double s = block_sum(a, red);
@@ -2861,6 +3011,8 @@ __global__ void __launch_bounds__(256) k_colsum(const double *__restrict__ part,
 // dst = (src - sum_i c_i v_i) * scale (dst may equal src; src null reads as 0); float4 over n/4 groups
 template <int NV>
 __global__ void __launch_bounds__(256) k_maxpy(float4 *dst, const float4 *src, VecSet V, float scale, size_t n4) {
+    pdl_trigger();
+    pdl_wait();
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n4; q += (size_t)gridDim.x * blockDim.x) {
         float4 x = src ? src[q] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -2901,10 +3053,10 @@ __global__ void __launch_bounds__(256) k_maxpy(float4 *dst, const float4 *src, V
 cudaError_t launch_mdot(const float *w, const VecSet &V, const double *wb, int nblk, double *part, double *out,
                         cudaStream_t s, const int *gate, double *host_out) {
     const int grid = (nblk + 7) / 8;
-#define OHM_MDOT(N) k_mdot<N><<<grid, 256, 0, s>>>(w, V, wb, nblk, part, gate)
+#define OHM_MDOT(N) launch_pdl(k_mdot<N>, grid, 256, 0, s, w, V, wb, nblk, part, gate)
     OHM_NV_SWITCH(V.k, OHM_MDOT)
 #undef OHM_MDOT
-    k_colsum<<<V.k + 1, 256, 0, s>>>(part, grid, V.k + 1, out, gate, host_out);
+    launch_pdl(k_colsum, V.k + 1, 256, 0, s, part, grid, V.k + 1, out, gate, host_out);
     return cudaGetLastError();
 }
 
@@ -2913,9 +3065,11 @@ cudaError_t launch_mdot(const float *w, const VecSet &V, const double *wb, int n
 template <int NV>
 __global__ void __launch_bounds__(256) k_mdot_d(const double *__restrict__ w, VecSetD V, const double *__restrict__ wb,
                                                 int nblk, double *__restrict__ part) {
+    pdl_trigger();
+    const int z = pdl_wait();
     __shared__ double sred[8][NV + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x * 8 + warp;
+    const int b = blockIdx.x * 8 + warp + z;
     double f[NV + 1];
 #pragma unroll
     for (int i = 0; i <= NV; i++) f[i] = 0.0;
@@ -2949,6 +3103,8 @@ __global__ void __launch_bounds__(256) k_mdot_d(const double *__restrict__ w, Ve
 
 template <int NV>
 __global__ void __launch_bounds__(256) k_maxpy_d(double2 *dst, const double2 *src, VecSetD V, double scale, size_t n2) {
+    pdl_trigger();
+    pdl_wait();
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n2; q += (size_t)gridDim.x * blockDim.x) {
         double2 x = src ? src[q] : make_double2(0.0, 0.0);
 #pragma unroll
@@ -2966,10 +3122,10 @@ __global__ void __launch_bounds__(256) k_maxpy_d(double2 *dst, const double2 *sr
 cudaError_t launch_mdot(const double *w, const VecSetD &V, const double *wb, int nblk, double *part, double *out,
                         cudaStream_t s, double *host_out) {
     const int grid = (nblk + 7) / 8;
-#define OHM_MDOTD(N) k_mdot_d<N><<<grid, 256, 0, s>>>(w, V, wb, nblk, part)
+#define OHM_MDOTD(N) launch_pdl(k_mdot_d<N>, grid, 256, 0, s, w, V, wb, nblk, part)
     OHM_NV_SWITCH(V.k, OHM_MDOTD)
 #undef OHM_MDOTD
-    k_colsum<<<V.k + 1, 256, 0, s>>>(part, grid, V.k + 1, out, nullptr, host_out);
+    launch_pdl(k_colsum, V.k + 1, 256, 0, s, part, grid, V.k + 1, out, nullptr, host_out);
     return cudaGetLastError();
 }
 
@@ -2978,7 +3134,7 @@ cudaError_t launch_maxpy(double *dst, const double *src, const VecSetD &V, doubl
     const int grid = (int)std::min<size_t>((n2 + 255) / 256, 152 * 16);
     double2 *d2 = reinterpret_cast<double2 *>(dst);
     const double2 *s2 = reinterpret_cast<const double2 *>(src);
-#define OHM_MAXPYD(N) k_maxpy_d<N><<<grid, 256, 0, s>>>(d2, s2, V, scale, n2)
+#define OHM_MAXPYD(N) launch_pdl(k_maxpy_d<N>, grid, 256, 0, s, d2, s2, V, scale, n2)
     OHM_NV_SWITCH(V.k, OHM_MAXPYD)
 #undef OHM_MAXPYD
     return cudaGetLastError();
@@ -2987,8 +3143,10 @@ cudaError_t launch_maxpy(double *dst, const double *src, const VecSetD &V, doubl
 // column sums of part[ncol][nrow] (column-major) in a fixed order, one thread block per column
 __global__ void __launch_bounds__(1024) k_colsum_cm(const double *__restrict__ part, int nrow, double *__restrict__ out,
                                                     double *__restrict__ host_out) {
+    pdl_trigger();
+    const int z = pdl_wait();
     __shared__ double red[32];
-    const double *col = part + (size_t)blockIdx.x * nrow;
+    const double *col = part + (size_t)(blockIdx.x + z) * nrow;
     double a = 0.0;
     for (int b = threadIdx.x; b < nrow; b += blockDim.x) a += col[b];
     const double s = block_sum(a, red);
@@ -3012,11 +3170,11 @@ cudaError_t launch_pair_apply_dots(const GridDev &g, const float *X, const float
             (cudaFuncSetAttribute(k_pair_op<true, false, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), \
              true);                                                                                            \
         (void)attr_;                                                                                           \
-        k_pair_op<true, false, N><<<npair, 512, sm, s>>>(g, X, nullptr, eta, (float)kc, w, nullptr, V, wt, part);  \
+        launch_full(k_pair_op<true, false, N>, npair, 512, sm, s, g, X, nullptr, eta, (float)kc, w, nullptr, V, wt, part);  \
     }
     OHM_NV_SWITCH(V.k, OHM_PAIRDOT)
 #undef OHM_PAIRDOT
-    k_colsum_cm<<<V.k + 1, 1024, 0, s>>>(part, npair, out, host_out);
+    launch_pdl(k_colsum_cm, V.k + 1, 1024, 0, s, part, npair, out, host_out);
     return cudaGetLastError();
 }
 
@@ -3025,7 +3183,7 @@ cudaError_t launch_maxpy(float *dst, const float *src, const VecSet &V, float sc
     const int grid = (int)std::min<size_t>((n4 + 255) / 256, 152 * 16);
     float4 *d4 = reinterpret_cast<float4 *>(dst);
     const float4 *s4 = reinterpret_cast<const float4 *>(src);
-#define OHM_MAXPY(N) k_maxpy<N><<<grid, 256, 0, s>>>(d4, s4, V, scale, n4)
+#define OHM_MAXPY(N) launch_pdl(k_maxpy<N>, grid, 256, 0, s, d4, s4, V, scale, n4)
     OHM_NV_SWITCH(V.k, OHM_MAXPY)
 #undef OHM_MAXPY
     return cudaGetLastError();
@@ -3037,9 +3195,11 @@ cudaError_t launch_maxpy(float *dst, const float *src, const VecSet &V, float sc
 template <int NV>
 __global__ void __launch_bounds__(256) k_mdot_blocks(const float *__restrict__ w, VecSet V, const double *__restrict__ wb,
                                                      int nblk, double *__restrict__ part, const int *__restrict__ gate) {
-    if (gate && !*gate) return;
+    pdl_trigger();
+    const int z = pdl_wait();
+    if (gate && !gate[z]) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x * 8 + warp;
+    const int b = blockIdx.x * 8 + warp + z;
     if (b >= nblk) return;
     double d[NV + 1];
     warp_block_dots<NV>(w, V, b, lane, wb[b], d);
@@ -3050,9 +3210,11 @@ __global__ void __launch_bounds__(256) k_mdot_blocks(const float *__restrict__ w
 // out[q][c] = sum of part[b][c] over instance q's blocks of every level, in a fixed order
 __global__ void __launch_bounds__(256) k_colsum_inst(const double *__restrict__ part, InstRanges R, int ncol,
                                                      double *__restrict__ out, const int *__restrict__ gate) {
-    if (gate && !*gate) return;
+    pdl_trigger();
+    const int z = pdl_wait();
+    if (gate && !gate[z]) return;
     __shared__ double red[32];
-    const int q = blockIdx.x;
+    const int q = blockIdx.x + z;
     for (int c = 0; c < ncol; c++) {
         double a = 0.0;
         for (int l = 0; l < R.nlev; l++) {
@@ -3066,10 +3228,10 @@ __global__ void __launch_bounds__(256) k_colsum_inst(const double *__restrict__ 
 
 cudaError_t launch_mdot_inst(const float *w, const VecSet &V, const double *wb, int nblk, const InstRanges &R, int ninst,
                              double *part, double *out, cudaStream_t s, const int *gate) {
-#define OHM_MDOTB(N) k_mdot_blocks<N><<<(nblk + 7) / 8, 256, 0, s>>>(w, V, wb, nblk, part, gate)
+#define OHM_MDOTB(N) launch_pdl(k_mdot_blocks<N>, (nblk + 7) / 8, 256, 0, s, w, V, wb, nblk, part, gate)
     OHM_NV_SWITCH(V.k, OHM_MDOTB)
 #undef OHM_MDOTB
-    k_colsum_inst<<<ninst, 256, 0, s>>>(part, R, V.k + 1, out, gate);
+    launch_pdl(k_colsum_inst, ninst, 256, 0, s, part, R, V.k + 1, out, gate);
     return cudaGetLastError();
 }
 
@@ -3079,8 +3241,10 @@ template <int NV>
 __global__ void __launch_bounds__(256) k_maxpy_inst(float4 *dst, const float4 *src, VecSet V,
                                                     const float *__restrict__ coef, const int *__restrict__ binst,
                                                     size_t n4, const int *__restrict__ gate) {
-    if (gate && !*gate) return;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
+    pdl_trigger();
+    const int z = pdl_wait();
+    if (gate && !gate[z]) return;
+    for (size_t e = z + blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
         const float *cq = coef + (size_t)binst[e / 384] * (KMAX + 1);
         float4 x = src[e];
 #pragma unroll
@@ -3109,7 +3273,7 @@ cudaError_t launch_maxpy_inst(float *dst, const float *src, const VecSet &V, con
     const int grid = (int)std::min<size_t>((n4 + 255) / 256, 152 * 16);
     float4 *d4 = reinterpret_cast<float4 *>(dst);
     const float4 *s4 = reinterpret_cast<const float4 *>(src);
-#define OHM_MAXPYI(N) k_maxpy_inst<N><<<grid, 256, 0, s>>>(d4, s4, V, coef, binst, n4, gate)
+#define OHM_MAXPYI(N) launch_pdl(k_maxpy_inst<N>, grid, 256, 0, s, d4, s4, V, coef, binst, n4, gate)
     OHM_NV_SWITCH(V.k, OHM_MAXPYI)
 #undef OHM_MAXPYI
     return cudaGetLastError();
@@ -3535,7 +3699,7 @@ template <typename T, int CS>
 __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_constant__ TailP<T> P_arg, int nu1, int nu2, int nc) {
     constexpr int NT = TailThreads<T, CS>::N;
     const int inst = blockIdx.x / CS;
-    if (P_arg.imask && !P_arg.imask[inst]) return;  // the whole cluster
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sh = reinterpret_cast<T *>(smem_raw);
     __shared__ TailP<T> P;  // indexed by grid below: kernel parameters are only read at fixed indices
@@ -3553,6 +3717,8 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
             lut[P.lut[s] + (o[2] * P.nby[s] + o[1]) * P.nbx[s] + o[0]] = b;
         }
     }
+    pdl_wait();
+    if (P.imask && !P.imask[inst]) return;  // the whole cluster
     if (any) __syncthreads();
     const int rank = tail_rank<CS>();
     // eta of every grid (divided ones: the planes read here), e = 0 on the first; the own cells' r
@@ -3818,7 +3984,7 @@ template bool tail_fits<double>(const SmallDev<double> &);
 template bool tail_fits<float>(const SmallDev<float> &);
 
 template <typename T, int CS>
-static void tail_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, int ninst, size_t bytes, cudaStream_t s) {
+static void tail_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute at[2], int ninst, size_t bytes, cudaStream_t s) {
     static const bool attr = (cudaFuncSetAttribute(k_tail<T, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_MAX),
                               CS > 8 ? cudaFuncSetAttribute(k_tail<T, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess,
                               true);
@@ -3828,18 +3994,24 @@ static void tail_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, int ni
     cfg.blockDim = dim3(TailThreads<T, CS>::N);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = s;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = CS;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = CS > 1 ? 1 : 0;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CS;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CS > 1 ? 2 : 1;
+    if (sizeof(T) == 8) {  // as launch_full
+        cfg.attrs = at + 1;
+        cfg.numAttrs = CS > 1 ? 1 : 0;
+    }
 }
 
 template <typename T, int CS>
 static cudaError_t launch_tail_cs(const TailP<T> &P, int ninst, size_t bytes, int nu_pre, int nu_post, int n_coarse,
                                   cudaStream_t s) {
     cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute at;
+    cudaLaunchAttribute at[2];
     tail_config<T, CS>(cfg, at, ninst, bytes, s);
     return cudaLaunchKernelEx(&cfg, k_tail<T, CS>, P, nu_pre, nu_post, n_coarse);
 }
@@ -3848,7 +4020,7 @@ static cudaError_t launch_tail_cs(const TailP<T> &P, int ninst, size_t bytes, in
 static bool tail_16() {
     static const bool ok = [] {
         cudaLaunchConfig_t cfg;
-        cudaLaunchAttribute at;
+        cudaLaunchAttribute at[2];
         tail_config<double, 16>(cfg, at, 1, TAIL_SMEM_MAX, nullptr);
         int n = 0;
         const bool fits = cudaOccupancyMaxActiveClusters(&n, k_tail<double, 16>, &cfg) == cudaSuccess && n > 0;
@@ -3894,6 +4066,8 @@ __device__ __forceinline__ bool lex_cell(const SmallDev<T> &sm, int s, size_t ti
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_lex_pass(SmallDev<T> sm, int s, double lamdt, int colour, int to_t) {
+    pdl_trigger();
+    pdl_wait();
     int q, cell;
     if (!lex_cell(sm, s, blockIdx.x * (size_t)blockDim.x + threadIdx.x, q, cell)) return;
     const LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
@@ -3919,6 +4093,8 @@ __global__ void __launch_bounds__(256) k_lex_pass(SmallDev<T> sm, int s, double 
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_lex_resid(SmallDev<T> sm, int s, double lamdt) {
+    pdl_trigger();
+    pdl_wait();
     int q, cell;
     if (!lex_cell(sm, s, blockIdx.x * (size_t)blockDim.x + threadIdx.x, q, cell)) return;
     const LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
@@ -3939,6 +4115,8 @@ __global__ void __launch_bounds__(256) k_lex_resid(SmallDev<T> sm, int s, double
 // r of grid s + 1 = mean of the 8 children of t on grid s; e of grid s + 1 = 0
 template <typename T>
 __global__ void __launch_bounds__(256) k_lex_restrict(SmallDev<T> sm, int s) {
+    pdl_trigger();
+    pdl_wait();
     int q, cell;
     if (!lex_cell(sm, s + 1, blockIdx.x * (size_t)blockDim.x + threadIdx.x, q, cell)) return;
     const LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
@@ -3960,6 +4138,8 @@ __global__ void __launch_bounds__(256) k_lex_restrict(SmallDev<T> sm, int s) {
 // e of grid s += trilinear interpolation of e of grid s + 1
 template <typename T>
 __global__ void __launch_bounds__(256) k_lex_prolong(SmallDev<T> sm, int s) {
+    pdl_trigger();
+    pdl_wait();
     int q, cell;
     if (!lex_cell(sm, s, blockIdx.x * (size_t)blockDim.x + threadIdx.x, q, cell)) return;
     const LexGrid<T> G{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2]};
@@ -3991,22 +4171,22 @@ static unsigned lex_grid(const SmallDev<T> &sm, int s) {
 template <typename T>
 cudaError_t launch_lex_sweeps(const SmallDev<T> &sm, int s, double lamdt, int nsweep, cudaStream_t st) {
     for (int i = 0; i < nsweep; i++) {
-        k_lex_pass<T><<<lex_grid(sm, s), 256, 0, st>>>(sm, s, lamdt, 0, 1);  // e -> t: red
-        k_lex_pass<T><<<lex_grid(sm, s), 256, 0, st>>>(sm, s, lamdt, 1, 0);  // t -> e: black
+        launch_pdl(k_lex_pass<T>, lex_grid(sm, s), 256, 0, st, sm, s, lamdt, 0, 1);  // e -> t: red
+        launch_pdl(k_lex_pass<T>, lex_grid(sm, s), 256, 0, st, sm, s, lamdt, 1, 0);  // t -> e: black
     }
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_lex_resid_restrict(const SmallDev<T> &sm, int s, double lamdt, cudaStream_t st) {
-    k_lex_resid<T><<<lex_grid(sm, s), 256, 0, st>>>(sm, s, lamdt);
-    k_lex_restrict<T><<<lex_grid(sm, s + 1), 256, 0, st>>>(sm, s);
+    launch_pdl(k_lex_resid<T>, lex_grid(sm, s), 256, 0, st, sm, s, lamdt);
+    launch_pdl(k_lex_restrict<T>, lex_grid(sm, s + 1), 256, 0, st, sm, s);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_lex_prolong(const SmallDev<T> &sm, int s, cudaStream_t st) {
-    k_lex_prolong<T><<<lex_grid(sm, s), 256, 0, st>>>(sm, s);
+    launch_pdl(k_lex_prolong<T>, lex_grid(sm, s), 256, 0, st, sm, s);
     return cudaGetLastError();
 }
 template cudaError_t launch_lex_sweeps<double>(const SmallDev<double> &, int, double, int, cudaStream_t);
