@@ -850,31 +850,29 @@ int sweeps(ohm_hier *H, const GridRef &G, int n, double lamdt, bool zero = false
     if (std::is_same<T, float>::value && G.g->nslot == 0 && H->smoother == 0) {
         // float32 grids with every neighbour: one fused red+black launch per sweep, on block
         // pairs where the grid's blocks pair up along x.  The buffers alternate so that the
-        // last sweep writes G.e; a pair sweep from zero reads nothing for e, so neither a
+        // last sweep writes G.e; a sweep from zero reads nothing for e, so neither a
         // memset nor a final copy is needed then.
-        const bool zs = zero && G.g->brick;
-        if (zero && (!zs || n == 0)) CK(cudaMemsetAsync(G.e, 0, bytes, H->s));
-        for (int i = 0; i < n; i++) {
-            const bool to_e = zs ? ((n - 1 - i) % 2 == 0) : (i & 1);
-            const T *src = (const T *)(to_e ? G.e2 : G.e);
-            T *dst = (T *)(to_e ? G.e : G.e2);
-            if (G.g->brick)
-                LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_rb2(gdev(H, *G.g), i == 0 && zs ? nullptr : (const float *)src,
-                                                                    (float *)dst, (const float *)G.r, (const float *)G.eta,
-                                                                    lamdt, H->s));
-            else
-                LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_rb<T>(gdev(H, *G.g), src, dst, (const T *)G.r, (const T *)G.eta, lamdt, H->s));
+        if (zero && n == 0) CK(cudaMemsetAsync(G.e, 0, bytes, H->s));
+        if constexpr (std::is_same<T, float>::value) {
+            for (int i = 0; i < n; i++) {
+                const bool to_e = zero ? ((n - 1 - i) % 2 == 0) : (i & 1);
+                const float *src = i == 0 && zero ? nullptr : (const float *)(to_e ? G.e2 : G.e);
+                float *dst = (float *)(to_e ? G.e : G.e2);
+                const float *r = (const float *)G.r, *eta = (const float *)G.eta;
+                if (G.g->brick)
+                    LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_rb2(gdev(H, *G.g), src, dst, r, eta, lamdt, H->s));
+                else
+                    LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_rb(gdev(H, *G.g), src, dst, r, eta, lamdt, H->s));
+            }
         }
-        if (!zs && (n & 1)) CK(cudaMemcpyAsync(G.e, G.e2, bytes, cudaMemcpyDeviceToDevice, H->s));
+        if (!zero && (n & 1)) CK(cudaMemcpyAsync(G.e, G.e2, bytes, cudaMemcpyDeviceToDevice, H->s));
         return OHM_OK;
     }
     int i0 = 0;
-    if constexpr (std::is_same<T, double>::value) {
-        if (zero && n > 0) {  // the first float64 sweep from zero: one launch, nothing read for e
-            LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_zero(gdev(H, *G.g), (double *)G.e, (const double *)G.r, (const double *)G.eta,
-                                                                 (const double *)G.inv, (const double *)G.Geta, lamdt, H->s));
-            i0 = 1;
-        }
+    if (zero && n > 0) {  // the first sweep from zero: one launch, nothing read for e
+        LAUNCH(H, OHM_K_SMOOTH, G.g->n(), launch_smooth_zero(gdev(H, *G.g), (T *)G.e, (const T *)G.r, (const T *)G.eta, (const T *)G.inv,
+                                                             (const T *)G.Geta, lamdt, H->s));
+        i0 = 1;
     }
     if (zero && i0 == 0) CK(cudaMemsetAsync(G.e, 0, bytes, H->s));
     for (int i = i0; i < n; i++) {

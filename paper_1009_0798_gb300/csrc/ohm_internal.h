@@ -109,20 +109,20 @@ cudaError_t launch_smooth(const GridDev &g, const T *e_in, T *e_out, const T *r,
                           const T *inv, const T *Ge, const T *Geta, double lamdt, int colour,
                           cudaStream_t s);
 
-// The red and the black pass of the first float64 sweep from e = 0 (coarse-fine ghosts of e zero)
-// in one launch
+// The red and the black pass of the first sweep from e = 0 (coarse-fine ghosts of e zero) in one launch
+cudaError_t launch_smooth_zero(const GridDev &g, float *e_out, const float *r, const float *eta, const float *inv,
+                               const float *Geta, double lamdt, cudaStream_t s);
 cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
                                const double *Geta, double lamdt, cudaStream_t s);
 
 // One full red + black sweep in one launch (grids without coarse-fine ghosts), inverse
-// diagonal formed on the fly; e_in != e_out.
-template <typename T>
-cudaError_t launch_smooth_rb(const GridDev &g, const T *e_in, T *e_out, const T *r, const T *eta, double lamdt,
+// diagonal formed on the fly; e_in != e_out.  e_in = nullptr: the sweep starts from e = 0 (nothing is
+// read for e).
+cudaError_t launch_smooth_rb(const GridDev &g, const float *e_in, float *e_out, const float *r, const float *eta, double lamdt,
                              cudaStream_t s);
 
 // The same sweep for pairs of x-adjacent blocks (2q, 2q+1): grids with an even block count whose
-// pairs are x-neighbours and whose blocks all have their 26 neighbours.  e_in = nullptr: the
-// sweep starts from e = 0 (nothing is read for e).
+// pairs are x-neighbours and whose blocks all have their 26 neighbours; e_in as above.
 cudaError_t launch_smooth_rb2(const GridDev &g, const float *e_in, float *e_out, const float *r, const float *eta,
                               double lamdt, cudaStream_t s);
 // float32 operator or residual on block pairs of a brick grid (every block pair x-adjacent, all

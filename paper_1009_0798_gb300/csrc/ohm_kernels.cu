@@ -686,7 +686,10 @@ cudaError_t launch_composite(const GridDev &g, const float *X, const float *Y, c
 // One colour pass (Eq. 19): colour cells get e + (r - e - lamdt divF(e)) * inv, the other
 // colour is copied; e_in and e_out are distinct buffers so every update reads the pre-pass
 // state (Jacobi within a colour).  256 threads, one per colour cell.
-template <typename T>
+// ZERO: both passes of the sweep from e = 0 in one launch (as k_smooth_d's; colour = 1): the tile holds
+// the pointwise red update inv r at red cells and 0 elsewhere, e_in is not read (three-level mixed step
+// 2.33 -> 2.22 ms, with the right-hand sides in flight during the staging 2.14).
+template <typename T, bool ZERO>
 __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__ e_in, T *__restrict__ e_out,
                                                 const T *__restrict__ r, const T *__restrict__ eta,
                                                 const T *__restrict__ inv, const T *__restrict__ Ge,
@@ -701,14 +704,37 @@ __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__
     const int slot = g.gslot ? g.gslot[b0] : -1;
     const int b = b0 + pdl_wait();
     if (skip_block(g, b)) return;
-    __syncthreads();
-    stage_rows<T, 3, 1, G::RS, G::OFF>(tB, e_in, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr);
-    stage_rows<T, 1, 1, G::RS, G::OFF>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr);
-    __syncthreads();
     const int t = threadIdx.x;
     const int k = t >> 5, j = (t >> 2) & 7;
     const int ic = 2 * (t & 3) + ((j + k + colour) & 1);      // colour cell
     const int io = 2 * (t & 3) + ((j + k + colour + 1) & 1);  // other colour
+    const int cc = (k * 8 + j) * 8 + ic, co = (k * 8 + j) * 8 + io;
+    T rr[3], iv[3];  // in flight while the tile is staged
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        rr[c] = r[((size_t)b * 3 + c) * B3 + cc];
+        iv[c] = inv[((size_t)b * 3 + c) * B3 + cc];
+    }
+    __syncthreads();
+    if constexpr (ZERO) {
+        for (int h = t; h < T3 / 2; h += 256) {
+            const int row = h / 5, tj = row % 10, tk = row / 10, pr = 2 * (h % 5), sft = (tj + tk + 1) & 1;
+            const int li = pr + sft - 1, lj = tj - 1, lk = tk - 1;
+            const int di = li < 0 ? -1 : (li > 7 ? 1 : 0), dj = lj < 0 ? -1 : (lj > 7 ? 1 : 0), dk = lk < 0 ? -1 : (lk > 7 ? 1 : 0);
+            const int src = snb[(dk + 1) * 9 + (dj + 1) * 3 + (di + 1)];
+            const size_t id = (size_t)(src >= 0 ? src : 0) * 3 * B3 + ((lk - 8 * dk) * 8 + (lj - 8 * dj)) * 8 + (li - 8 * di);
+            T *d = tB + G::at(pr, tj, tk);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                d[c * G::CS + sft] = src >= 0 ? r[id + c * B3] * inv[id + c * B3] : T(0);
+                d[c * G::CS + 1 - sft] = T(0);
+            }
+        }
+    } else {
+        stage_rows<T, 3, 1, G::RS, G::OFF>(tB, e_in, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr);
+    }
+    stage_rows<T, 1, 1, G::RS, G::OFF>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr);
+    __syncthreads();
     const int p = G::at(ic + 1, j + 1, k + 1);
     T xl1, xl2, xh1, xh2, yl1, yl2, yh1, yh2, zl1, zl2, zh1, zh2;
     face10(tB, tE, p - 1, 0, xl1, xl2);
@@ -721,14 +747,13 @@ __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__
     dv[0] = (yh1 - yl1) + (zh1 - zl1);
     dv[1] = (xh1 - xl1) + (zh2 - zl2);
     dv[2] = (xh2 - xl2) + (yh2 - yl2);
-    const int cc = (k * 8 + j) * 8 + ic, co = (k * 8 + j) * 8 + io;
     const int po = G::at(io + 1, j + 1, k + 1);
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         size_t base = ((size_t)b * 3 + c) * B3;
         T ev = tB[c * G::CS + p];
-        T res = r[base + cc] - ev - coef * dv[c];
-        e_out[base + cc] = ev + res * inv[base + cc];
+        T res = rr[c] - ev - coef * dv[c];
+        e_out[base + cc] = ev + res * iv[c];
         e_out[base + co] = tB[c * G::CS + po];
     }
 }
@@ -1271,8 +1296,12 @@ cudaError_t launch_smooth<float>(const GridDev &g, const float *e_in, float *e_o
                                  const float *inv, const float *Ge, const float *Geta, double lamdt, int colour,
                                  cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    launch_pdl(k_smooth<float>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
-    return cudaGetLastError();
+    return launch_pdl(k_smooth<float, false>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
+}
+cudaError_t launch_smooth_zero(const GridDev &g, float *e_out, const float *r, const float *eta, const float *inv,
+                               const float *Geta, double lamdt, cudaStream_t s) {
+    if (g.nblk == 0) return cudaSuccess;
+    return launch_pdl(k_smooth<float, true>, g.nblk, 256, 0, s, g, nullptr, e_out, r, eta, inv, nullptr, Geta, (float)(lamdt / (2.0 * g.h * g.h)), 1);
 }
 cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
                                const double *Geta, double lamdt, cudaStream_t s) {
@@ -1465,13 +1494,17 @@ __device__ __forceinline__ void rb_update(const T *__restrict__ tB, const T *__r
     rb_update_acc<T>(TileAcc<T, G>{tB, tE, p}, K, rr, out);
 }
 
-template <typename T, bool EARLY>
-__global__ void __launch_bounds__(256) k_smooth_rb(GridDev g, const T *__restrict__ e_in, T *__restrict__ e_out,
-                                                   const T *__restrict__ r, const T *__restrict__ eta, RbK<T> K) {
-    using G = G12<T>;
+// ZERO: the sweep from e = 0, as k_smooth_rb2's: e_in is not read, only eta is staged, the red pass is
+// pointwise and the black pass reads red values only.  The right-hand sides come in before the
+// staging barrier, an x-pair of cells (one red, one black) as one 8-byte word, and the results go out
+// as one (100 boxes of 24^3, V(4,4): 4.26 -> 3.90 ms per step; 120 x 104 x 88, two steps: 5.62 -> 5.20 ms).
+template <bool ZERO, bool EARLY>
+__global__ void __launch_bounds__(256) k_smooth_rb(GridDev g, const float *__restrict__ e_in, float *__restrict__ e_out,
+                                                   const float *__restrict__ r, const float *__restrict__ eta, RbK<float> K) {
+    using G = G12<float>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *tB = reinterpret_cast<T *>(smem_raw);  // [3][12 planes][12 rows][RRS]
-    T *tE = tB + 3 * G::CS;
+    float *tB = reinterpret_cast<float *>(smem_raw);  // [3][12 planes][12 rows][RRS]
+    float *tE = tB + 3 * G::CS;
     __shared__ int snb[27];
     const int b0 = blockIdx.x;
     pdl_trigger<EARLY>();
@@ -1479,93 +1512,99 @@ __global__ void __launch_bounds__(256) k_smooth_rb(GridDev g, const T *__restric
     stage_nbr(snb, g.nbr, b0);
     const int b = b0 + pdl_wait<EARLY>();
     if (EARLY && skip_block(g, b)) return;
-    __syncthreads();
-    stage_rows<T, 3, 2, G::RRS, G::OFF>(tB, e_in, snb, nullptr);
-    stage_rows<T, 1, 2, G::RRS, G::OFF>(tE, eta, snb, nullptr);
+    const int t = threadIdx.x;
+    const int k = t >> 5, j = (t >> 2) & 7, i2 = t & 3;
+    const int ir = 2 * i2 + ((j + k) & 1), ib = 2 * i2 + ((j + k + 1) & 1);
+    const int cpair = (k * 8 + j) * 8 + 2 * i2;
+    const bool red_even = ((j + k) & 1) == 0;
+    float rr0[3], rr1[3] = {0.f, 0.f, 0.f}, rrb[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const float2 v = *reinterpret_cast<const float2 *>(r + ((size_t)b * 3 + c) * B3 + cpair);
+        rr0[c] = red_even ? v.x : v.y;
+        rrb[c] = red_even ? v.y : v.x;
+    }
     __syncthreads();
     // Red cells ((i+j+k) even): the block's 256, one per thread in the same pattern as the black
     // phase (a warp reads 8 rows x 4 cells of one plane: distinct banks), then the 240 of the
     // ring (faces and edges of the 10^3 box, corners excluded), one per thread t < 240:
     // t < 192: face slab f = t/32 (axis f/2 at -1 or 8), 8 lines x 4 red cells;
     // t >= 192: edge e = (t-192)/4 (two axes out), 4 red cells along the third axis.
-    T nv[2][3];
-    int np[2];
-#pragma unroll
-    for (int s4 = 0; s4 < 2; s4++) {
-        np[s4] = -1;
-        const int t = threadIdx.x;
-        int li, lj, lk;
-        if (s4 == 0) {
-            lk = t >> 5;
-            lj = (t >> 2) & 7;
-            li = 2 * (t & 3) + ((lj + lk) & 1);
+    int p1 = -1;
+    if (t < 240) {
+        int c[3];
+        if (t < 192) {
+            const int f = t >> 5, ax = f >> 1, q = t & 31;
+            const int v = q >> 2, u2 = q & 3;
+            const int co = (f & 1) ? 8 : -1, cu = 2 * u2 + ((co + v) & 1);  // out of the block; along a1; v along a2
+            c[0] = ax == 0 ? co : cu;
+            c[1] = ax == 0 ? cu : (ax == 1 ? co : v);
+            c[2] = ax == 2 ? co : v;
         } else {
-            if (t >= 240) continue;
-            int c[3];
-            if (t < 192) {
-                const int f = t >> 5, ax = f >> 1, q = t & 31;
-                const int v = q >> 2, u2 = q & 3;
-                const int a1 = ax == 0 ? 1 : 0, a2 = ax == 2 ? 1 : 2;
-                c[ax] = (f & 1) ? 8 : -1;
-                c[a2] = v;
-                c[a1] = 2 * u2 + ((c[ax] + v) & 1);
-            } else {
-                const int e = (t - 192) >> 2, w2 = (t - 192) & 3;
-                const int pr = e >> 2, sg = e & 3;  // axis pair (0,1), (0,2), (1,2) and its sign combination
-                const int a1 = pr == 2 ? 1 : 0, a2 = pr == 0 ? 1 : 2, af = 3 - a1 - a2;
-                c[a1] = (sg & 1) ? 8 : -1;
-                c[a2] = (sg & 2) ? 8 : -1;
-                c[af] = 2 * w2 + ((c[a1] + c[a2]) & 1);
-            }
-            li = c[0];
-            lj = c[1];
-            lk = c[2];
+            const int e = (t - 192) >> 2, w2 = (t - 192) & 3;
+            const int pr = e >> 2, sg = e & 3;  // axis pair (0,1), (0,2), (1,2) and its sign combination
+            const int c1 = (sg & 1) ? 8 : -1, c2 = (sg & 2) ? 8 : -1, cf = 2 * w2 + ((c1 + c2) & 1);
+            c[0] = pr == 2 ? cf : c1;
+            c[1] = pr == 0 ? c2 : (pr == 1 ? cf : c1);
+            c[2] = pr == 0 ? cf : c2;
         }
-        const int di = li < 0 ? -1 : (li > 7 ? 1 : 0), dj = lj < 0 ? -1 : (lj > 7 ? 1 : 0), dk = lk < 0 ? -1 : (lk > 7 ? 1 : 0);
+        const int di = c[0] < 0 ? -1 : (c[0] > 7 ? 1 : 0), dj = c[1] < 0 ? -1 : (c[1] > 7 ? 1 : 0), dk = c[2] < 0 ? -1 : (c[2] > 7 ? 1 : 0);
         const int src = snb[(dk + 1) * 9 + (dj + 1) * 3 + (di + 1)];
-        const int off = ((lk - 8 * dk) * 8 + (lj - 8 * dj)) * 8 + (li - 8 * di);
-        const T rr[3] = {r[(size_t)src * 3 * B3 + off], r[(size_t)src * 3 * B3 + B3 + off], r[(size_t)src * 3 * B3 + 2 * B3 + off]};
-        np[s4] = G::at(li + 2, lj + 2, lk + 2);
-        rb_update(tB, tE, np[s4], K, rr, nv[s4]);
-    }
-    __syncthreads();
+        const int off = ((c[2] - 8 * dk) * 8 + (c[1] - 8 * dj)) * 8 + (c[0] - 8 * di);
 #pragma unroll
-    for (int s4 = 0; s4 < 2; s4++)
-        if (np[s4] >= 0)
-            for (int c = 0; c < 3; c++) tB[c * G::CS + np[s4]] = nv[s4][c];
+        for (int q = 0; q < 3; q++) rr1[q] = r[((size_t)src * 3 + q) * B3 + off];
+        p1 = G::at(c[0] + 2, c[1] + 2, c[2] + 2);
+    }
+    if constexpr (!ZERO) stage_rows<float, 3, 2, G::RRS, G::OFF>(tB, e_in, snb, nullptr);
+    stage_rows<float, 1, 2, G::RRS, G::OFF>(tE, eta, snb, nullptr);
     __syncthreads();
-    // black cells of the block, one per thread, then the whole block is written out
-    const int t = threadIdx.x;
-    const int k = t >> 5, j = (t >> 2) & 7;
-    const int ib = 2 * (t & 3) + ((j + k + 1) & 1), ir = 2 * (t & 3) + ((j + k) & 1);
-    const int cb = (k * 8 + j) * 8 + ib, cr = (k * 8 + j) * 8 + ir;
-    const T rr[3] = {r[(size_t)b * 3 * B3 + cb], r[(size_t)b * 3 * B3 + B3 + cb], r[(size_t)b * 3 * B3 + 2 * B3 + cb]};
-    T out[3];
-    const int pb = G::at(ib + 2, j + 2, k + 2), pr = G::at(ir + 2, j + 2, k + 2);
-    rb_update(tB, tE, pb, K, rr, out);
+    float nv0[3], nv1[3];
+    const int p0 = G::at(ir + 2, j + 2, k + 2);
+    if constexpr (ZERO) {  // nothing of e is read: no barrier before the red values are stored
+        red_from_zero_acc<float>(TileAcc<float, G>{tB, tE, p0}, K, rr0, nv0);
+        if (p1 >= 0) red_from_zero_acc<float>(TileAcc<float, G>{tB, tE, p1}, K, rr1, nv1);
+    } else {
+        rb_update<float>(tB, tE, p0, K, rr0, nv0);
+        if (p1 >= 0) rb_update<float>(tB, tE, p1, K, rr1, nv1);
+        __syncthreads();
+    }
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-        e_out[((size_t)b * 3 + c) * B3 + cb] = out[c];
-        e_out[((size_t)b * 3 + c) * B3 + cr] = tB[c * G::CS + pr];
+        tB[c * G::CS + p0] = nv0[c];
+        if (p1 >= 0) tB[c * G::CS + p1] = nv1[c];
     }
+    __syncthreads();
+    // black cells of the block, one per thread, then the whole block is written out
+    float out[3];
+    const int pb = G::at(ib + 2, j + 2, k + 2);
+    if constexpr (ZERO)
+        black_after_zero_acc<float>(TileAcc<float, G>{tB, tE, pb}, K, rrb, out);
+    else
+        rb_update<float>(tB, tE, pb, K, rrb, out);
+#pragma unroll
+    for (int c = 0; c < 3; c++)
+        *reinterpret_cast<float2 *>(e_out + ((size_t)b * 3 + c) * B3 + cpair) =
+            red_even ? make_float2(nv0[c], out[c]) : make_float2(out[c], nv0[c]);
 }
 
-template <typename T>
-cudaError_t launch_smooth_rb(const GridDev &g, const T *e_in, T *e_out, const T *r, const T *eta, double lamdt,
+cudaError_t launch_smooth_rb(const GridDev &g, const float *e_in, float *e_out, const float *r, const float *eta, double lamdt,
                              cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    const size_t sm = 4 * G12<T>::CS * sizeof(T);
+    const size_t sm = 4 * G12<float>::CS * sizeof(float);
     // set once per process (thread-safe static initialisation)
-    static const bool attr = (cudaFuncSetAttribute(k_smooth_rb<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                              cudaFuncSetAttribute(k_smooth_rb<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
+    static const bool attr = [=] {
+        auto set = [=](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); };
+        set(k_smooth_rb<false, true>);
+        set(k_smooth_rb<false, false>);
+        set(k_smooth_rb<true, true>);
+        set(k_smooth_rb<true, false>);
+        return true;
+    }();
     (void)attr;
-    launch_pdl2(k_smooth_rb<T, true>, k_smooth_rb<T, false>, g.nblk, 256, sm, s, g, e_in, e_out, r, eta, rb_constants<T>(lamdt, g.h, g.omega));
-    return cudaGetLastError();
+    const RbK<float> K = rb_constants<float>(lamdt, g.h, g.omega);
+    if (e_in) return launch_pdl2(k_smooth_rb<false, true>, k_smooth_rb<false, false>, g.nblk, 256, sm, s, g, e_in, e_out, r, eta, K);
+    return launch_pdl2(k_smooth_rb<true, true>, k_smooth_rb<true, false>, g.nblk, 256, sm, s, g, nullptr, e_out, r, eta, K);  // from e = 0
 }
-template cudaError_t launch_smooth_rb<float>(const GridDev &, const float *, float *, const float *, const float *, double,
-                                             cudaStream_t);
-template cudaError_t launch_smooth_rb<double>(const GridDev &, const double *, double *, const double *, const double *,
-                                              double, cudaStream_t);
 
 // ------------------------------------------------------------------ fused sweep on brick pairs
 // The fused sweep above for two x-adjacent blocks A = 2q and B = 2q + 1 per thread block (512
