@@ -3468,6 +3468,12 @@ template <typename T>
 struct TailP {  // no default member initialisers: the kernel keeps a __shared__ copy
     int n;
     T om1;                        // 1 - omega
+    // The axes of the arrays in shared memory: axis k is the grids' axis axes[k], component k the field's
+    // component axes[k] (the operator is the same under a relabelling of both), so that the planes that
+    // the cluster divides lie along the longest extent.  float32 keeps the order (its sums would round
+    // otherwise, and the mixed path's results move by up to the step's tolerance).
+    int axes[3];
+    int gx[MAX_SMALL], gy[MAX_SMALL];  // cells of the grid along its own x and y
     LexDims d[MAX_SMALL];
     int oe[MAX_SMALL], oE[MAX_SMALL], orr[MAX_SMALL], oi[MAX_SMALL];  // element offsets in shared memory: e[3n],
                                   // eta[n], r (first grid, divided: the own cells by colour, else [3n]) and, in
@@ -3533,16 +3539,29 @@ __device__ __forceinline__ void tail_store_cell(const TailP<T> &P, T *sh, int s,
     }
 }
 
-// index of cell (x, y, z) of grid s in global memory: component stride cst for ncomp components
+// index in global memory of cell (u, v, w) of grid s (axes of shared memory): component stride cst for
+// ncomp components
 template <typename T>
-__device__ __forceinline__ size_t tail_gidx(const TailP<T> &P, const int *lut, int s, int x, int y, int z, int ncomp, int &cst) {
+__device__ __forceinline__ size_t tail_gidx(const TailP<T> &P, const int *lut, int s, int u, int v, int w, int ncomp, int &cst) {
+    int x = u, y = v, z = w;
+    if constexpr (sizeof(T) == 8) {
+        x = P.axes[0] == 0 ? u : (P.axes[1] == 0 ? v : w);
+        y = P.axes[0] == 1 ? u : (P.axes[1] == 1 ? v : w);
+        z = P.axes[0] == 2 ? u : (P.axes[1] == 2 ? v : w);
+    }
     if (P.blocked[s]) {
         const int b = lut[P.lut[s] + ((z >> 3) * P.nby[s] + (y >> 3)) * P.nbx[s] + (x >> 3)];
         cst = B3;
         return (size_t)b * ncomp * B3 + ((z & 7) * 8 + (y & 7)) * 8 + (x & 7);
     }
     cst = P.d[s].n();
-    return P.d[s].id(x, y, z);
+    if constexpr (sizeof(T) == 4) return P.d[s].id(x, y, z);
+    return ((size_t)z * P.gy[s] + y) * P.gx[s] + x;
+}
+// the field's component of component c in shared memory
+template <typename T>
+__device__ __forceinline__ int tail_comp(const TailP<T> &P, int c) {
+    return sizeof(T) == 8 ? P.axes[c] : c;
 }
 
 // the planes of grid s that this block owns
@@ -3613,10 +3632,10 @@ __device__ __forceinline__ void tail_colour(const TailP<T> &P, T *sh, const int 
         size_t id = 0;
         int cst = 0;
         if (!P.own) id = inst3 * n + tail_gidx(P, lut, s, x, y, z, 3, cst);
-        auto rhs = [&](int c) { return s > 0 || (P.own && !dv) ? sh[P.orr[s] + c * n + q] : (P.own ? sh[P.orr[0] + o + c * own] : P.r0[id + (size_t)c * cst]); };
+        auto rhs = [&](int c) { return s > 0 || (P.own && !dv) ? sh[P.orr[s] + c * n + q] : (P.own ? sh[P.orr[0] + o + c * own] : P.r0[id + (size_t)tail_comp(P, c) * cst]); };
         const LexAcc<T> acc = D.acc(e, E, x, y, z);
         if constexpr (sizeof(T) == 8) {
-            const double rv = rhs(cc), iv = P.own ? sh[P.oi[s] + o + cc * own] : P.inv[s][id + (size_t)cc * cst];
+            const double rv = rhs(cc), iv = P.own ? sh[P.oi[s] + o + cc * own] : P.inv[s][id + (size_t)tail_comp(P, cc) * cst];
             const double coef = -P.K[s].ncoef;
             t[cc * own + il] = cc == 0 ? tail_update_d<0>(acc, coef, P.om1, rv, iv, zero)
                                        : (cc == 1 ? tail_update_d<1>(acc, coef, P.om1, rv, iv, zero)
@@ -3683,7 +3702,7 @@ __device__ __forceinline__ void tail_coarsest(const TailP<double> &P, double *sh
             };
             const double es_lo = E[q] + E[at(-1, 0)], es_hi = E[q] + E[at(1, 0)];
             int cst;
-            const size_t id = inst3 * n + tail_gidx(P, lut, s, x, y, z, 3, cst) + (size_t)c * cst;
+            const size_t id = inst3 * n + tail_gidx(P, lut, s, x, y, z, 3, cst) + (size_t)tail_comp(P, c) * cst;
             const double rv = s == 0 ? P.r0[id] : sh[P.orr[s] + c * n + q];
             const double inv = P.inv[s][id];
             const double k_lo = -P.K[s].ncoef * es_lo * inv, k_hi = -P.K[s].ncoef * es_hi * inv;
@@ -3770,7 +3789,8 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
         tail_planes<CS>(P, s, rank, z0, z1);
         const bool part = CS > 1 && P.divided[s] && z1 - z0 + 4 < D.nz;
         const int za = part ? z0 - 2 : 0, np = z0 < z1 ? (part ? z1 - z0 + 4 : D.nz) : 0;
-        if (!part && !P.blocked[s]) {
+        const bool same = sizeof(T) == 4 || (P.axes[0] == 0 && P.axes[1] == 1);  // the order of the grid's axes
+        if (!part && !P.blocked[s] && same) {
             for (int q = threadIdx.x; q < np * pl; q += NT) sh[P.oE[s] + q] = eta[q];
         } else
 #pragma unroll 4
@@ -3785,7 +3805,7 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
             for (int q = threadIdx.x; q < 3 * n; q += NT) sh[P.oe[0] + q] = T(0);
         if (!P.own || (s > 0 && sizeof(T) == 4)) continue;
         const bool full = s == 0 && !P.divided[0];  // r as it lies
-        if (full && !P.blocked[0]) {
+        if (full && !P.blocked[0] && same) {
             const T *r0 = P.r0 + (size_t)inst * 3 * n;
             for (int q = threadIdx.x; q < 3 * n; q += NT) sh[P.orr[0] + q] = r0[q];
             if (sizeof(T) == 4) continue;
@@ -3801,9 +3821,9 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
                 const int o = 3 * colour * own + i;
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    if (s == 0 && !full) sh[P.orr[0] + o + c * own] = P.r0[id + (size_t)c * cst];
-                    if (full && P.blocked[0]) sh[P.orr[0] + c * n + D.id(x, y, z)] = P.r0[id + (size_t)c * cst];
-                    if (sizeof(T) == 8) sh[P.oi[s] + o + c * own] = P.inv[s][id + (size_t)c * cst];
+                    if (s == 0 && !full) sh[P.orr[0] + o + c * own] = P.r0[id + (size_t)tail_comp(P, c) * cst];
+                    if (full && (P.blocked[0] || !same)) sh[P.orr[0] + c * n + D.id(x, y, z)] = P.r0[id + (size_t)tail_comp(P, c) * cst];
+                    if (sizeof(T) == 8) sh[P.oi[s] + o + c * own] = P.inv[s][id + (size_t)tail_comp(P, c) * cst];
                 }
             }
     }
@@ -3864,7 +3884,7 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
             if (s == 0) id = inst3 * n + tail_gidx(P, lut, 0, x, y, z, 3, cst);
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                const T rv = s == 0 && (dv || !P.own) ? P.r0[id + (size_t)c * cst] : sh[P.orr[s] + c * n + q];
+                const T rv = s == 0 && (dv || !P.own) ? P.r0[id + (size_t)tail_comp(P, c) * cst] : sh[P.orr[s] + c * n + q];
                 T v = v_mad(P.K[s].ncoef, o[c], v_sub(rv, e[c * n + q]));
                 if constexpr (sizeof(T) == 8) {
                     v = v_add(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -3943,7 +3963,7 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
         D.cell(q, x, y, z);
         const size_t id = inst3 * n + tail_gidx(P, lut, 0, x, y, z, 3, cst);
 #pragma unroll
-        for (int c = 0; c < 3; c++) P.e0[id + (size_t)c * cst] = sh[P.oe[0] + c * n + q];
+        for (int c = 0; c < 3; c++) P.e0[id + (size_t)tail_comp(P, c) * cst] = sh[P.oe[0] + c * n + q];
     }
 }
 
@@ -3970,6 +3990,14 @@ static bool tail_plan(const SmallDev<T> &sm, double lamdt, int cs, bool own, Tai
     P.own = own;
     P.om1 = (T)(1.0 - sm.omega);
     P.imask = sm.imask;
+    // the longest extent last (ties and float32: the grids' own order)
+    int last = 2;
+    if (sizeof(T) == 8 && sm.n > 0)
+        for (int ax = 1; ax >= 0; ax--)
+            if (sm.dims[0][ax] > sm.dims[0][last]) last = ax;
+    P.axes[2] = last;
+    P.axes[0] = last == 0 ? 1 : 0;
+    P.axes[1] = last == 2 ? 1 : 2;
     P.r0 = sm.r[0];
     P.e0 = sm.e[0];
     size_t off = 0, tmax = 0;
@@ -3980,8 +4008,11 @@ static bool tail_plan(const SmallDev<T> &sm, double lamdt, int cs, bool own, Tai
         return (int)o;
     };
     for (int s = 0; s < sm.n; s++) {
-        const int lx = ilog2_exact(sm.dims[s][0]), ly = ilog2_exact(sm.dims[s][1]), lz = ilog2_exact(sm.dims[s][2]);
-        const LexDims d{sm.dims[s][0], sm.dims[s][1], sm.dims[s][2], lx, ly, lx >= 0 && ly >= 0 && lz >= 0};
+        const int e0 = sm.dims[s][P.axes[0]], e1 = sm.dims[s][P.axes[1]], e2 = sm.dims[s][P.axes[2]];
+        const int lx = ilog2_exact(e0), ly = ilog2_exact(e1), lz = ilog2_exact(e2);
+        const LexDims d{e0, e1, e2, lx, ly, lx >= 0 && ly >= 0 && lz >= 0};
+        P.gx[s] = sm.dims[s][0];
+        P.gy[s] = sm.dims[s][1];
         const size_t n = (size_t)d.nx * d.ny * d.nz;
         if (n > 16384) return false;
         P.d[s] = d;
@@ -4001,8 +4032,8 @@ static bool tail_plan(const SmallDev<T> &sm, double lamdt, int cs, bool own, Tai
         P.blocked[s] = sm.origin[s] != nullptr;
         P.origin[s] = sm.origin[s];
         P.lut[s] = lut;
-        P.nbx[s] = d.nx / BS;
-        P.nby[s] = d.ny / BS;
+        P.nbx[s] = sm.dims[s][0] / BS;
+        P.nby[s] = sm.dims[s][1] / BS;
         P.nblk[s] = P.blocked[s] ? (int)(n / B3) : 0;
         lut += P.nblk[s];
     }

@@ -341,7 +341,7 @@ def test_fgmres_batch_takes_fewer_cycles(ohm):
 
 
 @pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("base", [(32, 32, 32), (48, 16, 32), (16, 24, 40)])
+@pytest.mark.parametrize("base", [(32, 32, 32), (48, 16, 32), (16, 24, 40), (16, 48, 32)])
 def test_coarse_solver_clusters_give_same_bits_and_match_oracle(ohm, orc, base, precision):
     """The coarsest-grid solver runs an instance on 8, 4, 2 or 1 thread blocks by the number of
     instances (up to 19, 38, 76, more): blocked grids among its own (16^3, 24x8x16), extents that are no
