@@ -129,8 +129,8 @@ typedef struct {
  * dimension is even and >= 4) and allocates all device scratch.  *out receives the handle
  * (NULL on failure).  Any base grid of multiples of 8 is accepted: the coarse grids below the
  * last one made of 8^3 blocks (under OHM_MIXED* also power-of-two grids of at most 16^3
- * cells) are stepped by grid-wide launches while they have more than 16384 cells and by a
- * one-thread-block solver below that (in shared memory where the grids fit). */
+ * cells) are stepped by grid-wide launches until they fit into the shared memory of the
+ * coarsest-grid solver, which runs the rest of the V-cycle in one launch. */
 int ohm_create_hierarchy(const ohm_hier_desc *d, ohm_hier **out);
 
 /* Copies eta (> 0 and finite, [nblocks][8][8][8], every block including covered ones) into
@@ -295,7 +295,7 @@ int ohm_op_apply_L_f32(ohm_hier *h, const float *X_dev, double dt, float *out_de
 #define OHM_K_GHOST          4  /* coarse-fine ghost fill                                     */
 #define OHM_K_SYNC_DOWN      5  /* covered cells from their children                          */
 #define OHM_K_UPDATE         6  /* B += e                                                     */
-#define OHM_K_BOTTOM         7  /* coarsest-grid V-cycle (one thread block)                   */
+#define OHM_K_BOTTOM         7  /* coarsest-grid V-cycle                                      */
 #define OHM_K_NORM           8  /* norm reduction                                             */
 #define OHM_K_KRYLOV         9  /* FGMRES vector kernels (multi-dot, multi-axpy)              */
 
