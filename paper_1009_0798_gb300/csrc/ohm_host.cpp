@@ -507,7 +507,7 @@ int allocate(ohm_hier *H, std::string &err, int64_t *dry_bytes = nullptr) {
                 want((void **)&H->fg.sn, K * KMAX * sizeof(double));
                 want((void **)&H->fg.g, K * (KMAX + 1) * sizeof(double));
                 want((void **)&H->fg.beta0, K * 5 * sizeof(double));  // beta0, beta, brest, target, hn
-                want((void **)&H->fg.cycles, K * 2 * sizeof(int) + sizeof(int));  // cycles, jend, any_need2
+                want((void **)&H->fg.cycles, K * 2 * sizeof(int) + 2 * sizeof(int));  // cycles, jend, any_need2
                 want((void **)&H->fg.live, K * 6);  // live, arn, act, need2, run, compute mask
             }
         }
@@ -1678,7 +1678,7 @@ int fg_cycle(ohm_hier *H, double lamdt) {
     int st;
     FG(FG_CYCLE, 0);
     for (int j = 0; j < m; j++) {
-        FG(FG_ACT, j);
+        if (j == 0) FG(FG_ACT, 0);  // (later steps: by FG_STEP of the one before)
         if ((st = fg_prof_mask(H))) return st;
         void *r_save = H->amrbuf.r, *e_save = H->amrbuf.e;
         H->amrbuf.r = H->kv[j];
@@ -1696,11 +1696,11 @@ int fg_cycle(ohm_hier *H, double lamdt) {
         // v_m, formed by the last step, is never read: that step orthogonalises only where a
         // norm must be measured, and scales nothing
         const bool last = j + 1 == m;
-        if ((st = maxpy_inst_dev(H, H->kv[j + 1], H->kv[j + 1], S, last ? H->fg.any_need2 : nullptr))) return st;
-        if ((st = mdot_inst_dev(H, H->kv[j + 1], none, H->fg.any_need2))) return st;
-        FG(FG_RENORM, j);
-        if (!last && (st = maxpy_inst_dev(H, H->kv[j + 1], H->kv[j + 1], none, H->fg.any_need2))) return st;
-        FG(FG_GIVENS, j);
+        const int *need2 = H->fg.any_need2 + (j & 1);
+        if ((st = maxpy_inst_dev(H, H->kv[j + 1], H->kv[j + 1], S, last ? need2 : nullptr))) return st;
+        if ((st = mdot_inst_dev(H, H->kv[j + 1], none, need2))) return st;
+        FG(FG_STEP, j);
+        if (!last && (st = maxpy_inst_dev(H, H->kv[j + 1], H->kv[j + 1], none, need2))) return st;
     }
     FG(FG_SOLVE, 0);
     VecSet Z;

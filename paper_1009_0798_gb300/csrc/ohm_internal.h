@@ -280,10 +280,10 @@ struct FgState {
     uint8_t *imask = nullptr;                  // [K]
     const double *dots = nullptr;
     float *coef = nullptr;
-    int *any_need2 = nullptr;                  // 1 when some instance needs the norm pass of the step
+    int *any_need2 = nullptr;                  // [2] 1 when some instance needs the norm pass of the step (odd / even)
     int K = 0, m = 0, max_outer = 0;
 };
-enum FgOp { FG_START, FG_CYCLE, FG_ACT, FG_ORTHO, FG_RENORM, FG_GIVENS, FG_SOLVE, FG_RESTART_MASK, FG_RESTART };
+enum FgOp { FG_START, FG_CYCLE, FG_ACT, FG_ORTHO, FG_STEP, FG_SOLVE, FG_RESTART_MASK, FG_RESTART };
 cudaError_t launch_fg(const FgState &f, FgOp op, int j, cudaStream_t s);
 
 // Batched hierarchies: per-instance products out[q][0..k] (layout [ninst][KMAX+1]; part:

@@ -1990,6 +1990,13 @@ __global__ void __launch_bounds__(128) k_fg(FgState f, int op, int j) {
         for (int i = 0; i < KMAX; i++) c[i] = 0.f;
         c[KMAX] = scale;
     };
+    auto act = [&](int step) {
+        if (q == 0) f.any_need2[step & 1] = 0;
+        const uint8_t a = f.arn[q] && f.cycles[q] < f.max_outer;
+        f.act[q] = a;
+        f.imask[q] = a;
+        f.cycles[q] += a;
+    };
     switch (op) {
         case FG_START: {  // v_0 = rhs / beta0 for the instances that iterate
             const double b = sqrt(fmax(d[0], 0.0));
@@ -2006,11 +2013,7 @@ __global__ void __launch_bounds__(128) k_fg(FgState f, int op, int j) {
             break;
         }
         case FG_ACT: {  // instances that take Arnoldi step j (their V-cycle is counted)
-            if (q == 0) *f.any_need2 = 0;
-            const uint8_t a = f.arn[q] && f.cycles[q] < f.max_outer;
-            f.act[q] = a;
-            f.imask[q] = a;
-            f.cycles[q] += a;
+            act(j);
             break;
         }
         case FG_ORTHO: {  // h_ij = <w, v_i>; one-pass normalisation unless cancellation is large
@@ -2029,38 +2032,41 @@ __global__ void __launch_bounds__(128) k_fg(FgState f, int op, int j) {
                 c[KMAX] = (float)(1.0 / f.hn[q]);
             } else {
                 f.need2[q] = 1;
-                atomicOr(f.any_need2, 1);  // the norm pass after orthogonalising runs
+                atomicOr(f.any_need2 + (j & 1), 1);  // the norm pass after orthogonalising runs
             }
             break;
         }
-        case FG_RENORM: {  // the norm measured after orthogonalising, where the one pass was refused
+        // the rest of step j's scalars in one launch: the norm measured after orthogonalising, where the
+        // one pass was refused, the Givens update, and the instances that take step j + 1 (the vector
+        // update that the measured norm scales follows; its gate is step j's flag)
+        case FG_STEP: {
             clear(1.f);
-            if (!f.act[q] || !f.need2[q]) break;
-            f.hn[q] = sqrt(fmax(d[0], 0.0));
-            if (f.hn[q] > 0) c[KMAX] = (float)(1.0 / f.hn[q]);
-            break;
-        }
-        case FG_GIVENS: {
-            if (!f.act[q]) break;
-            const double hnq = f.hn[q];
-            h(j + 1, j) = hnq;
-            for (int i = 0; i < j; i++) {
-                const double t = cs[i] * h(i, j) + sn[i] * h(i + 1, j);
-                h(i + 1, j) = -sn[i] * h(i, j) + cs[i] * h(i + 1, j);
-                h(i, j) = t;
+            if (f.act[q]) {
+                if (f.need2[q]) {
+                    f.hn[q] = sqrt(fmax(d[0], 0.0));
+                    if (f.hn[q] > 0) c[KMAX] = (float)(1.0 / f.hn[q]);
+                }
+                const double hnq = f.hn[q];
+                h(j + 1, j) = hnq;
+                for (int i = 0; i < j; i++) {
+                    const double t = cs[i] * h(i, j) + sn[i] * h(i + 1, j);
+                    h(i + 1, j) = -sn[i] * h(i, j) + cs[i] * h(i + 1, j);
+                    h(i, j) = t;
+                }
+                const double den = hypot(h(j, j), h(j + 1, j));
+                cs[j] = den > 0 ? h(j, j) / den : 1.0;
+                sn[j] = den > 0 ? h(j + 1, j) / den : 0.0;
+                h(j, j) = den;
+                h(j + 1, j) = 0.0;
+                g[j + 1] = -sn[j] * g[j];
+                g[j] = cs[j] * g[j];
+                f.jend[q] = j + 1;
+                if (fabs(g[j + 1]) <= f.target[q] * f.beta0[q] || !(hnq > 0)) {
+                    f.arn[q] = 0;
+                    f.live[q] = 0;  // converged (or breakdown): no restart
+                }
             }
-            const double den = hypot(h(j, j), h(j + 1, j));
-            cs[j] = den > 0 ? h(j, j) / den : 1.0;
-            sn[j] = den > 0 ? h(j + 1, j) / den : 0.0;
-            h(j, j) = den;
-            h(j + 1, j) = 0.0;
-            g[j + 1] = -sn[j] * g[j];
-            g[j] = cs[j] * g[j];
-            f.jend[q] = j + 1;
-            if (fabs(g[j + 1]) <= f.target[q] * f.beta0[q] || !(hnq > 0)) {
-                f.arn[q] = 0;
-                f.live[q] = 0;  // converged (or breakdown): no restart
-            }
+            if (j + 1 < f.m) act(j + 1);
             break;
         }
         case FG_SOLVE: {  // x += sum y_i z_i with R y = g
