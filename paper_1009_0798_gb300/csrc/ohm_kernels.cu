@@ -51,6 +51,12 @@ __device__ __forceinline__ int pdl_wait() {
 // launch, and blocks that come up beside a running grid are spread unevenly over the SMs (28 boxes of
 // 64^3: 13.7-13.9 ms per step launched early throughout, 13.4 with this bound).
 constexpr unsigned PDL_GRID = 1024;
+// Kernels that are captured into a graph are launched as before, too: a graph has short gaps of its own,
+// and batches of 20 to 76 boxes of 16^3 lost 1-6% to the uneven placement.
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return s != nullptr && cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
 static bool pdl_small(unsigned grid) { return grid <= PDL_GRID; }
 template <typename... E, typename... A>
 static cudaError_t launch_as(bool early, void (*k)(E...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
@@ -63,7 +69,7 @@ static cudaError_t launch_as(bool early, void (*k)(E...), unsigned grid, unsigne
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = early ? 1 : 0;
+    cfg.numAttrs = early && !capturing(s) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
 }
 template <typename... E, typename... A>
@@ -3461,11 +3467,10 @@ template <typename T>
 constexpr int tail_divide() {
     return sizeof(T) == 8 ? 64 : 512;
 }
-// threads: an instance on one thread block (large batches) in float32 wants 32 warps to hide latency
-template <typename T, int CS>
-struct TailThreads {
-    static constexpr int N = CS == 1 && sizeof(T) == 4 ? 1024 : 512;
-};
+// Threads: 512, and 1024 for an instance on one thread block in float32 whose first grid is large enough
+// for 32 warps.  Two blocks of 512 share an SM there, so that a batch of up to 304 small instances
+// (e.g. 200 boxes of 16^3) is one wave.
+constexpr int TAIL_WIDE_CELLS = 1024;
 // coarsest grids of at most this many cells per colour keep their coefficients in registers (six
 // threads per cell: components x the two axes of each)
 constexpr int TAIL_REG_SLOTS = 18;
@@ -3617,9 +3622,8 @@ __device__ __forceinline__ void tail_update_f(const LexAcc<float> &a, const RbK<
 // one colour pass of grid s (Jacobi within the colour: every new value is formed before any is stored).
 // float64 takes a thread per cell and component: its arithmetic is spread over the four schedulers of
 // the SM, each of which has a quarter of the float64 rate.
-template <typename T, int CS>
+template <typename T, int CS, int NT>
 __device__ __forceinline__ void tail_colour(const TailP<T> &P, T *sh, const int *lut, size_t inst3, int s, int colour, bool zero) {
-    constexpr int NT = TailThreads<T, CS>::N;
     const LexDims D = P.d[s];
     const int n = D.n(), row = D.slots() / D.nz, rank = tail_rank<CS>();
     const bool dv = P.divided[s];
@@ -3665,11 +3669,11 @@ __device__ __forceinline__ void tail_colour(const TailP<T> &P, T *sh, const int 
     tail_sync<CS>(dv);
 }
 
-template <typename T, int CS>
+template <typename T, int CS, int NT>
 __device__ __forceinline__ void tail_sweeps(const TailP<T> &P, T *sh, const int *lut, size_t inst3, int s, int nsweep, bool zero) {
     for (int k = 0; k < nsweep; k++) {
-        tail_colour<T, CS>(P, sh, lut, inst3, s, 0, zero && k == 0);
-        tail_colour<T, CS>(P, sh, lut, inst3, s, 1, false);
+        tail_colour<T, CS, NT>(P, sh, lut, inst3, s, 0, zero && k == 0);
+        tail_colour<T, CS, NT>(P, sh, lut, inst3, s, 1, false);
     }
 }
 
@@ -3759,9 +3763,8 @@ __device__ __forceinline__ T tail_face(const T *Ba, const T *Bc, int o0, int os,
     return v_mul(es, v_mad(v_add(dn, d0), qs, v_sub(Bc[o0], Bc[os])));
 }
 
-template <typename T, int CS>
-__global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_constant__ TailP<T> P_arg, int nu1, int nu2, int nc) {
-    constexpr int NT = TailThreads<T, CS>::N;
+template <typename T, int CS, int NT>
+__global__ void __launch_bounds__(NT, CS == 1 && sizeof(T) == 4 && NT == 512 ? 2 : 1) k_tail(const __grid_constant__ TailP<T> P_arg, int nu1, int nu2, int nc) {
     const int inst = blockIdx.x / CS;
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -3837,7 +3840,7 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
     const size_t inst3 = 3 * (size_t)inst;
     int s = 0;
     for (; s < P.n - 1; s++) {
-        tail_sweeps<T, CS>(P, sh, lut, inst3, s, nu1, true);
+        tail_sweeps<T, CS, NT>(P, sh, lut, inst3, s, nu1, true);
         // residual and its restriction, 8 lanes per coarse cell: in float64 each with the three outer
         // faces of its child (k_pair_op's octet form: the fluxes between the children cancel in their
         // sum).  A block takes the coarse cells of its planes, or half of a coarse plane where it owns
@@ -3914,7 +3917,7 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
             done = true;
         }
     }
-    if (!done) tail_sweeps<T, CS>(P, sh, lut, inst3, s, nc, true);
+    if (!done) tail_sweeps<T, CS, NT>(P, sh, lut, inst3, s, nc, true);
     for (s = P.n - 2; s >= 0; s--) {
         const LexDims D = P.d[s], C = P.d[s + 1];
         const int n = D.n(), ncs = C.n(), pl = D.nx * D.ny;
@@ -3956,7 +3959,7 @@ __global__ void __launch_bounds__(TailThreads<T, CS>::N, 1) k_tail(const __grid_
             tail_store_cell<CS>(P, sh, s, z, o, n, v, rank);  // no other block reads this cell in the pass
         }
         tail_sync<CS>(P.divided[s]);
-        tail_sweeps<T, CS>(P, sh, lut, inst3, s, nu2, false);
+        tail_sweeps<T, CS, NT>(P, sh, lut, inst3, s, nu2, false);
     }
     // e of the first grid: the own planes, or a share of the whole copy
     const LexDims D = P.d[0];
@@ -4059,15 +4062,15 @@ bool tail_fits(const SmallDev<T> &sm) {
 template bool tail_fits<double>(const SmallDev<double> &);
 template bool tail_fits<float>(const SmallDev<float> &);
 
-template <typename T, int CS>
+template <typename T, int CS, int NT>
 static void tail_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute at[2], int ninst, size_t bytes, cudaStream_t s) {
-    static const bool attr = (cudaFuncSetAttribute(k_tail<T, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_MAX),
-                              CS > 8 ? cudaFuncSetAttribute(k_tail<T, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess,
+    static const bool attr = (cudaFuncSetAttribute(k_tail<T, CS, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_MAX),
+                              CS > 8 ? cudaFuncSetAttribute(k_tail<T, CS, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess,
                               true);
     (void)attr;
     cfg = {};
     cfg.gridDim = dim3((unsigned)(ninst * CS));
-    cfg.blockDim = dim3(TailThreads<T, CS>::N);
+    cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = s;
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -4077,19 +4080,19 @@ static void tail_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute at[2], int 
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = CS > 1 ? 2 : 1;
-    if (sizeof(T) == 8) {  // as launch_full
+    if (sizeof(T) == 8 || capturing(s)) {  // as launch_full
         cfg.attrs = at + 1;
         cfg.numAttrs = CS > 1 ? 1 : 0;
     }
 }
 
-template <typename T, int CS>
+template <typename T, int CS, int NT = 512>
 static cudaError_t launch_tail_cs(const TailP<T> &P, int ninst, size_t bytes, int nu_pre, int nu_post, int n_coarse,
                                   cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[2];
-    tail_config<T, CS>(cfg, at, ninst, bytes, s);
-    return cudaLaunchKernelEx(&cfg, k_tail<T, CS>, P, nu_pre, nu_post, n_coarse);
+    tail_config<T, CS, NT>(cfg, at, ninst, bytes, s);
+    return cudaLaunchKernelEx(&cfg, k_tail<T, CS, NT>, P, nu_pre, nu_post, n_coarse);
 }
 
 // whether the device can hold a cluster of 16 of the float64 solver's blocks (asked once)
@@ -4097,9 +4100,9 @@ static bool tail_16() {
     static const bool ok = [] {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at[2];
-        tail_config<double, 16>(cfg, at, 1, TAIL_SMEM_MAX, nullptr);
+        tail_config<double, 16, 512>(cfg, at, 1, TAIL_SMEM_MAX, nullptr);
         int n = 0;
-        const bool fits = cudaOccupancyMaxActiveClusters(&n, k_tail<double, 16>, &cfg) == cudaSuccess && n > 0;
+        const bool fits = cudaOccupancyMaxActiveClusters(&n, k_tail<double, 16, 512>, &cfg) == cudaSuccess && n > 0;
         cudaGetLastError();
         return fits;
     }();
@@ -4111,7 +4114,9 @@ cudaError_t launch_tail(const SmallDev<T> &sm, double lamdt, int nu_pre, int nu_
     if (sm.n == 0) return cudaSuccess;
     TailP<T> P;
     size_t bytes = 0;
-    const int cs = tail_cluster<T>(sm.ninst);
+    // (a first grid that is not divided has nothing for a cluster to do)
+    const bool divide = (int64_t)sm.dims[0][0] * sm.dims[0][1] * sm.dims[0][2] > tail_divide<T>();
+    const int cs = divide ? tail_cluster<T>(sm.ninst) : 1;
     if (!tail_plan(sm, lamdt, cs, true, P, bytes) && !tail_plan(sm, lamdt, cs, false, P, bytes))
         return cudaErrorInvalidValue;  // callers ask tail_fits first
     if constexpr (sizeof(T) == 8) {
@@ -4121,8 +4126,12 @@ cudaError_t launch_tail(const SmallDev<T> &sm, double lamdt, int nu_pre, int nu_
         case 8: return launch_tail_cs<T, 8>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
         case 4: return launch_tail_cs<T, 4>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
         case 2: return launch_tail_cs<T, 2>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
-        default: return launch_tail_cs<T, 1>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
+        default: break;
     }
+    if constexpr (sizeof(T) == 4) {
+        if (P.d[0].slots() > TAIL_WIDE_CELLS / 2) return launch_tail_cs<T, 1, 1024>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
+    }
+    return launch_tail_cs<T, 1>(P, sm.ninst, bytes, nu_pre, nu_post, n_coarse, s);
 }
 template cudaError_t launch_tail<double>(const SmallDev<double> &, double, int, int, int, cudaStream_t);
 template cudaError_t launch_tail<float>(const SmallDev<float> &, double, int, int, int, cudaStream_t);
