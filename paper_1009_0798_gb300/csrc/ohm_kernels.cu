@@ -695,7 +695,12 @@ cudaError_t launch_composite(const GridDev &g, const float *X, const float *Y, c
 // ZERO: both passes of the sweep from e = 0 in one launch (as k_smooth_d's; colour = 1): the tile holds
 // the pointwise red update inv r at red cells and 0 elsewhere, e_in is not read (three-level mixed step
 // 2.33 -> 2.22 ms, with the right-hand sides in flight during the staging 2.14).
-template <typename T, bool ZERO>
+// EARLY = false (grids of more than PDL_GRID blocks): no early launch, and a general pass loads its right-hand
+// sides after the stencil.  Held through the staging they cost more registers than the latency is worth
+// once every SM has several waves of blocks: 128^3 34.8 us a pass, 38.8 loaded ahead, 41.9 launched early
+// with that; 160^3 61, 71, 76; at 64^3 and below the three are the same.  The pass from zero reads r and inv
+// in any case and gains from the head start (128^3 32.8 us).
+template <typename T, bool ZERO, bool EARLY>
 __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__ e_in, T *__restrict__ e_out,
                                                 const T *__restrict__ r, const T *__restrict__ eta,
                                                 const T *__restrict__ inv, const T *__restrict__ Ge,
@@ -705,22 +710,26 @@ __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__
     __shared__ __align__(16) T tE[G::CS];
     __shared__ int snb[27];
     const int b0 = blockIdx.x;
-    pdl_trigger();
+    pdl_trigger<EARLY>();
+    if (!EARLY && skip_block(g, b0)) return;  // (masked blocks return before they load anything)
     stage_nbr(snb, g.nbr, b0);
     const int slot = g.gslot ? g.gslot[b0] : -1;
-    const int b = b0 + pdl_wait();
-    if (skip_block(g, b)) return;
+    const int b = b0 + pdl_wait<EARLY>();
+    if (EARLY && skip_block(g, b)) return;
     const int t = threadIdx.x;
     const int k = t >> 5, j = (t >> 2) & 7;
     const int ic = 2 * (t & 3) + ((j + k + colour) & 1);      // colour cell
     const int io = 2 * (t & 3) + ((j + k + colour + 1) & 1);  // other colour
     const int cc = (k * 8 + j) * 8 + ic, co = (k * 8 + j) * 8 + io;
-    T rr[3], iv[3];  // in flight while the tile is staged
+    T rr[3], iv[3];
+    auto load_rhs = [&] {
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
-        rr[c] = r[((size_t)b * 3 + c) * B3 + cc];
-        iv[c] = inv[((size_t)b * 3 + c) * B3 + cc];
-    }
+        for (int c = 0; c < 3; c++) {
+            rr[c] = r[((size_t)b * 3 + c) * B3 + cc];
+            iv[c] = inv[((size_t)b * 3 + c) * B3 + cc];
+        }
+    };
+    if constexpr (EARLY || ZERO) load_rhs();  // in flight while the tile is staged
     __syncthreads();
     if constexpr (ZERO) {
         for (int h = t; h < T3 / 2; h += 256) {
@@ -754,6 +763,7 @@ __global__ void __launch_bounds__(256) k_smooth(GridDev g, const T *__restrict__
     dv[1] = (xh1 - xl1) + (zh2 - zl2);
     dv[2] = (xh2 - xl2) + (yh2 - yl2);
     const int po = G::at(io + 1, j + 1, k + 1);
+    if constexpr (!(EARLY || ZERO)) load_rhs();
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         size_t base = ((size_t)b * 3 + c) * B3;
@@ -1302,12 +1312,12 @@ cudaError_t launch_smooth<float>(const GridDev &g, const float *e_in, float *e_o
                                  const float *inv, const float *Ge, const float *Geta, double lamdt, int colour,
                                  cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    return launch_pdl(k_smooth<float, false>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
+    return launch_pdl2(k_smooth<float, false, true>, k_smooth<float, false, false>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
 }
 cudaError_t launch_smooth_zero(const GridDev &g, float *e_out, const float *r, const float *eta, const float *inv,
                                const float *Geta, double lamdt, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    return launch_pdl(k_smooth<float, true>, g.nblk, 256, 0, s, g, nullptr, e_out, r, eta, inv, nullptr, Geta, (float)(lamdt / (2.0 * g.h * g.h)), 1);
+    return launch_pdl2(k_smooth<float, true, true>, k_smooth<float, true, false>, g.nblk, 256, 0, s, g, nullptr, e_out, r, eta, inv, nullptr, Geta, (float)(lamdt / (2.0 * g.h * g.h)), 1);
 }
 cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
                                const double *Geta, double lamdt, cudaStream_t s) {

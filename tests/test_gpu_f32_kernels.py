@@ -271,3 +271,23 @@ def test_float32_coarsest_grid_solve_matches_oracle_vcycle(ohm, orc, base, omega
     got = host(e).reshape(r.shape)
     want = oracle_coarse_vcycle(o, m0, r, eta[0], dt, 2, 2, 4, omega if omega else 1.0)
     check32(got, want, f"coarsest solve {base} omega={omega}: grid {dims}")
+
+
+@pytest.mark.parametrize("start", ["iterate", "zero"])
+@pytest.mark.parametrize("base", [(128, 64, 64), (88, 96, 64)])
+def test_float32_colour_passes_on_both_sides_of_the_early_launch_bound(ohm, orc, base, start):
+    """The colour passes have an instance for grids of at most 1024 blocks (128 x 64 x 64) and one for
+    larger grids (88 x 96 x 64: 1056), which loads its right-hand sides at another place."""
+    h = W.uniform(*base, 1.0 / base[0])
+    o = orc.Oracle(h, 0.5)
+    g = mixed(ohm, h, 1.2)
+    dims, nb, ijk = ohm.ohm_mg_grid_info(g, 0)
+    e, r, eta = grid_inputs(dims, 61)
+    if start == "zero":
+        e = np.zeros_like(e)
+    dt = 5.0 * h.dx0 ** 2
+    e_in = None if start == "zero" else f32(grid_of_dense(e, ijk))[0]
+    out = torch.full((nb * 1536,), float("nan"), dtype=torch.float32, device="cuda")
+    ohm.ohm_op_grid_sweep_f32(g, 0, e_in, out, f32(grid_of_dense(r, ijk))[0], f32(grid_of_dense(eta, ijk))[0], dt, 1)
+    got = dense_of_grid(host(out).reshape(nb, 3, 8, 8, 8), ijk, dims, 3)
+    check32(got, oracle_sweep(o, 0, e, r, eta, dt, 1.2), f"colour passes {base} {start}")
