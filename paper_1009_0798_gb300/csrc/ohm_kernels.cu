@@ -58,6 +58,9 @@ static bool capturing(cudaStream_t s) {
     return s != nullptr && cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
 }
 static bool pdl_small(unsigned grid) { return grid <= PDL_GRID; }
+// As after <<< >>>, a refused launch also stays in the runtime's last error: every launcher ends in
+// cudaGetLastError(), which returns and clears it (left there, the process's next check would report it
+// from a call that succeeded).
 template <typename... E, typename... A>
 static cudaError_t launch_as(bool early, void (*k)(E...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
     cudaLaunchConfig_t cfg = {};
@@ -649,8 +652,9 @@ static cudaError_t launch_composite_t(const GridDev &g, const typename CompTypes
     (void)attr;
     auto go = [&](auto k, auto kl) {  // early on small grids
         const bool early = E && pdl_small(g.nblk);
-        return launch_as(early, early ? k : kl, g.nblk, 512, sm, s, g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
-                         vol, outS, coef2, 0.5 / g.h, 2.0 * g.h, ymx);
+        launch_as(early, early ? k : kl, g.nblk, 512, sm, s, g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
+                  vol, outS, coef2, 0.5 / g.h, 2.0 * g.h, ymx);
+        return cudaGetLastError();
     };
     if (partials)  // with norm partials (the block reductions are compiled out otherwise)
         return go(k_composite<TC, TO, true, YT, E>, k_composite<TC, TO, true, YT, false>);
@@ -1255,8 +1259,9 @@ static cudaError_t launch_composite_kind(const GridDev &g, const double *X, cons
     constexpr size_t sm = S::template bytes<TO>;
     static const bool attr = (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), true);
     (void)attr;
-    return launch_full(k, g.nblk * (8 / NZ), S::NT, sm, s, g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
-                       outS, coef2, 0.5 / g.h, 2.0 * g.h, keep_ss);
+    launch_full(k, g.nblk * (8 / NZ), S::NT, sm, s, g, X, Y, eta, Gx, Geta, a, coef, d, out, out2, reg, rsrc_tab, partials,
+                outS, coef2, 0.5 / g.h, 2.0 * g.h, keep_ss);
+    return cudaGetLastError();
 }
 
 template <int NZ, typename TO>
@@ -1312,12 +1317,14 @@ cudaError_t launch_smooth<float>(const GridDev &g, const float *e_in, float *e_o
                                  const float *inv, const float *Ge, const float *Geta, double lamdt, int colour,
                                  cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    return launch_pdl2(k_smooth<float, false, true>, k_smooth<float, false, false>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
+    launch_pdl2(k_smooth<float, false, true>, k_smooth<float, false, false>, g.nblk, 256, 0, s, g, e_in, e_out, r, eta, inv, Ge, Geta, (float)(lamdt / (2.0 * g.h * g.h)), colour);
+    return cudaGetLastError();
 }
 cudaError_t launch_smooth_zero(const GridDev &g, float *e_out, const float *r, const float *eta, const float *inv,
                                const float *Geta, double lamdt, cudaStream_t s) {
     if (g.nblk == 0) return cudaSuccess;
-    return launch_pdl2(k_smooth<float, true, true>, k_smooth<float, true, false>, g.nblk, 256, 0, s, g, nullptr, e_out, r, eta, inv, nullptr, Geta, (float)(lamdt / (2.0 * g.h * g.h)), 1);
+    launch_pdl2(k_smooth<float, true, true>, k_smooth<float, true, false>, g.nblk, 256, 0, s, g, nullptr, e_out, r, eta, inv, nullptr, Geta, (float)(lamdt / (2.0 * g.h * g.h)), 1);
+    return cudaGetLastError();
 }
 cudaError_t launch_smooth_zero(const GridDev &g, double *e_out, const double *r, const double *eta, const double *inv,
                                const double *Geta, double lamdt, cudaStream_t s) {
@@ -1618,8 +1625,11 @@ cudaError_t launch_smooth_rb(const GridDev &g, const float *e_in, float *e_out, 
     }();
     (void)attr;
     const RbK<float> K = rb_constants<float>(lamdt, g.h, g.omega);
-    if (e_in) return launch_pdl2(k_smooth_rb<false, true>, k_smooth_rb<false, false>, g.nblk, 256, sm, s, g, e_in, e_out, r, eta, K);
-    return launch_pdl2(k_smooth_rb<true, true>, k_smooth_rb<true, false>, g.nblk, 256, sm, s, g, nullptr, e_out, r, eta, K);  // from e = 0
+    if (e_in)
+        launch_pdl2(k_smooth_rb<false, true>, k_smooth_rb<false, false>, g.nblk, 256, sm, s, g, e_in, e_out, r, eta, K);
+    else  // from e = 0
+        launch_pdl2(k_smooth_rb<true, true>, k_smooth_rb<true, false>, g.nblk, 256, sm, s, g, nullptr, e_out, r, eta, K);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ fused sweep on brick pairs
@@ -4102,7 +4112,8 @@ static cudaError_t launch_tail_cs(const TailP<T> &P, int ninst, size_t bytes, in
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[2];
     tail_config<T, CS, NT>(cfg, at, ninst, bytes, s);
-    return cudaLaunchKernelEx(&cfg, k_tail<T, CS, NT>, P, nu_pre, nu_post, n_coarse);
+    cudaLaunchKernelEx(&cfg, k_tail<T, CS, NT>, P, nu_pre, nu_post, n_coarse);
+    return cudaGetLastError();
 }
 
 // whether the device can hold a cluster of 16 of the float64 solver's blocks (asked once)
