@@ -366,3 +366,58 @@ def test_coarse_solver_clusters_give_same_bits_and_match_oracle(ohm, orc, base, 
                 want, _ = o.cn_step(bs[pick[q]], dts[pick[q]], -1.0, 2, 1, 5, 2)
                 assert rel_err(out[q], want) < 1e-12
         g.close()
+
+
+@pytest.mark.parametrize("edge", [40, 56])
+def test_float64_coarse_solver_on_every_cluster_size(ohm, orc, edge):
+    """The float64 coarsest-grid solver runs an instance on 16, 8, 4, 2 or 1 thread blocks (up to 8, 19, 38,
+    76 instances, more).  40^3 and 56^3 end on 5^3 and 7^3, which are still divided over the thread
+    blocks: planes per block 1, 2 or 4, the last block partly filled, some blocks without planes."""
+    h = W.uniform(edge, edge, edge, 1.0 / edge)
+    bs, etas = instances(h, 2, 400)
+    dts = [6.0 * h.dx0 ** 2, 9.0 * h.dx0 ** 2]
+    wants = []
+    for q in (0, 1):
+        wants.append(orc.Oracle(h, 0.5, etas[q]).cn_step(bs[q], dts[q], -1.0, 2, 1, 5, 2)[0])
+    first = None
+    for K in (2, 12, 20, 40, 80):
+        pick = [0] + [1] * (K - 1)
+        g = make(ohm, h, K, nu_pre=2, nu_post=1, n_coarse=5, max_outer=2)
+        ohm.ohm_set_eta(g, dev(stack(h, [etas[q] for q in pick])))
+        B = dev(stack(h, [bs[q] for q in pick]))
+        ohm.ohm_cn_step_batch(g, B, [dts[q] for q in pick], -1.0)
+        out = unstack(h, host(B).reshape(-1, 3, 8, 8, 8), K)
+        first = out[0] if first is None else first
+        assert np.array_equal(out[0], first), K
+        for q in (0, K - 1):
+            assert rel_err(out[q], wants[pick[q]]) < 1e-12, (K, q)
+        g.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_refined_batch_of_many_blocks_same_bits_as_alone(ohm, orc, precision):
+    """40 instances of three levels (8 + 64 + 64 blocks): the refined levels of 2560 blocks take the float64
+    kernels' whole blocks (alone: slabs of two planes) with flux registers, refluxing and ghosts, and the
+    float32 kernels of large grids.  The bits are those of the instance alone; float64 is the oracle's."""
+    from tests.helpers import amr_three_level
+    h = amr_three_level(16)
+    assert [hi - lo for lo, hi in level_ranges(h)] == [8, 64, 64]
+    K = 40
+    bs, etas = instances(h, 2, 500)
+    dts = [6.0 * h.dx(2) ** 2, 9.0 * h.dx(2) ** 2]
+    pick = [0] + [1] * (K - 1)
+    g = make(ohm, h, K, precision=precision, max_outer=2)
+    ohm.ohm_set_eta(g, dev(stack(h, [etas[q] for q in pick])))
+    B = dev(stack(h, [bs[q] for q in pick]))
+    ohm.ohm_cn_step_batch(g, B, [dts[q] for q in pick], -1.0)
+    out = unstack(h, host(B).reshape(-1, 3, 8, 8, 8), K)
+    for q in (0, K - 1):
+        a = pick[q]
+        one = make(ohm, h, 1, precision=precision, max_outer=2)
+        ohm.ohm_set_eta(one, dev(etas[a]))
+        b1 = dev(bs[a])
+        ohm.ohm_cn_step_batch(one, b1, [dts[a]], -1.0)
+        assert np.array_equal(host(b1).reshape(out[q].shape), out[q])
+        if precision == 0:
+            want, _ = orc.Oracle(h, 0.5, etas[a]).cn_step(bs[a], dts[a], -1.0, 2, 2, 8, 2)
+            assert rel_err(out[q], want) < 1e-12

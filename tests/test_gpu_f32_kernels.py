@@ -291,3 +291,25 @@ def test_float32_colour_passes_on_both_sides_of_the_early_launch_bound(ohm, orc,
     ohm.ohm_op_grid_sweep_f32(g, 0, e_in, out, f32(grid_of_dense(r, ijk))[0], f32(grid_of_dense(eta, ijk))[0], dt, 1)
     got = dense_of_grid(host(out).reshape(nb, 3, 8, 8, 8), ijk, dims, 3)
     check32(got, oracle_sweep(o, 0, e, r, eta, dt, 1.2), f"colour passes {base} {start}")
+
+
+@pytest.mark.parametrize("base", [(48, 16, 32), (16, 48, 32), (96, 32, 32)])
+def test_float32_vcycle_with_blocked_grids_in_the_coarse_solver_matches_oracle(ohm, orc, base):
+    """One V(2,1) cycle of the mixed step (V-cycle budget 1, no tolerance) on boxes whose coarse grids are
+    made of 8^3 blocks and still small enough for the coarsest-grid solver: 24 x 8 x 16, 8 x 24 x 16 and,
+    below a swept 48 x 16 x 16, 24 x 8 x 8.  Its increment B - b is the float32 cycle's correction of the
+    residual; against the oracle's it carries the rounding of the residual, of the coarse eta and of a dozen
+    chained passes, each held to a few u above: the single-pass tolerance, 34 u, covers their sum."""
+    h = W.uniform(*base, 1.0 / base[0])
+    rng = np.random.default_rng(71)
+    b = rng.standard_normal((h.nblocks, 3, 8, 8, 8)).astype(np.float32).astype(np.float64)
+    eta = (10 ** rng.uniform(-0.5, 0.5, (h.nblocks, 1, 8, 8, 8))).astype(np.float32).astype(np.float64)
+    g = ohm.ohm_create_hierarchy(h.base_cells, h.dx0, h.blocks, lam=0.5, precision=ohm.OHM_MIXED, nu_pre=2, nu_post=1,
+                                 n_coarse=4, max_outer=1)
+    ohm.ohm_set_eta(g, torch.from_numpy(eta).cuda())
+    B = torch.from_numpy(b).cuda()
+    dt = 5.0 * h.dx0 ** 2
+    st = ohm.ohm_cn_step(g, B, None, dt, -1.0)
+    assert st["cycles"] == 1
+    want, _ = orc.Oracle(h, 0.5, eta).cn_step(b, dt, -1.0, 2, 1, 4, 1)
+    check32(host(B).reshape(b.shape) - b, want - b, f"V-cycle {base}")
