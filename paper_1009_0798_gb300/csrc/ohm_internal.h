@@ -46,7 +46,7 @@ template <typename T>
 struct SmallDev {
     int n = 0;                      // number of small grids
     int ninst = 1;                  // instances; the arrays of grid s hold them one after another
-                                    // (instance q at q * ncomp * cells(s)), one thread block each
+                                    // (instance q at q * ncomp * cells(s))
     const uint8_t *imask = nullptr; // instances whose flag is 0 are skipped
     double omega = 1.0;             // relaxation factor folded into inv (1 = Gauss-Seidel)
     int dims[MAX_SMALL][3];

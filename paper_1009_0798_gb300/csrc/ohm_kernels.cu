@@ -319,31 +319,6 @@ __device__ __forceinline__ void stage_rows(T *__restrict__ tile, const TS *__res
     }
 }
 
-// Element-wise staging, same tile layout as stage_rows: consecutive threads take consecutive
-// cells of a tile row, so global loads are coalesced along x and shared-memory stores of a
-// warp fall on consecutive addresses (stage_rows, one thread per row, stores 32 different
-// rows at the same column at once, which for padded row strides hits few banks).
-template <typename T, int NC, int HW, int RS>
-__device__ __forceinline__ void stage_cells(T *__restrict__ tile, const T *__restrict__ F, const int *__restrict__ snb,
-                                            const T *__restrict__ ghost) {
-    constexpr int S = 8 + 2 * HW, S2 = S * S, S3 = S2 * S;
-    for (int e = threadIdx.x; e < S3; e += blockDim.x) {
-        const int tk = e / S2, rem = e - tk * S2, tj = rem / S, ti = rem - tj * S;
-        const int li = ti - HW, lj = tj - HW, lk = tk - HW;
-        const int di = li < 0 ? -1 : (li > 7 ? 1 : 0), dj = lj < 0 ? -1 : (lj > 7 ? 1 : 0), dk = lk < 0 ? -1 : (lk > 7 ? 1 : 0);
-        const int src = snb[(dk + 1) * 9 + (dj + 1) * 3 + (di + 1)];
-        const int dst = (tk * S + tj) * RS + ti;
-        if (src >= 0) {
-            const T *p = F + (size_t)src * NC * B3 + ((lk - 8 * dk) * 8 + (lj - 8 * dj)) * 8 + (li - 8 * di);
-#pragma unroll
-            for (int c = 0; c < NC; c++) tile[c * S2 * RS + dst] = p[c * B3];
-        } else {
-#pragma unroll
-            for (int c = 0; c < NC; c++) tile[c * S2 * RS + dst] = ghost ? ghost[c * T3 + e] : T(0);
-        }
-    }
-}
-
 // neighbour ids of block b into shared memory (call before stage_rows, then __syncthreads)
 __device__ __forceinline__ void stage_nbr(int *snb, const int *__restrict__ nbr, int b) {
     if (threadIdx.x < 27) snb[threadIdx.x] = __ldg(nbr + b * 27 + threadIdx.x);
@@ -893,12 +868,10 @@ __global__ void __launch_bounds__(32 * NZ) k_smooth_d(GridDev g, const double *_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
     __shared__ int snb[27];
-    const int b0 = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
-    pdl_trigger<false>();
-    if (skip_block(g, b0)) return;  // (masked blocks return before they load anything)
-    stage_nbr(snb, g.nbr, b0);
-    const int slot = g.gslot ? g.gslot[b0] : -1;
-    const int b = b0 + pdl_wait<false>();
+    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
+    if (skip_block(g, b)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b);
+    const int slot = g.gslot ? g.gslot[b] : -1;
     __syncthreads();
     stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
     const int t = threadIdx.x, i2 = t & 3, j = (t >> 2) & 7, kl = t >> 5;
@@ -1070,12 +1043,10 @@ __global__ void __launch_bounds__(64 * NZ, 16 / NZ)
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS;
     double *G1 = P + S::SUMS, *G2 = G1 + S::FACES, *ES = G2 + S::FACES;  // ES: !FLUX only
     __shared__ int snb[27];
-    const int b0 = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ)), t = threadIdx.x;
-    pdl_trigger<false>();
-    if (skip_block(g, b0)) return;  // (masked blocks return before they load anything)
-    stage_nbr(snb, g.nbr, b0);
-    const int slot = g.gslot ? g.gslot[b0] : -1;
-    const int b = b0 + pdl_wait<false>();
+    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ)), t = threadIdx.x;
+    if (skip_block(g, b)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b);
+    const int slot = g.gslot ? g.gslot[b] : -1;
     if (g.covered && g.covered[b]) {
         if (NORMS && t < 3 && !(keep_ss && t == 1)) partials[(size_t)blockIdx.x * 3 + t] = 0.0;
         return;
@@ -1385,16 +1356,15 @@ __device__ __forceinline__ V v_zero() {
     return v_splat<V>(0.0f);
 }
 
-// The relaxed update ev + res / den: float32 through the hardware's approximate reciprocal
+// The relaxed update ev + res / den of the float32 sweeps, through the hardware's approximate reciprocal
 // (rcp.approx, relative error below 2^-23; a smoothing weight needs no correctly rounded
-// quotient) and one FMA, float64 with an exact division.
+// quotient) and one FMA.
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 __device__ __forceinline__ float rb_relax(float ev, float res, float den) { return v_mad(res, rcp_approx(den), ev); }
-__device__ __forceinline__ double rb_relax(double ev, double res, double den) { return v_add(ev, __ddiv_rn(res, den)); }
 
 // The point update of one colour pass (Eq. 19 with R from Eq. 20 and alpha from Eqs. 21-23),
 // written against an accessor that returns component C of the field, or eta, at a compile-time
@@ -2285,12 +2255,10 @@ __global__ void __launch_bounds__(32 * NZ) k_resid_restrict_d(GridDev g, const d
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *tB = reinterpret_cast<double *>(smem_raw), *tE = tB + 3 * S::CS, *P = tE + S::CS, *side = P + S::SUMS;
     __shared__ int snb[27];
-    const int b0 = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
-    pdl_trigger<false>();
-    if (skip_block(g, b0)) return;  // (masked blocks return before they load anything)
-    stage_nbr(snb, g.nbr, b0);
-    const int slot = g.gslot ? g.gslot[b0] : -1, t = threadIdx.x;
-    const int b = b0 + pdl_wait<false>();
+    const int b = blockIdx.x / (8 / NZ), z0 = NZ * (blockIdx.x % (8 / NZ));
+    if (skip_block(g, b)) return;  // (masked blocks return before they load anything)
+    stage_nbr(snb, g.nbr, b);
+    const int slot = g.gslot ? g.gslot[b] : -1, t = threadIdx.x;
     __syncthreads();
     stage_slab<NZ, 1>(tE, eta, snb, slot >= 0 && Geta ? Geta + (size_t)slot * T3 : nullptr, z0);
     stage_slab<NZ, 3>(tB, e, snb, slot >= 0 && Ge ? Ge + (size_t)slot * 3 * T3 : nullptr, z0);
@@ -2496,8 +2464,7 @@ __global__ void __launch_bounds__(256) k_prolong_add_d(GridDev g, GridDev gc, co
                                                        const double *__restrict__ lex, int3 ld, double *__restrict__ fine,
                                                        int *__restrict__ err) {
     __shared__ double win[3 * 216], wx8[3 * 288], wy8[3 * 384];  // [6][6][6], [6][6][8], [6][8][8] per component
-    pdl_trigger<false>();
-    const int b = blockIdx.x + pdl_wait<false>();
+    const int b = blockIdx.x;
     if (skip_block(g, b)) return;
     const int o = lex ? 0 : g.octant[b];
     const int pb = lex ? 0 : g.parent[b];
@@ -2747,8 +2714,6 @@ cudaError_t launch_ghost_fill(const GridDev &g, const GridDev &gc, const TS_ *co
 }
 template cudaError_t launch_ghost_fill<double, double>(const GridDev &, const GridDev &, const double *, int, double *,
                                                        int *, cudaStream_t);
-template cudaError_t launch_ghost_fill<double, float>(const GridDev &, const GridDev &, const double *, int, float *,
-                                                      int *, cudaStream_t);
 template cudaError_t launch_ghost_fill<float, float>(const GridDev &, const GridDev &, const float *, int, float *,
                                                      int *, cudaStream_t);
 
@@ -3981,13 +3946,12 @@ __global__ void __launch_bounds__(NT, CS == 1 && sizeof(T) == 4 && NT == 512 ? 2
         tail_sync<CS>(P.divided[s]);
         tail_sweeps<T, CS, NT>(P, sh, lut, inst3, s, nu2, false);
     }
-    // e of the first grid: the own planes, or a share of the whole copy
+    // e of the first grid: the own planes (all of them where one block has the instance)
     const LexDims D = P.d[0];
     const int n = D.n(), pl = D.nx * D.ny;
     int z0, z1;
     tail_planes<CS>(P, 0, rank, z0, z1);
-    const int step = CS > 1 && !P.divided[0] ? CS * NT : NT;
-    for (int q = z0 * pl + threadIdx.x + (CS > 1 && !P.divided[0] ? rank * NT : 0); q < z1 * pl; q += step) {
+    for (int q = z0 * pl + threadIdx.x; q < z1 * pl; q += NT) {
         int x, y, z, cst;
         D.cell(q, x, y, z);
         const size_t id = inst3 * n + tail_gidx(P, lut, 0, x, y, z, 3, cst);
