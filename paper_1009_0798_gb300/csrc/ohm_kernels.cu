@@ -3966,16 +3966,6 @@ static int ilog2_exact(int v) {
     return (1 << l) == v ? l : -1;
 }
 
-// cluster size: enough thread blocks per instance to use the SMs, and no more than one wave of them.
-// float64 takes 16 (the largest the hardware forms, beyond the portable 8) for few instances: its
-// passes are bound by the SMs' float64 units.
-static bool tail_16();
-template <typename T>
-static int tail_cluster(int ninst) {
-    if (sizeof(T) == 8 && ninst <= 8 && tail_16()) return 16;
-    return ninst <= 19 ? 8 : (ninst <= 38 ? 4 : (ninst <= 76 ? 2 : 1));
-}
-
 // the solver's table and shared-memory bytes; false when the grids do not fit
 template <typename T>
 static bool tail_plan(const SmallDev<T> &sm, double lamdt, int cs, bool own, TailP<T> &P, size_t &bytes) {
@@ -4080,18 +4070,36 @@ static cudaError_t launch_tail_cs(const TailP<T> &P, int ninst, size_t bytes, in
     return cudaGetLastError();
 }
 
-// whether the device can hold a cluster of 16 of the float64 solver's blocks (asked once)
-static bool tail_16() {
-    static const bool ok = [] {
+// clusters of CS of the solver's blocks that the device holds at once (asked once, for the largest shared memory)
+template <typename T, int CS>
+static int tail_resident() {
+    static const int n = [] {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at[2];
-        tail_config<double, 16, 512>(cfg, at, 1, TAIL_SMEM_MAX, nullptr);
-        int n = 0;
-        const bool fits = cudaOccupancyMaxActiveClusters(&n, k_tail<double, 16, 512>, &cfg) == cudaSuccess && n > 0;
+        tail_config<T, CS, 512>(cfg, at, 1, TAIL_SMEM_MAX, nullptr);
+        int k = 0;
+        if (cudaOccupancyMaxActiveClusters(&k, k_tail<T, CS, 512>, &cfg) == cudaSuccess) return k;
         cudaGetLastError();
-        return fits;
+        return 0;
     }();
-    return ok;
+    return n;
+}
+
+// Cluster size: the largest of which all instances run at once.  float64 goes up to 16 (the largest the
+// hardware forms, beyond the portable 8): its passes are bound by the SMs' float64 units.  A cluster
+// lies within one GPC, so fewer fit than the SMs would hold: on GB300 7 of 16 thread blocks, 15 of 8, 36 of
+// 4, 76 of 2.  One instance more takes a second wave: 16^3 and below, V(2,2), 16 coarsest sweeps in float64
+// 125 us on clusters of 16 (8 instances 247), 154 of 8 (16 instances 298), 207 of 4 (37: 399), 329 of 2
+// (77: 641), 537 on one block each; V(1,1), 4 coarsest sweeps in float32 39 of 8 (16: 72), 50 of 4 (37: 96), 70 of 2
+// (77: 119), 69 on one.
+template <typename T>
+static int tail_cluster(int ninst) {
+    if constexpr (sizeof(T) == 8) {
+        if (ninst <= tail_resident<T, 16>()) return 16;
+    }
+    if (ninst <= tail_resident<T, 8>()) return 8;
+    if (ninst <= tail_resident<T, 4>()) return 4;
+    return ninst <= tail_resident<T, 2>() ? 2 : 1;
 }
 
 template <typename T>

@@ -370,8 +370,8 @@ def test_coarse_solver_clusters_give_same_bits_and_match_oracle(ohm, orc, base, 
 
 @pytest.mark.parametrize("edge", [40, 56])
 def test_float64_coarse_solver_on_every_cluster_size(ohm, orc, edge):
-    """The float64 coarsest-grid solver runs an instance on 16, 8, 4, 2 or 1 thread blocks (up to 8, 19, 38,
-    76 instances, more).  40^3 and 56^3 end on 5^3 and 7^3, which are still divided over the thread
+    """The float64 coarsest-grid solver runs an instance on 16, 8, 4, 2 or 1 thread blocks, by the number of
+    instances (2, 12, 20, 40, 80 of them here).  40^3 and 56^3 end on 5^3 and 7^3, which are still divided over the thread
     blocks: planes per block 1, 2 or 4, the last block partly filled, some blocks without planes."""
     h = W.uniform(edge, edge, edge, 1.0 / edge)
     bs, etas = instances(h, 2, 400)
