@@ -973,8 +973,16 @@ static cudaError_t launch_smooth_slab(const GridDev &g, const double *e_in, doub
     return cudaGetLastError();
 }
 
-// Slab height by the number of blocks: whole blocks do the least work, but a grid should give
-// every SM several thread blocks of equal share
+// Slab height by the number of blocks, one rule for the colour passes, the composite and the restricted
+// residual: whole blocks do the least work, but a grid should give every SM several thread blocks of equal
+// share.  us a launch for slabs of 2 / 4 / 8 planes (ncu, warm L2):
+//   blocks             8                   64                  216                512                2744              4096
+//   colour pass    9.1/ 8.8/10.1      9.3/ 9.0/10.9      14.0/13.7/15.9     28.5/25.0/27.1     113/101/102       159/145/144
+//   from zero      6.5/ 6.2/ 7.1      6.9/ 6.1/ 7.5      11.3/10.2/12.1     21.2/19.6/21.0      87/ 82/ 79       125/115/109
+//   residual       9.2/10.8/14.2     11.4/11.2/15.0      21.3/20.2/23.8     46.9/39.5/42.9     198/173/176       292/252/252
+//   restricted    10.2/ 8.5/ 9.2     10.5/ 8.8/10.1      15.2/12.7/14.4     32.9/22.6/23.6     130/ 92/ 88       185/131/123
+// Two planes serve the residual of few blocks; the passes are within 5% of their best there and on the
+// other ranges, the restricted residual, which would take four planes for few blocks too, within 20%.
 constexpr int SLAB2_BLOCKS = 256, SLAB4_BLOCKS = 2048;
 template <bool ZERO>
 static cudaError_t launch_smooth_d(const GridDev &g, const double *e_in, double *e_out, const double *r, const double *eta,
@@ -3446,15 +3454,19 @@ struct LexDims {
 
 constexpr int TAIL_LUT = 64;                  // blocks of the blocked grids of a tail, all together
 constexpr size_t TAIL_SMEM_MAX = 220 * 1024;
-// grids of more cells are divided over the cluster: a pass over fewer takes one block less than the
-// barriers of the division
+// Grids of more cells are divided over the cluster: a pass over fewer takes one block less than the barriers
+// of the division.  us of the whole solver with the line at 8 / 64 / 512 / 4096 cells, one instance.  float64, V(2,2), 16
+// coarsest sweeps: from 8^3 91 / 70 / 98 / 98, from 12^3 228 / 105 / 111 / 261, from 16^3 146 / 125 / 158 / 522, from
+// 10^3 (on 5^3, 125 cells) 185 / 185 / 154 / 230.  float32, V(1,1), 4 coarsest sweeps: from 8^3 37 / 31 / 24 / 24, from 12^3 48 / 41 /
+// 36 / 40, from 16^3 49 / 43 / 39 / 57, from 20^3 68 / 68 / 60 / 60.
 template <typename T>
 constexpr int tail_divide() {
     return sizeof(T) == 8 ? 64 : 512;
 }
 // Threads: 512, and 1024 for an instance on one thread block in float32 whose first grid is large enough
 // for 32 warps.  Two blocks of 512 share an SM there, so that a batch of up to 304 small instances
-// (e.g. 200 boxes of 16^3) is one wave.
+// (e.g. 200 boxes of 16^3) is one wave.  us with 512 / 1024 threads, V(1,1), 4 coarsest sweeps: 8^3 and below 24 / 26 for 100
+// instances, 28 / 49 for 200; from 12^3 53 / 51 and 59 / 88; from 16^3 74 / 69 and 135 / 124; from 20^3 123 / 106 for 100.
 constexpr int TAIL_WIDE_CELLS = 1024;
 // coarsest grids of at most this many cells per colour keep their coefficients in registers (six
 // threads per cell: components x the two axes of each)

@@ -15,7 +15,7 @@ that grid) and to the oracle's FP64 restatement of the step, and compares elemen
   `k_prolong_add<float>`), Sec. 2.2;
 * the float32 operator L X on a uniform hierarchy (`k_pair_op`) and on a 3-level AMR hierarchy
   (`k_composite<float,float>`, with coarse-fine ghosts and refluxing);
-* the coarsest-grid solve (`k_bottom_sm`, with the grid-wide steps before it where a grid is
+* the coarsest-grid solve (`k_tail<float>`, with the grid-wide steps before it where a grid is
   large) against the same V-cycle composed from the oracle's grid passes.
 
 Tolerance.  Inputs are O(1) normal fields and eta = 10^U(-0.5, 0.5) per cell, dt = 5 h^2 (so
@@ -247,8 +247,8 @@ def oracle_coarse_vcycle(o, m0, r, eta0, dt, nu1, nu2, nc, omega):
 
 
 # 32^3: power-of-two grids 16^3 .. 2^3 in the shared-memory solver; 48 x 24 x 24: 24 x 12 x 12,
-# 12 x 6 x 6 and 6 x 3 x 3 (other extents); 56^3: 28^3 stepped grid-wide (more than 16384 cells),
-# then 14^3 and 7^3 in shared memory
+# 12 x 6 x 6 and 6 x 3 x 3 (other extents); 56^3: 28^3 stepped grid-wide (it does not fit into shared
+# memory), then 14^3 and 7^3 in shared memory
 COARSE_BASES = [(32, 32, 32), (48, 24, 24), (56, 56, 56)]
 
 
