@@ -26,8 +26,8 @@ __device__ __forceinline__ int tix(int i, int j, int k) { return (k * TS + j) * 
 // Programmatic dependent launch.  The kernels of a step follow one another on one stream and many of
 // them are short (a 64^3 step: 150 launches of 2-10 us), so each is launched while the one before it
 // drains: its thread blocks come up, read the block tables (which never change) and wait for the
-// grid before them to complete: 64^3 mixed step 1.67 -> 1.53 ms, three-level mixed step 2.50 -> 2.33,
-// 128^3 float-float step 3.56 -> 3.43.  Every kernel launched through launch_pdl calls pdl_trigger() and,
+// grid before them to complete: 64^3 mixed step 1.67 -> 1.53 ms, three-level mixed step (64^3 base, 3 V-cycles)
+// 2.50 -> 2.33, 128^3 float-float step 3.56 -> 3.43.  Every kernel launched through launch_pdl calls pdl_trigger() and,
 // before it touches anything that another kernel writes and before any return, pdl_wait().  A load
 // through a const __restrict__ parameter could be moved above the wait, so pdl_wait returns an opaque 0
 // that goes into the block (or element) index from which the addresses of such loads are formed; the
@@ -673,7 +673,7 @@ cudaError_t launch_composite(const GridDev &g, const float *X, const float *Y, c
 // state (Jacobi within a colour).  256 threads, one per colour cell.
 // ZERO: both passes of the sweep from e = 0 in one launch (as k_smooth_d's; colour = 1): the tile holds
 // the pointwise red update inv r at red cells and 0 elsewhere, e_in is not read (three-level mixed step
-// 2.33 -> 2.22 ms, with the right-hand sides in flight during the staging 2.14).
+// of 3 V-cycles 2.33 -> 2.22 ms, with the right-hand sides in flight during the staging 2.14).
 // EARLY = false (grids of more than PDL_GRID blocks): no early launch, and a general pass loads its right-hand
 // sides after the stencil.  Held through the staging they cost more registers than the latency is worth
 // once every SM has several waves of blocks: 128^3 34.8 us a pass, 38.8 loaded ahead, 41.9 launched early
